@@ -48,7 +48,7 @@ __device__ __forceinline__ void bin_finish_body(const float *__restrict__ partia
     }
 }
 
-// steps: the step counter to advance by K here (no later kernel of the push reads it), or null.
+// steps: the step counter, advanced by K here (the push's later kernels subtract K), or null.
 __global__ void __launch_bounds__(BF_THREADS) bin_finish_kernel(const float *__restrict__ partials,
                                                                 int n_slots, const int *slot_begin,
                                                                 int B, int K, float *Jb,
@@ -62,30 +62,74 @@ __global__ void __launch_bounds__(BF_THREADS) bin_finish_kernel(const float *__r
 __global__ void __launch_bounds__(BF_THREADS) bin_finish_group_kernel(const __grid_constant__ FinishGroupArgs g) {
     int j = 0;
     while (j + 1 < g.n && (int)blockIdx.x >= g.cta_begin[j + 1]) ++j;
-    if (g.advance && (int)blockIdx.x == g.cta_begin[j] && threadIdx.x == 0) *g.steps[j] += g.K[j];
+    if ((int)blockIdx.x == g.cta_begin[j] && threadIdx.x == 0) *g.steps[j] += g.K[j];
     bin_finish_body(g.partials[j], g.n_slots[j], g.slot_begin[j], g.B[j], g.K[j], g.Jb[j],
                     g.hsum[j], g.Jtot[j], g.Jsum[j], (int)blockIdx.x - g.cta_begin[j]);
 }
 
-__global__ void advance_steps_group_kernel(const __grid_constant__ FinishGroupArgs g) {
-    const int j = threadIdx.x;
-    if (j < g.n) *g.steps[j] += g.K[j];
-}
-
 // ------------------------------------------------------------------ K4
-// Register-tiled like a GEMM micro-kernel.  A CTA owns 32 consecutive lags (one per lane) and
-// LC_ROWS rows (b, mu) of LC_ROWS / 3 bins; its W <= LC_WARPS warps take consecutive ranges of
-// ceil(K / W) steps of the block.  Per step a thread loads its lag's total current J(t - l)
-// (one 16-byte shared-memory load from the CTA's window of J samples) and the step's LC_ROWS
-// binned currents (broadcast 16-byte loads) and does 3 LC_ROWS FMAs into FP32 partial sums over
-// the warp's steps.  The warps' partials are then added in step order in an unevaluated float
-// pair (TwoSum, ~48 bits; GB300's FP64 pipe is narrow) and each lag sum gets one FP64 add.
-// At most 16 warps a CTA, so that two CTAs share an SM: one CTA's staging and final sums then
-// overlap the other's FMAs, and a grid a little larger than the SM count (N = 512: 175 CTAs)
-// still runs in one wave.
+// Register-tiled like a GEMM micro-kernel.  A tile is 32 consecutive lags (one per lane) times
+// LC_ROWS rows (b, mu) of LC_ROWS / 3 bins.  Its warps take consecutive ranges of ks steps of
+// the block: per step a thread loads its lag's total current J(t - l) (one 16-byte shared-memory
+// load from the CTA's window of J samples) and the step's LC_ROWS binned currents (broadcast
+// 16-byte loads) and does 3 LC_ROWS FMAs into FP32 partial sums over the warp's steps.  The
+// warps' partials are then added in step order in an unevaluated float pair (TwoSum, ~48 bits;
+// GB300's FP64 pipe is narrow) and each lag sum gets one FP64 add.
+//
+// What bounds it: the FMAs when a grid fills the SMs, otherwise the chain staging -> steps ->
+// final sums of one CTA.  So (lag_corr_plan):
+//   - a tile's steps are spread over as many warps as give about three warps a scheduler over
+//     the GPU, down to LC_MIN_STEPS steps a warp: with one warp per 32 steps a 32-step block ran
+//     one warp a tile, 23.3 us (ncu), nearly all of it 36 read-modify-writes of the sums in turn;
+//   - the tile's warps go to a cluster of CTAs of four warps where the grid can fill the SMs
+//     (smaller pieces balance better: N = 512, K = 1000 had 175 CTAs of 16 warps, two on 23 of
+//     the 152 SMs), each CTA staging its own steps alone; the ranks read each other's partials
+//     through distributed shared memory and each finishes its share of the tile's sums;
+//   - a CTA alone has at least LC_FINAL_WARPS warps (those without steps take part in the
+//     staging and the final sums), and every warp fetches the sums it will update into L2 first.
+// Measured (ncu, cold caches, us, before -> now): K = 32, 8 bins, 8 lags 23.3 -> 7.7; K = 77, 37
+// bins, 123 lags 15.5 -> 8.4; K = 1000, 100 bins, 200 lags 24.6 -> 18.6; K = 512, 64 bins, 1000
+// lags 30.5 -> 27.9; K = 256, 64 bins, 500 lags 13.0 -> 13.4.  The cluster form starts at
+// LC_FILL_TILES = half the SMs: below it a tile's CTA has an SM to itself either way, and one
+// CTA's barriers are cheaper than a cluster's.
 constexpr int LC_ROWS = 12;   // 4 bins x 3 components a thread
 constexpr int LC_OUT = 3 * LC_ROWS;
-constexpr int LC_WARPS = 16;
+constexpr int LC_WARPS = 16;      // warps of a tile, and of a CTA that holds a tile alone
+constexpr int LC_CTA_WARPS = 4;   // warps of a CTA of a cluster
+constexpr int LC_FINAL_WARPS = 12;   // fewest warps of a CTA that holds a tile alone
+constexpr int LC_BATCH = 5;       // sums a warp updates at a time (all of them with 8 or more warps)
+constexpr int LC_MIN_STEPS = 4;   // fewest steps a warp is worth starting for
+constexpr int LC_FILL_WARPS = 152 * 12;   // three warps a scheduler on every SM
+constexpr int LC_FILL_TILES = 76;         // tiles from which clusters of small CTAs balance better
+
+// Warps with steps of one tile, steps a warp, the CTAs (cluster ranks) they run in, the warps
+// with steps of a CTA and all its warps.
+struct LagCorrPlan {
+    int warps, ks, ranks, step_warps, cta_warps;
+};
+
+LagCorrPlan lag_corr_plan(int K, int tiles) {
+    LagCorrPlan p;
+    // at least ceil(K / 32) warps up to LC_WARPS, so that an FP32 partial sum never covers more
+    // steps than ceil(K / LC_WARPS) or 32, whichever is more
+    const int lo = std::max(1, std::min(LC_WARPS, (K + 31) / 32));
+    const int hi = std::max(lo, std::min(LC_WARPS, K / LC_MIN_STEPS));
+    const int want = (LC_FILL_WARPS + tiles - 1) / std::max(tiles, 1);
+    p.warps = std::max(lo, std::min(hi, want));
+    p.ks = (K + p.warps - 1) / p.warps;
+    p.warps = (K + p.ks - 1) / p.ks;
+    p.ranks = tiles >= LC_FILL_TILES ? (p.warps + LC_CTA_WARPS - 1) / LC_CTA_WARPS : 1;
+    p.step_warps = p.ranks > 1 ? LC_CTA_WARPS : p.warps;
+    p.cta_warps = p.ranks > 1 ? LC_CTA_WARPS : std::max(p.warps, LC_FINAL_WARPS);
+    return p;
+}
+
+size_t lag_corr_smem(const LagCorrPlan &p) {
+    const size_t steps = (size_t)p.step_warps * p.ks;
+    const size_t staging = steps * LC_ROWS * sizeof(float) + (steps + 31) * sizeof(float4);
+    const size_t partials = (size_t)p.step_warps * LC_OUT * 32 * sizeof(float);
+    return std::max(staging, partials);
+}
 
 // (s, c) += x exactly as an unevaluated float pair (_rn keeps it from being contracted)
 __device__ __forceinline__ void lc_pair_add(float &s, float &c, float x) {
@@ -95,42 +139,58 @@ __device__ __forceinline__ void lc_pair_add(float &s, float &c, float x) {
     s = t;
     c = __fadd_rn(c, e);
 }
+
+// t0_dev: the device step counter, which the push's bin finish has already advanced by K.
 __global__ void __launch_bounds__(32 * LC_WARPS, 2) lag_corr_kernel(const float *__restrict__ Jb,
                                                                     const double *__restrict__ Jring,
                                                                     int R, double *Csum, int K,
-                                                                    int B, int L, long long t0_host,
-                                                                    const long long *t0_dev,
-                                                                    long long *steps,
-                                                                    unsigned *ticket) {
-    const long long t0 = t0_dev ? *t0_dev : t0_host;
-    // staging: rows [K][LC_ROWS], then the J window [K + 31] as float4 (x, y, z, 0); after the
-    // step loop the same space holds the warps' partials [warp][LC_OUT][32]
+                                                                    int B, int L, int ks,
+                                                                    int step_warps,
+                                                                    const long long *t0_dev) {
+    // staging: rows [steps][LC_ROWS] of this CTA's steps, then their J window [steps + 31] as
+    // float4 (x, y, z, 0); after the step loop the same space holds the warps' partials
+    // [warp][LC_OUT][32]
     extern __shared__ float4 lc_smem4[];
     float *sA = reinterpret_cast<float *>(lc_smem4);
-    float4 *sW = lc_smem4 + (K * LC_ROWS) / 4;
     float *sP = reinterpret_cast<float *>(lc_smem4);
+    const int nrank = (int)gridDim.z, rank = (int)blockIdx.z;   // a cluster spans grid z
     const int l0 = blockIdx.x * 32;
     const int b0 = blockIdx.y * (LC_ROWS / 3);
-    const int nthreads = blockDim.x;
+    const int nthreads = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cta_warps = nthreads >> 5;
+    const int steps_cta = step_warps * ks;
+    const int kc0 = min(K, rank * steps_cta), kc = min(K - kc0, steps_cta);   // this CTA's steps
+    float4 *sW = lc_smem4 + steps_cta * (LC_ROWS / 4);
+
+    // the tile's sums are shared out by warps over all ranks: output o (of all 32 lags) goes to
+    // warp o mod ngw of the tile; its 256 bytes come into L2 while the staging and the steps run
+    const int l = l0 + lane;
+    const int gw = rank + nrank * warp, ngw = nrank * cta_warps;
+    auto sums = [&](int o) { return Csum + ((size_t)(b0 + o / 9) * 9 + ((o / 3) % 3) * 3 + o % 3) * L + l; };
+    if ((lane & 15) == 0 && l < L)
+        for (int o = gw; o < LC_OUT && b0 + o / 9 < B; o += ngw)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(sums(o)));
+    const float *Jk = Jb + (size_t)kc0 * B * 3;
     if (B % 4 == 0 && (reinterpret_cast<uintptr_t>(Jb) & 15) == 0) {
         // every bin group is whole and its 12 floats of a step start on a 16-byte boundary:
         // three asynchronous 16-byte copies a step, all in flight at once
-        for (int q = threadIdx.x; q < 3 * K; q += nthreads) {
+        for (int q = threadIdx.x; q < 3 * kc; q += nthreads) {
             const int k = q / 3, j = q - 3 * k;
-            cp_async16(sA + k * LC_ROWS + 4 * j, Jb + ((size_t)k * B + b0) * 3 + 4 * j);
+            cp_async16(sA + k * LC_ROWS + 4 * j, Jk + ((size_t)k * B + b0) * 3 + 4 * j);
         }
     } else {
-        for (int q = threadIdx.x; q < K * LC_ROWS; q += nthreads) {
-            const int k = q / LC_ROWS, r = q % LC_ROWS, b = b0 + r / 3;
-            sA[q] = b < B ? Jb[((size_t)k * B + b) * 3 + r % 3] : 0.f;
+        for (int q = threadIdx.x; q < kc * LC_ROWS; q += nthreads) {
+            const int k = q / LC_ROWS, r = q - k * LC_ROWS;
+            if (b0 + r / 3 < B) cp_async4(sA + q, Jk + ((size_t)k * B + b0) * 3 + r);
+            else sA[q] = 0.f;
         }
     }
-    // window entry w holds J(tw0 + w), tw0 = t0 - l0 - 31: lane l at step k reads w = k - l + 31.
-    // Ring slot of entry w: (tw0 mod R) + w brought into [0, R) with 32-bit arithmetic (one
-    // 64-bit remainder a thread instead of one an entry).
-    const long long tw0 = t0 - l0 - 31;
+    // window entry w holds J(tw0 + w), tw0 = t0 + kc0 - l0 - 31: lane l at the CTA's step k reads
+    // w = k - l + 31.  Ring slot of entry w: (tw0 mod R) + w brought into [0, R) with 32-bit
+    // arithmetic (one 64-bit remainder a thread instead of one an entry).
+    const long long tw0 = *t0_dev - K + kc0 - l0 - 31;
     const int m0 = (int)(tw0 % R);   // in (-R, R)
-    for (int w = threadIdx.x; w < K + 31; w += nthreads) {
+    for (int w = threadIdx.x; w < kc + 31; w += nthreads) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (tw0 + w >= 0) {
             int slot = m0 + w;
@@ -143,9 +203,7 @@ __global__ void __launch_bounds__(32 * LC_WARPS, 2) lag_corr_kernel(const float 
     }
     cp_async_wait_all();
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = nthreads >> 5;
-    const int ks = (K + nwarps - 1) / nwarps;
-    const int k_begin = min(K, ks * warp), k_end = min(K, k_begin + ks);
+    const int k_begin = min(kc, ks * warp), k_end = min(kc, k_begin + ks);
     float acc[LC_OUT];
 #pragma unroll
     for (int o = 0; o < LC_OUT; ++o) acc[o] = 0.f;
@@ -172,37 +230,38 @@ __global__ void __launch_bounds__(32 * LC_WARPS, 2) lag_corr_kernel(const float 
         }
     }
     __syncthreads();   // staging no longer read: its space takes the partials
+    if (warp < step_warps) {
 #pragma unroll
-    for (int o = 0; o < LC_OUT; ++o) sP[(warp * LC_OUT + o) * 32 + lane] = acc[o];
-    __syncthreads();
-    for (int q = threadIdx.x; q < LC_OUT * 32; q += nthreads) {
-        const int o = q >> 5, ln = q & 31;
-        const int l = l0 + ln, r = o / 3, b = b0 + r / 3;
-        if (l >= L || b >= B) continue;
-        double *dst = Csum + ((size_t)b * 9 + (r % 3) * 3 + o % 3) * L + l;
-        const double old = *dst;   // in flight while the partials are added
-        float s = 0.f, c = 0.f;
-        for (int w = 0; w < nwarps; ++w) lc_pair_add(s, c, sP[(w * LC_OUT + o) * 32 + ln]);
-        *dst = old + ((double)s + (double)c);
+        for (int o = 0; o < LC_OUT; ++o) sP[(warp * LC_OUT + o) * 32 + lane] = acc[o];
     }
-    if (steps) {   // the last CTA to finish advances the step counter: every CTA has read it
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            if (atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1) {
-                *steps += K;
-                *ticket = 0;
+    cluster_sync_all();   // every rank's partials are complete (one CTA: a CTA barrier)
+    for (int o0 = gw; o0 < LC_OUT && b0 + o0 / 9 < B; o0 += LC_BATCH * ngw) {   // warp-uniform
+        double old[LC_BATCH];
+#pragma unroll
+        for (int u = 0; u < LC_BATCH; ++u) {
+            const int o = o0 + u * ngw;
+            old[u] = (o < LC_OUT && b0 + o / 9 < B && l < L) ? *sums(o) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < LC_BATCH; ++u) {
+            const int o = o0 + u * ngw;
+            if (o >= LC_OUT || b0 + o / 9 >= B) break;   // warp-uniform
+            float s = 0.f, c = 0.f;
+            const float *mine = sP + o * 32 + lane;
+            if (nrank == 1) {
+                for (int w = 0; w < step_warps; ++w) lc_pair_add(s, c, mine[w * LC_OUT * 32]);
+            } else {
+                for (int q = 0; q < nrank; ++q) {   // step order: ranks, then warps
+                    const uint32_t peer = mapa_shared(smem_u32(mine), (uint32_t)q);
+#pragma unroll
+                    for (int w = 0; w < LC_CTA_WARPS; ++w)
+                        lc_pair_add(s, c, ld_shared_cluster_f32(peer + (uint32_t)(w * LC_OUT * 32 * sizeof(float))));
+                }
             }
+            if (l < L) *sums(o) = old[u] + ((double)s + (double)c);
         }
     }
-}
-
-int lag_corr_warps(int K) { return std::max(1, std::min(LC_WARPS, (K + 31) / 32)); }
-
-size_t lag_corr_smem(int K) {
-    const size_t staging = (size_t)K * LC_ROWS * sizeof(float) + (size_t)(K + 31) * sizeof(float4);
-    const size_t partials = (size_t)lag_corr_warps(K) * LC_OUT * 32 * sizeof(float);
-    return staging > partials ? staging : partials;
+    cluster_sync_all();   // peers have read this CTA's partials: its shared memory may go
 }
 
 // ------------------------------------------------------------------ K5
@@ -365,8 +424,6 @@ __global__ void hnema_finalize_group_kernel(const HnemaGroupArgs a, double *mean
     }
 }
 
-__global__ void advance_steps_kernel(long long *steps, int K) { *steps += K; }
-
 __global__ void lag_counts_kernel(long long T_s, int L, long long *count) {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l < L) count[l] = T_s > l ? T_s - l : 0;
@@ -384,18 +441,18 @@ void launch_bin_finish(const float *partials, int n_slots, const int *slot_begin
 }
 
 namespace {
-size_t lc_sm_set = 48 * 1024;   // the largest dynamic shared memory opted into so far
 // the per-CTA weight table: up to two CTAs an SM and a table within the default 48 KB
 constexpr int GK_TABLE_CTAS = 304;
 constexpr int GK_TABLE_LAGS = 6144;
+
+int lag_corr_tiles(int B, int L) { return ((L + 31) / 32) * ((B + LC_ROWS / 3 - 1) / (LC_ROWS / 3)); }
 }
 
-cudaError_t lag_corr_prepare(int k_max) {
-    const size_t sm = lag_corr_smem(k_max);
-    if (sm <= lc_sm_set) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(lag_corr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)sm);
-    if (e == cudaSuccess) lc_sm_set = sm;
+cudaError_t lag_corr_prepare() {
+    // a tile alone in its CTA stages at most 1024 steps or 16 warps' partials: below 80 KB
+    LagCorrPlan p{LC_WARPS, 64, 1, LC_WARPS, LC_WARPS};
+    static const cudaError_t e = cudaFuncSetAttribute(
+        lag_corr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lag_corr_smem(p));
     return e;
 }
 
@@ -406,21 +463,27 @@ void launch_bin_finish_group(FinishGroupArgs g, cudaStream_t s) {
     if (g.cta_begin[g.n] > 0) bin_finish_group_kernel<<<g.cta_begin[g.n], BF_THREADS, 0, s>>>(g);
 }
 
-void launch_advance_steps_group(const FinishGroupArgs &g, cudaStream_t s) {
-    if (g.n >= 1) advance_steps_group_kernel<<<1, 32, 0, s>>>(g);
-}
-
-void launch_lag_corr(const float *Jb, const double *Jring, int R, double *Csum, int K, int B,
-                     int L, long long t0, const long long *t0_dev, long long *steps,
-                     unsigned *ticket, cudaStream_t s) {
-    if (L <= 0 || K <= 0 || B <= 0) return;
-    dim3 grid((L + 31) / 32, (B + LC_ROWS / 3 - 1) / (LC_ROWS / 3));
-    const int threads = 32 * lag_corr_warps(K);
-    const size_t sm = lag_corr_smem(K);
-    if (sm > lc_sm_set && lag_corr_prepare(K) != cudaSuccess)
-        return;   // the launch is skipped; the caller's cudaGetLastError reports the failure
-    lag_corr_kernel<<<grid, threads, sm, s>>>(Jb, Jring, R, Csum, K, B, L, t0, t0_dev, steps,
-                                              ticket);
+cudaError_t launch_lag_corr(const float *Jb, const double *Jring, int R, double *Csum, int K, int B,
+                            int L, const long long *t0_dev, cudaStream_t s) {
+    if (L <= 0 || K <= 0 || B <= 0) return cudaSuccess;
+    const cudaError_t ready = lag_corr_prepare();
+    if (ready != cudaSuccess) return ready;
+    const LagCorrPlan p = lag_corr_plan(K, lag_corr_tiles(B, L));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((L + 31) / 32), (unsigned)((B + LC_ROWS / 3 - 1) / (LC_ROWS / 3)),
+                       (unsigned)p.ranks);
+    cfg.blockDim = dim3((unsigned)(32 * p.cta_warps), 1, 1);
+    cfg.dynamicSmemBytes = lag_corr_smem(p);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = (unsigned)p.ranks;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, lag_corr_kernel, Jb, Jring, R, Csum, K, B, L, p.ks,
+                              p.step_warps, t0_dev);
 }
 
 int launch_gk_kappa(const double *Csum, int B, int L, long long T_s, double coef_dt,
@@ -466,10 +529,6 @@ void launch_hnema_finalize(const double *hsum, int B, long long T_s, double coef
 void launch_hnema_finalize_group(const HnemaGroupArgs &a, double *mean, double *kappa,
                                  cudaStream_t s) {
     hnema_finalize_group_kernel<<<dim3(4, a.n), 128, 0, s>>>(a, mean, kappa);
-}
-
-void launch_advance_steps(long long *steps, int K, cudaStream_t s) {
-    advance_steps_kernel<<<1, 1, 0, s>>>(steps, K);
 }
 
 void launch_lag_counts(long long T_s, int L, long long *count, cudaStream_t s) {

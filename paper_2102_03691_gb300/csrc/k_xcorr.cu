@@ -52,8 +52,8 @@ __device__ __forceinline__ void xc_pair_add(float &s, float &c, float x) {
 
 // ring[(t0 + k) mod R][j] = Jb[k][j]: the block's binned currents join the history ring
 __global__ void jb_ring_store_kernel(const float *__restrict__ Jb, int K, int n, float *ring,
-                                     int R, long long t0_host, const long long *t0_dev) {
-    const long long t0 = t0_dev ? *t0_dev : t0_host;
+                                     int R, const long long *t0_dev) {
+    const long long t0 = *t0_dev - K;   // the bin finish has advanced the counter
     const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (q >= (long long)K * n) return;
     const long long k = q / n, j = q - k * n;
@@ -65,12 +65,12 @@ __global__ void jb_ring_store_kernel(const float *__restrict__ Jb, int K, int n,
 constexpr int XW_THREADS = 256;
 __global__ void __launch_bounds__(XW_THREADS) xc_window_kernel(const float *__restrict__ ring, int R,
                                                                int n, int K, int L, int U_pad,
-                                                               int rows_pad, long long t0_host,
+                                                               int rows_pad,
                                                                const long long *t0_dev,
                                                                uint16_t *Whi, uint16_t *Wlo,
                                                                float *inv_scale) {
     const int j = blockIdx.x;
-    const long long t0 = t0_dev ? *t0_dev : t0_host;
+    const long long t0 = *t0_dev - K;
     const long long tw0 = t0 - (L - 1);
     const int Uw = K + L - 1;
     const int base = (int)(((tw0 % R) + R) % R);   // ring row of u = 0
@@ -371,20 +371,18 @@ cudaError_t xcorr_prepare() {
     return e;
 }
 
-void launch_jb_ring_store(const float *Jb, int K, int nb, float *ring, int R, long long t0,
+void launch_jb_ring_store(const float *Jb, int K, int nb, float *ring, int R,
                           const long long *t0_dev, cudaStream_t s) {
     const long long total = (long long)K * nb * 3;
     if (total <= 0) return;
-    jb_ring_store_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(Jb, K, 3 * nb, ring, R, t0, t0_dev);
+    jb_ring_store_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(Jb, K, 3 * nb, ring, R, t0_dev);
 }
 
 cudaError_t launch_bin_xcorr(const XcPlan &pl, XcTcParams p, const float *ring, int R, int K,
-                             long long t0, const long long *t0_dev, void *Whi, void *Wlo,
-                             cudaStream_t s) {
+                             const long long *t0_dev, void *Whi, void *Wlo, cudaStream_t s) {
     if (p.L <= 0 || K <= 0 || pl.n <= 0) return cudaSuccess;
     if (K + p.L - 1 > R || K + p.L - 1 > pl.U_pad) return cudaErrorInvalidValue;
-    xc_window_kernel<<<pl.n, XW_THREADS, 0, s>>>(ring, R, pl.n, K, p.L, pl.U_pad, pl.rows_pad, t0,
-                                                 t0_dev, static_cast<uint16_t *>(Whi),
+    xc_window_kernel<<<pl.n, XW_THREADS, 0, s>>>(ring, R, pl.n, K, p.L, pl.U_pad, pl.rows_pad, t0_dev, static_cast<uint16_t *>(Whi),
                                                  static_cast<uint16_t *>(Wlo),
                                                  const_cast<float *>(p.inv_scale));
     const cudaError_t attr = xcorr_prepare();

@@ -220,13 +220,13 @@ void launch_shc_tc_reduce(const ShcTcParams &p, double *Ksum, cudaStream_t s);
 // ---------------------------------------------------------------- K3 .. K5
 // Jb[k][b][a] = sum of partial slots of bin b; HNEMA sums += sum_k Jb (FP64);
 // Jsum[a] += sum_k Jtot[k][a].
-// steps (or null): the device step counter, advanced by K by the same launch when no later
-// kernel of the push reads it.
+// steps (or null): the device step counter, advanced by K by the same launch (the correlation
+// kernels that follow in the push subtract K).
 void launch_bin_finish(const float *partials, int n_slots, const int *slot_begin, int B, int K,
                        float *Jb, double *hsum, const double *Jtot, double *Jsum, long long *steps,
                        cudaStream_t s);
-// The bin finish (as launch_bin_finish) and the step counters (*steps += K) of up to
-// TC_MAX_GROUP systems, one launch each; cta_begin is filled by the launcher.
+// The bin finish (as launch_bin_finish, step counters included) of up to TC_MAX_GROUP systems
+// in one launch; cta_begin is filled by the launcher.
 struct FinishGroupArgs {
     const float *partials[TC_MAX_GROUP];
     int n_slots[TC_MAX_GROUP];
@@ -239,21 +239,14 @@ struct FinishGroupArgs {
     long long *steps[TC_MAX_GROUP];
     int cta_begin[TC_MAX_GROUP + 1];
     int n;
-    int advance;   // 1: the bin finish also advances the step counters (no correlation kernels)
 };
 void launch_bin_finish_group(FinishGroupArgs g, cudaStream_t s);
-void launch_advance_steps_group(const FinishGroupArgs &g, cudaStream_t s);
 // Csum[b][mu][nu][l] += sum_k Jb[k][b][mu] J(t0+k-l)^nu over t0+k-l >= 0.
-// lag_corr_prepare(k_max): opt into the shared memory of blocks up to k_max steps (call outside
-// any stream capture).
-cudaError_t lag_corr_prepare(int k_max);
-// steps, ticket: when steps is not null, the last CTA to finish adds K to *steps (the push's
-// last reader of the counter) and resets *ticket, a device counter that starts at 0.
-void launch_lag_corr(const float *Jb, const double *Jring, int R, double *Csum, int K, int B,
-                     int L, long long t0, const long long *t0_dev, long long *steps,
-                     unsigned *ticket, cudaStream_t s);
-// *steps += K (one thread; last kernel of a push)
-void launch_advance_steps(long long *steps, int K, cudaStream_t s);
+// t0_dev: the device step counter, already advanced by K (t0 = *t0_dev - K).
+cudaError_t launch_lag_corr(const float *Jb, const double *Jring, int R, double *Csum, int K, int B,
+                            int L, const long long *t0_dev, cudaStream_t s);
+// Opt into the kernel's shared memory (call outside any stream capture).
+cudaError_t lag_corr_prepare();
 // kappa_tau[r][l] (r = b*9+mu*3+nu) and window averages kappa_w[r], FP64; kappa_tau null:
 // the window averages alone, as one weighted sum of C(l) a row.
 // inv_scratch: [L] doubles of device scratch (the reciprocal lag counts of this read).
@@ -276,7 +269,8 @@ struct HnemaGroupArgs {
 void launch_hnema_finalize_group(const HnemaGroupArgs &a, double *mean, double *kappa, cudaStream_t s);
 // ---------------------------------------------------------------- bin-bin cross-correlations
 // ring[(t0 + k) mod R][3b+mu] = Jb[k][b][mu] (nb output rows of 3 components)
-void launch_jb_ring_store(const float *Jb, int K, int nb, float *ring, int R, long long t0,
+// t0_dev: the device step counter, already advanced by K (as for launch_bin_xcorr)
+void launch_jb_ring_store(const float *Jb, int K, int nb, float *ring, int R,
                           const long long *t0_dev, cudaStream_t s);
 // Tensor-core cross-correlation (k_xcorr.cu): n = 3 nb rows; column tiles of nj <= XC_NJ_MAX
 // rows j; row tiles of 128 rows i; the window copies hold 8 x rows_pad rows of U_pad steps.
@@ -303,8 +297,7 @@ int xcorr_make_maps(const XcPlan &pl, const void *Whi, const void *Wlo, XcTcPara
 // already in the ring: the window kernel (scales + eight shifted FP16 hi/lo copies of
 // [t0 - L + 1, t0 + K)) then the tensor-core kernel.  Needs K + L - 1 <= min(R, U_pad).
 cudaError_t launch_bin_xcorr(const XcPlan &pl, XcTcParams p, const float *ring, int R, int K,
-                             long long t0, const long long *t0_dev, void *Whi, void *Wlo,
-                             cudaStream_t s);
+                             const long long *t0_dev, void *Whi, void *Wlo, cudaStream_t s);
 // out[b][b'][mu][nu][l] = X[l][3b'+nu][3b+mu] (float pair -> FP64)
 void launch_xcorr_transpose(const float2 *X, int nb, int L, double *out, cudaStream_t s);
 // count[l] = max(T_s - l, 0)

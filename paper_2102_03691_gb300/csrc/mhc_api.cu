@@ -266,8 +266,7 @@ mhc_status reset_accumulators(mhc_handle *h) {
     if (h->prm.flags & MHC_FLAG_GKMA) {
         if ((s = dev_alloc(h, "Csum", sizeof(double) * B * 9 * L)) != MHC_OK) return s;
         if ((s = dev_alloc(h, "Jring", sizeof(double) * h->R_ring * 3)) != MHC_OK) return s;
-        if ((s = dev_alloc(h, "lc_ticket", sizeof(unsigned))) != MHC_OK) return s;
-        MHC_CUDA(h, lag_corr_prepare(h->prm.k_max));
+        MHC_CUDA(h, lag_corr_prepare());
     }
     if (has_xcorr(h)) {   // lag-major [L][3R][3R] float-pair sums, the ring of past binned
                           // currents, and the tensor-core kernel's window copies
@@ -874,27 +873,20 @@ mhc_status pack_block(mhc_handle *h, const float *v, const float *W, int K) {
     return MHC_OK;
 }
 
-// The correlation kernels of a push (after its bin finish): GKMA lag correlation and the
-// cross-correlations.
-// advance: the lag correlation, when no cross-correlation kernel follows it, also advances the
-// device step counter (*advanced is set then).
-mhc_status correlate_block(mhc_handle *h, int K, bool advance = false, bool *advanced = nullptr) {
-    if (advanced) *advanced = false;
+// The correlation kernels of a push (after its bin finish, which has advanced the device step
+// counter): GKMA lag correlation and the cross-correlations.
+mhc_status correlate_block(mhc_handle *h, int K) {
+    const long long *steps = dptr<long long>(h, "steps_dev");
     if (h->prm.flags & MHC_FLAG_GKMA) {
-        const bool adv = advance && !has_xcorr(h);
-        launch_lag_corr(dptr<float>(h, "Jb"), dptr<double>(h, "Jring"), h->R_ring,
-                        dptr<double>(h, "Csum"), K, (int)n_out_bins(h), h->prm.n_lags, h->steps,
-                        dptr<long long>(h, "steps_dev"),
-                        adv ? dptr<long long>(h, "steps_dev") : nullptr,
-                        dptr<unsigned>(h, "lc_ticket"), h->stream);
-        if (advanced) *advanced = adv;
+        MHC_CUDA(h, launch_lag_corr(dptr<float>(h, "Jb"), dptr<double>(h, "Jring"), h->R_ring,
+                                    dptr<double>(h, "Csum"), K, (int)n_out_bins(h), h->prm.n_lags,
+                                    steps, h->stream));
         h->launches++;
     }
     if (has_xcorr(h)) {
         launch_jb_ring_store(dptr<float>(h, "Jb"), K, (int)n_out_bins(h), dptr<float>(h, "Jbring"),
-                             h->R_ring, h->steps, dptr<long long>(h, "steps_dev"), h->stream);
-        MHC_CUDA(h, launch_bin_xcorr(h->xc_plan, h->xcp, dptr<float>(h, "Jbring"), h->R_ring, K,
-                                     h->steps, dptr<long long>(h, "steps_dev"),
+                             h->R_ring, steps, h->stream);
+        MHC_CUDA(h, launch_bin_xcorr(h->xc_plan, h->xcp, dptr<float>(h, "Jbring"), h->R_ring, K, steps,
                                      dptr<void>(h, "Xwin_hi"), dptr<void>(h, "Xwin_lo"), h->stream));
         h->launches += 3;
     }
@@ -902,27 +894,15 @@ mhc_status correlate_block(mhc_handle *h, int K, bool advance = false, bool *adv
     return MHC_OK;
 }
 
-// Kernels that close a push: bin finish + HNEMA sums, correlations, step counter.
+// Kernels that close a push: bin finish + HNEMA sums + step counter, correlations.
 mhc_status finish_kernels(mhc_handle *h, int K) {
-    // without correlation kernels (which read the step counter) the bin finish advances it, and
-    // with the lag correlation alone that kernel does
-    const bool corr = (h->prm.flags & MHC_FLAG_GKMA) || has_xcorr(h);
     launch_bin_finish(dptr<float>(h, "partials"), (int)slot_stride(h), dptr<int>(h, "slot_begin"),
                       (int)n_out_bins(h), K, dptr<float>(h, "Jb"), dptr<double>(h, "hsum"),
                       dptr<double>(h, "Jtot"), dptr<double>(h, "Jsum"),
-                      corr ? nullptr : dptr<long long>(h, "steps_dev"), h->stream);
+                      dptr<long long>(h, "steps_dev"), h->stream);
     h->launches++;
-    if (corr) {
-        bool advanced = false;
-        mhc_status s = correlate_block(h, K, true, &advanced);
-        if (s != MHC_OK) return s;
-        if (!advanced) {
-            launch_advance_steps(dptr<long long>(h, "steps_dev"), K, h->stream);
-            h->launches++;
-        }
-    }
     MHC_CUDA(h, cudaGetLastError());
-    return MHC_OK;
+    return correlate_block(h, K);
 }
 
 void count_push(mhc_handle *h, int K) {
@@ -1845,8 +1825,8 @@ mhc_status group_pack(mhc_group *g, const std::vector<const float *> &vs,
     return MHC_OK;
 }
 
-// The kernels that close a group push: one bin-finish launch for all systems, each system's
-// correlation kernels, one launch for all step counters.
+// The kernels that close a group push: one bin-finish launch for all systems (which advances
+// their step counters), each system's correlation kernels.
 mhc_status group_finish(mhc_group *g, const std::vector<int> &Ks) {
     mhc_handle *h0 = g->hs[0];
     FinishGroupArgs fg{};
@@ -1864,21 +1844,13 @@ mhc_status group_finish(mhc_group *g, const std::vector<int> &Ks) {
         fg.Jsum[j] = dptr<double>(h, "Jsum");
         fg.steps[j] = dptr<long long>(h, "steps_dev");
     }
-    // without correlation kernels (which read the step counters) the bin finish advances them
-    bool corr = false;
-    for (mhc_handle *h : g->hs) corr = corr || (h->prm.flags & MHC_FLAG_GKMA) || has_xcorr(h);
-    fg.advance = corr ? 0 : 1;
     launch_bin_finish_group(fg, h0->stream);
     h0->launches++;
     MHC_CUDA(h0, cudaGetLastError());
-    if (!corr) return MHC_OK;
     for (int j = 0; j < fg.n; ++j) {
         const mhc_status s = correlate_block(g->hs[j], Ks[j]);
         if (s != MHC_OK) return s;
     }
-    launch_advance_steps_group(fg, h0->stream);
-    h0->launches++;
-    MHC_CUDA(h0, cudaGetLastError());
     return MHC_OK;
 }
 
@@ -2199,7 +2171,6 @@ mhc_status group_push_staged(mhc_group *g, const std::vector<const float *> &vs,
             for (size_t j = 0; j < n; ++j) l0[j] = g->hs[j]->launches;
             cudaStream_t user = h0->stream;
             // graph: grouped pack -> grouped projection -> grouped bin finish -> correlations
-            //        -> step counters
             MHC_CUDA(h0, cudaStreamBeginCapture(g->cap_stream, cudaStreamCaptureModeThreadLocal));
             for (size_t j = 0; j < n; ++j) g->hs[j]->stream = g->cap_stream;
             s = group_pack(g, vs, ws, Ks);

@@ -14,7 +14,9 @@ namespace {
 
 constexpr int PACK_THREADS = 512;
 
-__device__ __forceinline__ void store_split(const PackArgs &a, size_t idx, float val) {
+// Row r (0: velocities, 1..3: virials) of step k at column d.
+__device__ __forceinline__ void store_split(const PackArgs &a, int k, int r, size_t d, float val) {
+    const size_t idx = (size_t)(4 * k + r) * a.D_ld + d;
     if (a.split == SPLIT_BF16) {
         __nv_bfloat16 hi = __float2bfloat16_rn(val);
         __nv_bfloat16 lo = __float2bfloat16_rn(val - __bfloat162float(hi));
@@ -26,7 +28,7 @@ __device__ __forceinline__ void store_split(const PackArgs &a, size_t idx, float
         static_cast<__half *>(a.Bt_hi)[idx] = hi;
         static_cast<__half *>(a.Bt_lo)[idx] = lo;
     } else {
-        a.Bt32[idx] = val;
+        a.Bd32[d * a.b_cols + 4 * k + r] = val;
     }
 }
 
@@ -130,19 +132,17 @@ __global__ void __launch_bounds__(PACK_THREADS) pack_kernel(const PackArgs a) {
     // split into hi/lo (inputs re-read from L2).
     // (direction-major columns b*npad + i when npad > 0)
     const float mul[4] = {s_mul[0], s_mul[1], s_mul[2], s_mul[3]};
-    const size_t r0 = (size_t)(4 * k) * a.D_ld;
-    const size_t ld = (size_t)a.D_ld;
     const size_t cs_i = a.npad ? 1 : 3, cs_b = a.npad ? (size_t)a.npad : 1;
     for (int i = threadIdx.x; i < a.N; i += PACK_THREADS) {
         const float sm = a.sqm[i], ism = a.isqm[i];
 #pragma unroll
         for (int b = 0; b < 3; ++b)
-            store_split(a, r0 + cs_i * i + cs_b * b, (sm * v[(size_t)i * 3 + b]) * mul[0]);
+            store_split(a, k, 0, cs_i * i + cs_b * b, (sm * v[(size_t)i * 3 + b]) * mul[0]);
 #pragma unroll
         for (int al = 0; al < 3; ++al)
 #pragma unroll
             for (int b = 0; b < 3; ++b)
-                store_split(a, r0 + (1 + al) * ld + cs_i * i + cs_b * b,
+                store_split(a, k, 1 + al, cs_i * i + cs_b * b,
                             (W[(size_t)i * 9 + 3 * al + b] * ism) * mul[1 + al]);
     }
 }
@@ -159,14 +159,8 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
     return v;
 }
 
-// Four consecutive values of one row: one 8-byte store each for hi and lo (16-byte for FP32).
-__device__ __forceinline__ void store_split4(const PackArgs &a, size_t idx, float x0, float x1,
-                                             float x2, float x3) {
-    if (a.split == SPLIT_FP32) {
-        *reinterpret_cast<float4 *>(a.Bt32 + idx) = make_float4(x0, x1, x2, x3);
-        return;
-    }
-    const float x[4] = {x0, x1, x2, x3};
+// Four consecutive values of one row: one 8-byte store each for hi and lo.
+__device__ __forceinline__ void store_split4(const PackArgs &a, size_t idx, const float (&x)[4]) {
     uint32_t h[4], l[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -347,15 +341,21 @@ __device__ __forceinline__ void pack_bulk_body(const PackArgs &a, int k, uint32_
                 }
                 col = 3 * (size_t)a0 + 4 * (size_t)g;
             }
-            float x[4];
+            float x[4][4];   // [row][value]
 #pragma unroll
-            for (int e = 0; e < 4; ++e) x[e] = sv[3 * ia[e] + bb[e]] * s_mul[0];
-            store_split4(a, r0 + col, x[0], x[1], x[2], x[3]);
+            for (int e = 0; e < 4; ++e) {
+                x[0][e] = sv[3 * ia[e] + bb[e]] * s_mul[0];
 #pragma unroll
-            for (int al = 0; al < 3; ++al) {
+                for (int al = 0; al < 3; ++al) x[1 + al][e] = sw[9 * ia[e] + 3 * al + bb[e]] * s_mul[1 + al];
+            }
+            if (a.split == SPLIT_FP32) {   // d-major: the step's four rows are 16 bytes of a d
 #pragma unroll
-                for (int e = 0; e < 4; ++e) x[e] = sw[9 * ia[e] + 3 * al + bb[e]] * s_mul[1 + al];
-                store_split4(a, r0 + (size_t)(1 + al) * ld + col, x[0], x[1], x[2], x[3]);
+                for (int e = 0; e < 4; ++e)
+                    *reinterpret_cast<float4 *>(a.Bd32 + (col + e) * a.b_cols + 4 * k) =
+                        make_float4(x[0][e], x[1][e], x[2][e], x[3][e]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) store_split4(a, r0 + (size_t)r * ld + col, x[r]);
             }
         }
     }
@@ -418,7 +418,7 @@ int pack_threads(int N) { return N <= 4 * 128 ? 128 : N <= 8 * 1024 ? 256 : 512;
 bool bulk_ok(const PackArgs &a) {
     const auto al16 = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
     return a.N % 4 == 0 && al16(a.v) && al16(a.W) && al16(a.sqm) && al16(a.isqm) &&
-           (a.split == SPLIT_FP32 ? al16(a.Bt32) : true);
+           (a.split == SPLIT_FP32 ? al16(a.Bd32) : true);
 }
 
 template <int THREADS>

@@ -68,6 +68,10 @@ __global__ void prepare_kernel(const T *E, int layout, int64_t ld, int64_t D, in
     }
     __syncthreads();
     for (int r = ty; r < 32; r += 8) {
+        if (SPLIT == SPLIT_FP32_D) {   // d-major: Et32[d][n], row pitch M_pad
+            Et32[(size_t)(d0 + r) * ((size_t)gridDim.y * 32) + n0 + tx] = (float)(tile[tx][r] * scale);
+            continue;
+        }
         const int64_t n = n0 + r, d = d0 + tx;
         const double x = tile[r][tx] * scale;
         const size_t idx = (size_t)n * D_ld + d;
@@ -144,10 +148,12 @@ void launch_prepare_modes(const void *E, int dtype, int layout, int64_t ld, int6
     if (dtype == 1) {
         if (split == SPLIT_BF16) MHC_PREP(double, SPLIT_BF16);
         else if (split == SPLIT_FP16) MHC_PREP(double, SPLIT_FP16);
+        else if (split == SPLIT_FP32_D) MHC_PREP(double, SPLIT_FP32_D);
         else MHC_PREP(double, SPLIT_FP32);
     } else {
         if (split == SPLIT_BF16) MHC_PREP(float, SPLIT_BF16);
         else if (split == SPLIT_FP16) MHC_PREP(float, SPLIT_FP16);
+        else if (split == SPLIT_FP32_D) MHC_PREP(float, SPLIT_FP32_D);
         else MHC_PREP(float, SPLIT_FP32);
     }
 #undef MHC_PREP

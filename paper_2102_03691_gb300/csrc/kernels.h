@@ -8,6 +8,7 @@
 namespace mhc {
 
 enum Split { SPLIT_FP32 = 0, SPLIT_BF16 = 1, SPLIT_FP16 = 2 };
+constexpr int SPLIT_FP32_D = 3;   // launch_prepare_modes: FP32, stored d-major
 
 constexpr int TC_MAX_GROUP = 16;  // systems per grouped launch
 constexpr int TC_MAX_SPLIT = 16;  // d-axis splits of one projection
@@ -39,7 +40,8 @@ struct PackArgs {
     long long t0;          // global index of the block's first step (if t0_dev is null)
     const long long *t0_dev;   // device step counter read at run time (graph replay)
     void *Bt_hi, *Bt_lo;   // [rows][D_ld] 16-bit (split != FP32)
-    float *Bt32;           // [rows][D_ld] (split == FP32)
+    float *Bd32;           // [D_ld][b_cols], d-major: step k in columns 4k .. 4k+3 (split == FP32)
+    int b_cols;
     float *col_scale;      // [4K] 2^-(s_row + e_exp): undoes both power-of-two scales
     double *Jtot;          // [K][3]
     double *Jring;         // [R][3] ring of past J (GKMA) or null
@@ -73,6 +75,7 @@ void launch_max_abs(const void *E, int dtype, int layout, int64_t ld, int64_t D,
                     unsigned *out_bits, cudaStream_t s);
 // Gather the kept modes in bin order (perm), transpose to mode-major and split:
 //   Et[n'][c] = E[d(c), perm[n']] * 2^e_exp   (zero for n' >= M_eff or d(c) >= D)
+// (SPLIT_FP32_D: Et[c][n'], row pitch M_pad)
 // with d(c) = c (npad == 0) or, direction-major, d(b*npad + i) = 3i+b for i < D/3.
 void launch_prepare_modes(const void *E, int dtype, int layout, int64_t ld, int64_t D,
                           int64_t M_eff, const int *perm, int e_exp, int split, void *Et_hi,
@@ -84,20 +87,54 @@ void launch_orthonormality(const void *E, int dtype, int layout, int64_t ld, int
                            unsigned long long *out_bits, cudaStream_t s);
 
 // ---------------------------------------------------------------- FP32 path
-// R[c][n] = sum_{d < Dk} Bt32[c][d] Et32[n][d] for c < C (rows of the block), n < Mp;
-// both operands have row pitch ld (Dk a multiple of 16).
 // Measured FP32 FMA throughput of the device (the comparison path's peak), TFLOP/s.
 cudaError_t measure_fp32_fma(cudaStream_t s, int sm_count, double *tflops);
-void launch_sgemm(const float *Et32, const float *Bt32, float *R, int Dk, int ld, int Mp, int C,
-                  cudaStream_t s);
-// J_n^a(k) = R[4k][n] R[4k+1+a][n]; segmented bin sums into partials[k][a][slot].
-void launch_fp32_bin_epilogue(const float *R, int Mp, int K, const int *mode_bin,
-                              const int *mode_slot, float *partials, int n_slots, cudaStream_t s);
-// Direction-resolved epilogue over the three per-direction products R_b = R + b*rstride:
-// Xdot = sum_b R_b[4k][n], J_n^{ab}(k) = Xdot R_b[4k+1+a][n]; bin-run sums into
-// partials[k][a][b*n_slots + slot].
-void launch_fp32_dir_epilogue(const float *R, size_t rstride, int Mp, int K, const int *mode_bin,
-                              const int *mode_slot, float *partials, int n_slots, cudaStream_t s);
+
+// The product R[c][n] = sum_{d < Dk} Bd32[d][c] Ed32[d][n] of a block (c < C, n < Mp), once for
+// each of ndir segments of d (segment b at rows b Dk).  Tiles of 128 modes x 128 columns, mode
+// tile major; the tiles below t0 (whole waves of `ctas` CTAs) run whole, the chunks of the others
+// (nch of SGEMM_CHUNK d's each) are cut into `parts` ranges of equal length (to one chunk), one a
+// CTA.  Range q starts at tail chunk floor(q T / parts); a tile's segments are the ranges that
+// touch it, in chunk order.
+constexpr int SGEMM_CHUNK = 128;    // d elements
+constexpr int SGEMM_MAX_SEG = 8;    // most pieces of a tile (planes of R)
+struct SgemmPlan {
+    int ndir, n_mt, n_ct, n_kb, nch, tiles, t0, parts, ctas, max_seg;
+    __host__ __device__ long long tail_chunks() const { return (long long)(tiles - t0) * nch; }
+    __host__ __device__ long long part_begin(int q) const { return (long long)q * tail_chunks() / parts; }
+    __host__ __device__ int part_of(long long g) const {   // the largest q with part_begin(q) <= g
+        const long long T = tail_chunks();
+        return (int)(((g + 1) * parts + T - 1) / T - 1);
+    }
+    // k-block of tail chunk g in the tail's tiles laid end to end (chunk_kb k-blocks a chunk)
+    __host__ __device__ int tail_kb(long long g, int chunk_kb) const {
+        const int tl = (int)(g / nch);
+        return tl * n_kb + (int)(g - (long long)tl * nch) * chunk_kb;
+    }
+    __host__ __device__ int segments(int tile) const {
+        if (tile < t0) return 1;
+        const long long g0 = (long long)(tile - t0) * nch;
+        return 1 + part_of(g0 + nch - 1) - part_of(g0);
+    }
+};
+struct SgemmParams {
+    CUtensorMap tmA, tmB;   // Ed32 [D][Mp], Bd32 [D][cols]: boxes of 16 d's x 128
+    float *R;               // plane s of direction b: R + (s ndir + b) rstride, [C][Mp]
+    size_t rstride;
+    SgemmPlan plan;
+    int C, Mp, dir_cols;    // dir_cols: d's of a direction segment (0 without the split)
+    long long wait_limit;   // SM cycles a barrier wait may take before the CTA gives up
+    int *status;
+};
+// cut false: every tile runs whole (R is one plane).
+SgemmPlan sgemm_plan(int64_t Mp, int C, int64_t Dk, int ndir, int sms, bool cut);
+int sgemm_make_maps(const float *Ed32, int64_t Mp, const float *Bd32, int64_t cols, int64_t D, SgemmParams &p);
+cudaError_t launch_sgemm(const SgemmParams &p, cudaStream_t s);
+// From the product (its planes added in order): J_n^a(k) = R[4k][n] R[4k+1+a][n], segmented bin
+// sums into partials[k][a][slot]; with three direction segments R_b, Xdot = sum_b R_b[4k][n] and
+// J_n^{ab}(k) = Xdot R_b[4k+1+a][n] into partials[k][a][b*n_slots + slot].
+void launch_fp32_epilogue(const SgemmParams &p, int K, const int *mode_bin, const int *mode_slot,
+                          float *partials, int n_slots, cudaStream_t s);
 
 // ---------------------------------------------------------------- tensor-core path
 constexpr int TC_BM = 128;        // modes per tile = TMEM lanes
@@ -168,6 +205,9 @@ bool tc_config_supported(const TcConfig &c);
 // Encode a 2D 16-bit tensor map: rows x cols (cols innermost, row pitch ld elements).
 int tc_make_tmap(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint64_t ld,
                  uint32_t box_rows, uint32_t box_cols);
+// The same for FP32, unswizzled.
+int tc_make_tmap_f32(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint64_t ld,
+                     uint32_t box_rows, uint32_t box_cols);
 cudaError_t launch_tc_single(const TcParams<1> &p, const TcConfig &c, cudaStream_t s);
 // With prob[0].n_split > 1: sum the splits' partial projections of the block (in split order)
 // and run the tile epilogue (Eq. 16 product, bin-run sums into partials).

@@ -69,6 +69,20 @@ int mhc::tc_make_tmap(CUtensorMap *m, const void *base, uint64_t rows, uint64_t 
     return r == CUDA_SUCCESS ? 0 : (int)r;
 }
 
+int mhc::tc_make_tmap_f32(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint64_t ld,
+                          uint32_t box_rows, uint32_t box_cols) {
+    auto fn = tmap_encode_fn();
+    if (!fn) return -1;
+    cuuint64_t dims[2] = {cols, rows};
+    cuuint64_t strides[1] = {ld * 4};
+    cuuint32_t box[2] = {box_cols, box_rows};
+    cuuint32_t estr[2] = {1, 1};
+    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(base), dims, strides, box,
+                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? 0 : (int)r;
+}
+
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
@@ -140,6 +154,7 @@ struct mhc_handle {
     TcConfig tc{256, 64, 2, 0, 0};
     std::map<int, TcConfig> tuned;  // K -> config
     TcParams<1> tcp{};
+    SgemmParams sgp{};    // FP32 path
     XcPlan xc_plan{};     // cross-correlations (MHC_FLAG_XCORR): tensor-core plan and parameters
     XcTcParams xcp{};
 };
@@ -338,6 +353,11 @@ int sched_units(const mhc_handle *h, const TcConfig &c) {
     return std::max(1, h->sm_count / 2);
 }
 
+// The FP32 path's tiles and cuts for C columns (with the direction split, one product a segment).
+SgemmPlan fp32_plan(const mhc_handle *h, int C) {
+    return sgemm_plan(h->M_pad, C, h->dir ? h->N_pad : h->D_ld, h->dir ? 3 : 1, h->sm_count, true);
+}
+
 // Sort kept modes by bin (stable), build the per-mode bin/slot tables of the fused
 // epilogue, gather+split E into the stored order and set up the tensor maps.
 mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_t B) {
@@ -410,22 +430,35 @@ mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_
     // stored eigenvectors
     const size_t ecount = (size_t)h->M_pad * h->D_ld;
     if (is_tc(h)) {
-        dev_free(h, "Et32");
+        dev_free(h, "Ed32");
         if ((s = dev_alloc(h, "Et_hi", ecount * 2, false)) != MHC_OK) return s;
         if ((s = dev_alloc(h, "Et_lo", ecount * 2, false)) != MHC_OK) return s;
         if (h->dir && (s = dev_alloc(h, "dir_park", sizeof(float) * DIR_PARK_CTA_FLOATS * h->sm_count,
                                      false)) != MHC_OK)
             return s;
     } else {
-        if ((s = dev_alloc(h, "Et32", ecount * 4, false)) != MHC_OK) return s;
-        if ((s = dev_alloc(h, "R", sizeof(float) * h->B_rows * h->M_pad * (h->dir ? 3 : 1), false)) != MHC_OK)
+        if ((s = dev_alloc(h, "Ed32", ecount * 4, false)) != MHC_OK) return s;
+        // planes of R: the most that any block length up to k_max cuts a tile into
+        size_t worst = 1;
+        for (int nct = 1; nct <= (4 * K + 127) / 128; ++nct)
+            worst = std::max(worst, (size_t)fp32_plan(h, 128 * nct).max_seg);
+        if ((s = dev_alloc(h, "R", sizeof(float) * worst * h->B_rows * h->M_pad * (h->dir ? 3 : 1), false)) != MHC_OK)
             return s;
+        SgemmParams &P = h->sgp;
+        if (sgemm_make_maps(dptr<float>(h, "Ed32"), h->M_pad, dptr<float>(h, "Bd32"), h->B_rows, h->D_ld, P))
+            return fail(h, MHC_ERR_CUDA, "cuTensorMapEncodeTiled failed");
+        P.R = dptr<float>(h, "R");
+        P.rstride = (size_t)h->B_rows * h->M_pad;
+        P.Mp = (int)h->M_pad;
+        P.dir_cols = (int)h->N_pad;
+        P.wait_limit = 2000000000ll;
+        P.status = h->status;
     }
     // Eraw is already in the stored column order (direction-major with the split)
     launch_prepare_modes(dptr<float>(h, "Eraw"), MHC_F32, MHC_MODE_MAJOR, h->D_ld,
                          h->dir ? h->D_ld : h->D, h->M_eff, dptr<int>(h, "perm"), h->e_exp,
-                         h->split, dptr<void>(h, "Et_hi"), dptr<void>(h, "Et_lo"),
-                         dptr<float>(h, "Et32"), h->D_ld, h->M_pad, 0, h->stream);
+                         is_tc(h) ? h->split : SPLIT_FP32_D, dptr<void>(h, "Et_hi"),
+                         dptr<void>(h, "Et_lo"), dptr<float>(h, "Ed32"), h->D_ld, h->M_pad, 0, h->stream);
     h->launches++;
     MHC_CUDA(h, cudaGetLastError());
 
@@ -537,26 +570,14 @@ mhc_status run_projection(mhc_handle *h, int K) {
                                     sizeof(float) * K * 3 * slot_stride(h), h->stream));
         return MHC_OK;
     }
-    if (!is_tc(h) && h->dir) {
-        // one product per direction segment of d, then Xdot = sum over segments
-        const size_t rstride = (size_t)h->B_rows * h->M_pad;
-        for (int b = 0; b < 3; ++b)
-            launch_sgemm(dptr<float>(h, "Et32") + b * h->N_pad, dptr<float>(h, "Bt32") + b * h->N_pad,
-                         dptr<float>(h, "R") + b * rstride, (int)h->N_pad, (int)h->D_ld,
-                         (int)h->M_pad, 4 * K, h->stream);
-        launch_fp32_dir_epilogue(dptr<float>(h, "R"), rstride, (int)h->M_pad, K,
-                                 dptr<int>(h, "mode_bin"), dptr<int>(h, "mode_slot"),
-                                 dptr<float>(h, "partials"), (int)h->n_slots, h->stream);
-        h->launches += 4;
-        MHC_CUDA(h, cudaGetLastError());
-        return MHC_OK;
-    }
     if (!is_tc(h)) {
-        launch_sgemm(dptr<float>(h, "Et32"), dptr<float>(h, "Bt32"), dptr<float>(h, "R"),
-                     (int)h->D_ld, (int)h->D_ld, (int)h->M_pad, 4 * K, h->stream);
-        launch_fp32_bin_epilogue(dptr<float>(h, "R"), (int)h->M_pad, K, dptr<int>(h, "mode_bin"),
-                                 dptr<int>(h, "mode_slot"), dptr<float>(h, "partials"),
-                                 (int)h->n_slots, h->stream);
+        // with the direction split one product per segment of d, then Xdot = sum over segments
+        SgemmParams &P = h->sgp;
+        P.C = 4 * K;
+        P.plan = fp32_plan(h, P.C);
+        MHC_CUDA(h, launch_sgemm(P, h->stream));
+        launch_fp32_epilogue(P, K, dptr<int>(h, "mode_bin"), dptr<int>(h, "mode_slot"),
+                             dptr<float>(h, "partials"), (int)h->n_slots, h->stream);
         h->launches += 2;
         MHC_CUDA(h, cudaGetLastError());
         return MHC_OK;
@@ -855,7 +876,8 @@ PackArgs pack_args(mhc_handle *h, const float *v, const float *W, int K) {
     a.t0_dev = dptr<long long>(h, "steps_dev");
     a.Bt_hi = dptr<void>(h, "Bt_hi");
     a.Bt_lo = dptr<void>(h, "Bt_lo");
-    a.Bt32 = dptr<float>(h, "Bt32");
+    a.Bd32 = dptr<float>(h, "Bd32");
+    a.b_cols = (int)h->B_rows;
     a.col_scale = dptr<float>(h, "col_scale");
     a.Jtot = dptr<double>(h, "Jtot");
     a.Jring = (h->prm.flags & MHC_FLAG_GKMA) ? dptr<double>(h, "Jring") : nullptr;
@@ -1275,11 +1297,11 @@ mhc_status mhc_set_modes(mhc_handle *h, int64_t n_atoms, int64_t n_modes, const 
     MHC_CUDA(h, cudaMemcpyAsync(dptr<float>(h, "isqm"), isq.data(), 4 * n_atoms, cudaMemcpyHostToDevice, h->stream));
     const size_t bcount = (size_t)h->B_rows * h->D_ld;
     if (is_tc(h)) {
-        dev_free(h, "Bt32");
+        dev_free(h, "Bd32");
         if ((s = dev_alloc(h, "Bt_hi", bcount * 2)) != MHC_OK) return s;
         if ((s = dev_alloc(h, "Bt_lo", bcount * 2)) != MHC_OK) return s;
     } else {
-        if ((s = dev_alloc(h, "Bt32", bcount * 4)) != MHC_OK) return s;
+        if ((s = dev_alloc(h, "Bd32", bcount * 4)) != MHC_OK) return s;
     }
     if ((s = dev_alloc(h, "col_scale", sizeof(float) * 4 * K)) != MHC_OK) return s;
     if ((s = dev_alloc(h, "Jtot", sizeof(double) * 3 * K)) != MHC_OK) return s;

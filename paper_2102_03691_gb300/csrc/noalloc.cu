@@ -137,15 +137,15 @@ extern "C" mhc_status mhc_binned_current_noalloc(int32_t n_atoms, int32_t n_mode
     int *mode_bin = reinterpret_cast<int *>(s + o_bin);
     int *mode_slot = reinterpret_cast<int *>(s + o_slot);
     int *slot_begin = reinterpret_cast<int *>(s + o_sbeg);
-    float *Et32 = reinterpret_cast<float *>(s + o_E);
-    float *Bt32 = reinterpret_cast<float *>(s + o_Bt);
+    float *Ed32 = reinterpret_cast<float *>(s + o_E);
+    float *Bd32 = reinterpret_cast<float *>(s + o_Bt);
     float *partials = reinterpret_cast<float *>(s + o_part);
     double *hsum = reinterpret_cast<double *>(s + o_hsum);
     double *jsum = reinterpret_cast<double *>(s + o_jsum);
 
     // cleared every call: status word, B-operand padding columns, HNEMA sums
     e = cudaMemsetAsync(status, 0, sizeof(int), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(Bt32, 0, sizeof(float) * B_rows * D_ld, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(Bd32, 0, sizeof(float) * B_rows * D_ld, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(hsum, 0, o_jsum + sizeof(double) * 3 - o_hsum, st);
     if (e != cudaSuccess) return MHC_ERR_CUDA;
     noalloc_tables_kernel<<<1, 256, 0, st>>>(bin_of_mode, (int)M, (int)M_pad, n_bins, mass_amu,
@@ -160,8 +160,8 @@ extern "C" mhc_status mhc_binned_current_noalloc(int32_t n_atoms, int32_t n_mode
         (e = cudaStreamSynchronize(st)) != cudaSuccess)
         return MHC_ERR_CUDA;
     if (h_status) return MHC_ERR_INVALID_ARG;
-    launch_prepare_modes(E, MHC_F32, MHC_MODE_MAJOR, ld, D, M, perm, 0, SPLIT_FP32, nullptr,
-                         nullptr, Et32, D_ld, M_pad, 0, st);
+    launch_prepare_modes(E, MHC_F32, MHC_MODE_MAJOR, ld, D, M, perm, 0, SPLIT_FP32_D, nullptr,
+                         nullptr, Ed32, D_ld, M_pad, 0, st);
     PackArgs a{};
     a.v = v;
     a.W = W;
@@ -171,18 +171,30 @@ extern "C" mhc_status mhc_binned_current_noalloc(int32_t n_atoms, int32_t n_mode
     a.K = K;
     a.D_ld = (int)D_ld;
     a.split = SPLIT_FP32;
-    a.Bt32 = Bt32;
+    a.Bd32 = Bd32;
+    a.b_cols = (int)B_rows;
     a.col_scale = reinterpret_cast<float *>(s + o_cs);
     a.Jtot = J;
     launch_pack(a, st);
-    launch_sgemm(Et32, Bt32, reinterpret_cast<float *>(s + o_R), (int)D_ld, (int)D_ld, (int)M_pad,
-                 4 * K, st);
-    launch_fp32_bin_epilogue(reinterpret_cast<float *>(s + o_R), (int)M_pad, K, mode_bin, mode_slot,
-                             partials, (int)M_pad, st);
+    // the scratch holds one plane of the product: every tile runs whole
+    SgemmParams P{};
+    if (sgemm_make_maps(Ed32, M_pad, Bd32, B_rows, D_ld, P)) return MHC_ERR_CUDA;
+    P.R = reinterpret_cast<float *>(s + o_R);
+    P.rstride = (size_t)B_rows * M_pad;
+    P.C = 4 * K;
+    P.Mp = (int)M_pad;
+    P.wait_limit = 2000000000ll;
+    P.status = status;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return MHC_ERR_CUDA;
+    P.plan = sgemm_plan(M_pad, P.C, D_ld, 1, sms, false);
+    if ((e = launch_sgemm(P, st)) != cudaSuccess) return MHC_ERR_CUDA;
+    launch_fp32_epilogue(P, K, mode_bin, mode_slot, partials, (int)M_pad, st);
     launch_bin_finish(partials, (int)M_pad, slot_begin, n_bins, K, Jb, hsum, J, jsum, nullptr, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return MHC_ERR_CUDA;
     if ((e = cudaMemcpyAsync(&h_status, status, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
         (e = cudaStreamSynchronize(st)) != cudaSuccess)
         return MHC_ERR_CUDA;
+    if (h_status == DEV_TIMEOUT) return MHC_ERR_TIMEOUT;
     return h_status ? MHC_ERR_INVALID_ARG : MHC_OK;
 }

@@ -67,7 +67,7 @@ struct Unit {
 // last, partial wave is spread over all of them instead of leaving most idle.  Tail-local chunk
 // g; part q starts at chunk floor(q T / sk_parts), T = the tail's chunks.
 __device__ __forceinline__ long long sk_tail_chunks(const TcProblem &P) {
-    return (long long)(P.n_tiles - P.sk_t0) * P.sk_nch;
+    return (long long)(P.n_tiles - P.sk_t0) * P.sk_sub * P.sk_nch;
 }
 __device__ __forceinline__ long long sk_begin(const TcProblem &P, int q) {
     return (long long)q * sk_tail_chunks(P) / P.sk_parts;
@@ -77,12 +77,12 @@ __device__ __forceinline__ int sk_part_of(const TcProblem &P, long long g) {
     const long long T = sk_tail_chunks(P);
     return (int)(((g + 1) * P.sk_parts + T - 1) / T - 1);
 }
-// Segments of a tile under the balanced split (1: one part holds the whole tile).  Every tail
-// part holds at least one chunk (sk_parts <= T), so the segments of a tail tile are the parts
-// that touch it, in chunk order.
-__device__ __forceinline__ int sk_segments(const TcProblem &P, int tile) {
+// Segments of sub-tile `sub` of a tile (a tile has one without the direction split) under the
+// balanced split (1: one part holds all of it).  Every tail part holds at least one chunk
+// (sk_parts <= T), so the segments of a sub-tile are the parts that touch it, in chunk order.
+__device__ __forceinline__ int sk_segments(const TcProblem &P, int tile, int sub = 0) {
     if (tile < P.sk_t0) return 1;
-    const long long g0 = (long long)(tile - P.sk_t0) * P.sk_nch;
+    const long long g0 = ((long long)(tile - P.sk_t0) * P.sk_sub + sub) * P.sk_nch;
     return 1 + sk_part_of(P, g0 + P.sk_nch - 1) - sk_part_of(P, g0);
 }
 
@@ -127,15 +127,18 @@ struct UnitIter {
                 return true;
             }
             if (g >= g_end) return false;
-            const int tl = (int)(g / P.sk_nch), tile = P.sk_t0 + tl;
-            const int c0 = (int)(g - (long long)tl * P.sk_nch);
+            const int sl = (int)(g / P.sk_nch), tl = sl / P.sk_sub, sub = sl - tl * P.sk_sub;
+            const int tile = P.sk_t0 + tl;
+            const int c0 = (int)(g - (long long)sl * P.sk_nch);
             const int c1 = (int)min((long long)P.sk_nch, (long long)c0 + (g_end - g));
             u.prob = 0;
             u.mt = tile / P.n_col_tiles;
             u.ct = tile - u.mt * P.n_col_tiles;
-            u.kb_lo = c0 * CHUNK_KB;
-            u.kb_hi = min(P.n_kb, c1 * CHUNK_KB);
-            u.seg = (c0 == 0 && c1 == P.sk_nch) ? -1 : sk_part_of(P, g) - sk_part_of(P, g - c0);
+            u.kb_lo = (sub * P.sk_nch + c0) * CHUNK_KB;
+            u.kb_hi = min(P.n_kb, (sub * P.sk_nch + c1) * CHUNK_KB);
+            u.seg = (P.sk_sub == 1 && c0 == 0 && c1 == P.sk_nch)
+                        ? -1
+                        : sub * P.sk_planes + sk_part_of(P, g) - sk_part_of(P, g - c0);
             g += c1 - c0;
             return true;
         }
@@ -455,7 +458,9 @@ __global__ void __launch_bounds__(128 + BN, 1) tc_modal_kernel(const __grid_cons
                 tc_fence_before();
                 mbar_arrive(&acc_empty[abuf]);
                 if (++abuf == 2) { abuf = 0; aphase ^= 1u; }
-                if constexpr (DIR) dir_maybe_park(acc, P, kb0 + CHUNK_KB);
+                if constexpr (DIR) {
+                    if (u.seg < 0) dir_maybe_park(acc, P, kb0 + CHUNK_KB);
+                }
             }
             if (!ok) break;
             if (u.seg >= 0) {   // the split finish kernel adds the segments and runs the epilogue
@@ -696,7 +701,9 @@ __global__ void __launch_bounds__(128 + BN, 1) tc_modal_pair_kernel(const __grid
                     else mbar_arrive_cluster_relaxed(empty_leader[abuf]);
                 }
                 if (++abuf == 2) { abuf = 0; aphase ^= 1u; }
-                if constexpr (DIR) dir_maybe_park(acc, P, kb0 + CHUNK_KB);
+                if constexpr (DIR) {
+                    if (u.seg < 0) dir_maybe_park(acc, P, kb0 + CHUNK_KB);
+                }
             }
             if (!ok) break;
             if (u.seg >= 0) {   // the split finish kernel adds the segments and runs the epilogue
@@ -819,33 +826,17 @@ cudaError_t dispatch(const TcParams<NPROB> &p, const TcConfig &c, cudaStream_t s
 // held whole return at once (the projection kernel ran their epilogue).  The segments come
 // into shared memory by 16-byte asynchronous copies, FIN_SEGS at a time (up to 16 KB a warp
 // in flight without holding registers), and each lane then reads its own mode's values.
+// With the direction split (DIR) the three sub-tiles' sums are formed one after the other, Xdot
+// is their sum, and each direction's bracket sums take the epilogue.
 constexpr int FIN_STEPS = 8;
 constexpr int FIN_SEGS = 4;
 constexpr int FIN_COLS = 4 * FIN_STEPS;                          // columns of a warp
 constexpr int FIN_SMEM = 4 * FIN_SEGS * FIN_COLS * 32 * 4;       // 4 warps, 64 KB
-__global__ void __launch_bounds__(128) tc_split_finish_kernel(const __grid_constant__ TcParams<1> p) {
-    extern __shared__ float4 fin_smem4[];
-    griddep_launch_dependents();
-    griddep_wait();   // the projection's stored segments
-    const TcProblem &P = p.prob[0];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = blockIdx.x * 4 + warp;   // 32-mode group (warp-uniform)
-    if (g * 32 >= P.m_pad) return;
-    const int n0 = g * 32;
-    const int kbase = blockIdx.y * FIN_STEPS;
-    const int c0 = kbase * 4;              // first of the warp's columns
-    int nseg = P.n_split;
-    if (P.sk_parts > 0) {
-        nseg = sk_segments(P, (n0 / P.sk_tm) * P.n_col_tiles + c0 / P.sk_bn);
-        if (nseg < 2) return;
-    }
-    const int bin = P.mode_bin[n0 + lane];
-    const int slot = P.mode_slot[n0 + lane];
-    const uint32_t take = seg_scan_masks(bin, lane);
-    float *st = reinterpret_cast<float *>(fin_smem4) + (size_t)warp * FIN_SEGS * FIN_COLS * 32;
+// acc += the planes p0 .. p0 + nseg - 1 of the warp's columns c0 .. of the 32 modes from n0
+__device__ __forceinline__ void fin_add(float (&acc)[FIN_COLS], const TcProblem &P, int p0, int nseg, int c0,
+                                        int n0, float *st, int lane) {
     const size_t sstride = (size_t)P.ws_cols * P.m_pad;
-    const float *src = P.split_ws + (size_t)c0 * P.m_pad + n0;
-    float acc[FIN_COLS];
+    const float *src = P.split_ws + p0 * sstride + (size_t)c0 * P.m_pad + n0;
 #pragma unroll
     for (int j = 0; j < FIN_COLS; ++j) acc[j] = 0.f;
     for (int s0 = 0; s0 < nseg; s0 += FIN_SEGS) {
@@ -863,8 +854,51 @@ __global__ void __launch_bounds__(128) tc_split_finish_kernel(const __grid_const
             for (int j = 0; j < FIN_COLS; ++j) acc[j] += st[(s * FIN_COLS + j) * 32 + lane];
         __syncwarp();                  // the staging area is refilled by the next batch
     }
-    epilogue_steps<FIN_STEPS>(acc, step_scales(P, kbase, lane), P, kbase, take, slot,
-                              (size_t)P.n_slots, 0);
+}
+
+template <bool DIR>
+__global__ void __launch_bounds__(128) tc_split_finish_kernel(const __grid_constant__ TcParams<1> p) {
+    extern __shared__ float4 fin_smem4[];
+    griddep_launch_dependents();
+    griddep_wait();   // the projection's stored segments
+    const TcProblem &P = p.prob[0];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = blockIdx.x * 4 + warp;   // 32-mode group (warp-uniform)
+    if (g * 32 >= P.m_pad) return;
+    const int n0 = g * 32;
+    const int kbase = blockIdx.y * FIN_STEPS;
+    const int c0 = kbase * 4;              // first of the warp's columns
+    int nseg = P.n_split, tile = 0;
+    if (P.sk_parts > 0) {
+        tile = (n0 / P.sk_tm) * P.n_col_tiles + c0 / P.sk_bn;
+        nseg = sk_segments(P, tile);
+        if (DIR ? tile < P.sk_t0 : nseg < 2) return;
+    }
+    const int bin = P.mode_bin[n0 + lane];
+    const int slot = P.mode_slot[n0 + lane];
+    const uint32_t take = seg_scan_masks(bin, lane);
+    float *st = reinterpret_cast<float *>(fin_smem4) + (size_t)warp * FIN_SEGS * FIN_COLS * 32;
+    const float4 sc = step_scales(P, kbase, lane);
+    if constexpr (!DIR) {
+        float acc[FIN_COLS];
+        fin_add(acc, P, 0, nseg, c0, n0, st, lane);
+        epilogue_steps<FIN_STEPS>(acc, sc, P, kbase, take, slot, (size_t)P.n_slots, 0);
+    } else {
+        float acc[3][FIN_COLS];
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+            fin_add(acc[b], P, b * P.sk_planes, sk_segments(P, tile, b), c0, n0, st, lane);
+#pragma unroll
+        for (int s = 0; s < FIN_STEPS; ++s) {
+            const float x = (acc[0][4 * s] + acc[1][4 * s]) + acc[2][4 * s];
+#pragma unroll
+            for (int b = 0; b < 3; ++b) acc[b][4 * s] = x;
+        }
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+            epilogue_steps<FIN_STEPS>(acc[b], sc, P, kbase, take, slot, 3 * (size_t)P.n_slots,
+                                      (size_t)b * P.n_slots);
+    }
 }
 
 }  // namespace
@@ -873,9 +907,11 @@ cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s) {
     const TcProblem &P = p.prob[0];
     if ((P.n_split <= 1 && P.sk_parts <= 0) || !P.split_ws || P.m_pad % 128 || P.ws_cols % FIN_COLS)
         return cudaErrorInvalidValue;
-    static const cudaError_t smem_ok = cudaFuncSetAttribute(
-        tc_split_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FIN_SMEM);
-    if (smem_ok != cudaSuccess) return smem_ok;
+    static const cudaError_t smem_ok[2] = {
+        cudaFuncSetAttribute(tc_split_finish_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FIN_SMEM),
+        cudaFuncSetAttribute(tc_split_finish_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FIN_SMEM)};
+    const bool dir = P.dir_seg_kb > 0;
+    if (smem_ok[dir] != cudaSuccess) return smem_ok[dir];
     const dim3 grid((unsigned)(P.m_pad / 128), (unsigned)((P.K + FIN_STEPS - 1) / FIN_STEPS));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -887,7 +923,8 @@ cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tc_split_finish_kernel, p);
+    return dir ? cudaLaunchKernelEx(&cfg, tc_split_finish_kernel<true>, p)
+               : cudaLaunchKernelEx(&cfg, tc_split_finish_kernel<false>, p);
 }
 
 const TcConfig TC_CONFIGS[TC_NUM_CONFIGS] = {
@@ -917,11 +954,13 @@ cudaError_t launch_tc_single(const TcParams<1> &p, const TcConfig &c, cudaStream
                           P.kb_split % (PROMOTE_D / c.bk)))
         return cudaErrorInvalidValue;
     const int parts = c.grid / (c.pair ? 2 : 1);
-    if (P.sk_parts > 0 && (P.dir_seg_kb || !P.split_ws || P.sk_bn != c.bn ||
-                           P.sk_nch != (P.n_kb + PROMOTE_D / c.bk - 1) / (PROMOTE_D / c.bk) ||
+    const int chunk_kb = PROMOTE_D / c.bk;
+    if (P.sk_parts > 0 && (!P.split_ws || P.sk_bn != c.bn || P.sk_sub != (P.dir_seg_kb ? 3 : 1) ||
+                           (P.dir_seg_kb ? P.sk_sub * P.sk_nch * chunk_kb != P.n_kb || P.sk_planes < 1
+                                         : P.sk_nch != (P.n_kb + chunk_kb - 1) / chunk_kb) ||
                            P.sk_tm != (c.pair ? 2 : 1) * TC_BM || P.sk_t0 < 0 ||
                            P.sk_t0 % parts || P.sk_t0 >= P.n_tiles || P.sk_parts > parts ||
-                           (long long)P.sk_parts > (long long)(P.n_tiles - P.sk_t0) * P.sk_nch))
+                           (long long)P.sk_parts > (long long)(P.n_tiles - P.sk_t0) * P.sk_sub * P.sk_nch))
         return cudaErrorInvalidValue;
     if (p.prob[0].dir_seg_kb) {
         if (!p.prob[0].dir_park || c.grid > p.dir_park_ctas) return cudaErrorInvalidValue;

@@ -166,7 +166,11 @@ struct TcProblem {   // 128-byte aligned through CUtensorMap
     // stores segment s (the s-th range that touches it, in chunk order) to split_ws[s]; the
     // finish kernel adds its segments in order.  sk_tm: modes per tile (128, or 256 for CTA
     // pairs); sk_bn: columns per tile.
-    int sk_parts, sk_nch, sk_tm, sk_bn, sk_t0;
+    // sk_sub = 3 (direction split; else 1): each direction segment of a remaining tile is a
+    // sub-tile of sk_nch chunks of its own in that chunk space, so no range's sums mix directions;
+    // sub-tile b stores its segment s to split_ws[b sk_planes + s], whole or cut, and the finish
+    // kernel forms the tile's products.
+    int sk_parts, sk_nch, sk_tm, sk_bn, sk_t0, sk_sub, sk_planes;
 };
 constexpr int DIR_PARK_THREADS = 256;                        // epilogue threads of the widest tile
 constexpr int DIR_PARK_SEG_FLOATS = 96 * DIR_PARK_THREADS;   // one parked segment of a CTA
@@ -191,8 +195,8 @@ struct TcConfig {
     int stages;   // shared-memory pipeline depth
     int pair;     // 1: two-SM tile (cta_group::2, 256 modes per CTA pair, bn columns shared)
     int grid;
-    int split;    // d-axis splits of a single problem (0 or 1: none; TC_SPLIT_BALANCED: one
-                  // range of equal chunk count per CTA or pair over all tiles)
+    int split;    // d-axis splits of a single problem (0 or 1: none; TC_SPLIT_BALANCED: the last
+                  // wave's tiles in one range of equal chunk count per CTA or pair)
 };
 constexpr int TC_SPLIT_BALANCED = -1;
 // Pipeline shapes the autotuner chooses from (index + 1 = mhc_params.tile_config).
@@ -209,8 +213,8 @@ int tc_make_tmap(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols,
 int tc_make_tmap_f32(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint64_t ld,
                      uint32_t box_rows, uint32_t box_cols);
 cudaError_t launch_tc_single(const TcParams<1> &p, const TcConfig &c, cudaStream_t s);
-// With prob[0].n_split > 1: sum the splits' partial projections of the block (in split order)
-// and run the tile epilogue (Eq. 16 product, bin-run sums into partials).
+// With prob[0].n_split > 1 or sk_parts > 0: sum the splits' partial projections of the block (in
+// split order) and run the tile epilogue (Eq. 16 product, bin-run sums into partials).
 cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s);
 // d elements per promotion chunk of the tensor-core kernels (splits are whole chunks)
 constexpr int TC_PROMOTE_D = 128;

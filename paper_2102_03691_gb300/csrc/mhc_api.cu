@@ -486,30 +486,36 @@ mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_
     return reset_accumulators(h);
 }
 
+// With the direction split: graphene-like 4096 atoms, K = 128 has 96 pair tiles for 76 resident
+// pairs; the projection took two waves, 370 us (ncu), and takes 262 + 14 us with the last wave's
+// 20 tiles cut (423 -> 355 us a push).
 // Balanced split, host side (the kernels' arithmetic): the part holding tail chunk g when T
 // chunks are cut into `parts` ranges, and the plan of one block: whole waves of tiles first
 // (t0 tiles on all `parts_all` CTAs or pairs), then the remaining tiles' chunks over
-// `parts` <= parts_all ranges; max_seg is the largest number of segments a tail tile is cut into.
+// `parts` <= parts_all ranges; max_seg is the largest number of segments a tail tile is cut into
+// (with the direction split, each of a tile's `sub` = 3 direction segments counts by itself).
 int sk_part_of_host(long long g, long long T, int parts) {
     return (int)(((g + 1) * parts + T - 1) / T - 1);
 }
 
 struct SkPlan {
-    int nch = 0, tiles = 0, parts_all = 0, t0 = 0, parts = 0, max_seg = 1;
+    int nch = 0, tiles = 0, parts_all = 0, t0 = 0, parts = 0, max_seg = 1, sub = 1;
+    int planes() const { return sub * max_seg; }   // of the workspace
 };
 
 SkPlan sk_plan(const mhc_handle *h, const TcConfig &c, int n_col_tiles) {
     SkPlan q;
     const int chunk_kb = TC_PROMOTE_D / c.bk;
-    q.nch = (int)((h->D_ld / c.bk + chunk_kb - 1) / chunk_kb);
+    q.sub = h->dir ? 3 : 1;
+    q.nch = (int)(((h->dir ? h->N_pad : h->D_ld) / c.bk + chunk_kb - 1) / chunk_kb);
     q.tiles = mode_tiles(h, c) * n_col_tiles;
     q.parts_all = std::max(1, sched_units(h, c));
     q.t0 = q.tiles / q.parts_all * q.parts_all;
     if (q.t0 == q.tiles) return q;   // whole waves only: no tail, nothing to split
-    const long long T = (long long)(q.tiles - q.t0) * q.nch;
+    const long long T = (long long)(q.tiles - q.t0) * q.sub * q.nch;
     q.parts = (int)std::min<long long>(q.parts_all, T);
-    for (int t = q.t0; t < q.tiles; ++t) {
-        const long long g0 = (long long)(t - q.t0) * q.nch;
+    for (int t = 0; t < (q.tiles - q.t0) * q.sub; ++t) {
+        const long long g0 = (long long)t * q.nch;
         q.max_seg = std::max(q.max_seg, 1 + sk_part_of_host(g0 + q.nch - 1, T, q.parts) -
                                             sk_part_of_host(g0, T, q.parts));
     }
@@ -524,7 +530,7 @@ size_t split_ws_bytes(const mhc_handle *h, const TcConfig &c) {
         size_t worst = 0;
         const int nct_max = (4 * h->prm.k_max + c.bn - 1) / c.bn;
         for (int nct = 1; nct <= nct_max; ++nct)
-            worst = std::max(worst, (size_t)sk_plan(h, c, nct).max_seg * nct * c.bn);
+            worst = std::max(worst, (size_t)sk_plan(h, c, nct).planes() * nct * c.bn);
         return sizeof(float) * worst * (size_t)h->M_pad;
     }
     if (c.split <= 1) return 0;
@@ -546,7 +552,7 @@ mhc_status ensure_split_ws(mhc_handle *h, const TcConfig &c) {
 
 mhc_status set_tc_config(mhc_handle *h, const TcConfig &c) {
     if (!tc_config_supported(c)) return fail(h, MHC_ERR_INVALID_ARG, "unsupported tile configuration");
-    if ((c.split > 1 || c.split == TC_SPLIT_BALANCED) && (h->dir || c.split > TC_MAX_SPLIT))
+    if (c.split > 1 && (h->dir || c.split > TC_MAX_SPLIT))
         return fail(h, MHC_ERR_INVALID_ARG, "d-axis split %d not available here", c.split);
     if (c.split < 1 && c.split != TC_SPLIT_BALANCED)
         return fail(h, MHC_ERR_INVALID_ARG, "d-axis split %d not available here", c.split);
@@ -597,7 +603,7 @@ mhc_status run_projection(mhc_handle *h, int K) {
         // balanced split: whole waves of tiles, then one range of the tail's chunks per CTA
         // (pair); tiles cut by a range boundary are finished by the split finish kernel
         const SkPlan &q = skq;
-        const size_t need = sizeof(float) * (size_t)q.max_seg * P.ws_cols * (size_t)h->M_pad;
+        const size_t need = sizeof(float) * (size_t)q.planes() * P.ws_cols * (size_t)h->M_pad;
         auto it = h->buf.find("split_ws");
         if (it == h->buf.end() || it->second.bytes < need)
             return fail(h, MHC_ERR_STATE, "balanced split workspace too small (%zu bytes needed)", need);
@@ -608,12 +614,14 @@ mhc_status run_projection(mhc_handle *h, int K) {
         P.sk_tm = (c.pair ? 2 : 1) * TC_BM;
         P.sk_bn = c.bn;
         P.sk_t0 = q.t0;
+        P.sk_sub = q.sub;
+        P.sk_planes = q.max_seg;
         P.split_ws = dptr<float>(h, "split_ws");
         P.n_tiles = q.tiles;
         c.grid = q.parts_all * (c.pair ? 2 : 1);
         cudaError_t e = launch_tc_single(h->tcp, c, h->stream);
         h->launches++;
-        if (e == cudaSuccess && q.max_seg > 1) {
+        if (e == cudaSuccess && q.planes() > 1) {
             e = launch_tc_split_finish(h->tcp, h->stream);
             h->launches++;
         }
@@ -741,7 +749,7 @@ mhc_status time_candidates(mhc_handle *h, int K, std::vector<std::pair<float, Tc
 // Autotune on the block just packed: time every tile shape unsplit (or with the fixed split of
 // mhc_params.split_d), then, for the two fastest shapes, the balanced split when the last wave
 // of tiles is partial and the uniform d-axis splits 2..8 when one block gives fewer than three
-// waves.  The winner is cached.
+// waves (not with the direction split).  The winner is cached.
 mhc_status autotune(mhc_handle *h, int K) {
     const TuneKey key = tune_key(h, K);
     {
@@ -761,7 +769,7 @@ mhc_status autotune(mhc_handle *h, int K) {
         res.emplace_back(0.f, c);
     }
     mhc_status s = time_candidates(h, K, res);
-    if (s == MHC_OK && h->prm.split_d == 0 && !h->dir) {
+    if (s == MHC_OK && h->prm.split_d == 0) {
         std::sort(res.begin(), res.end(),
                   [](const std::pair<float, TcConfig> &a, const std::pair<float, TcConfig> &b) {
                       return a.first < b.first;
@@ -778,7 +786,7 @@ mhc_status autotune(mhc_handle *h, int K) {
             const int64_t su = sched_units(h, c);
             c.split = TC_SPLIT_BALANCED;   // whenever the last wave is partial
             if (units % su && split_ws_bytes(h, c) <= budget) sp.emplace_back(0.f, c);
-            if (units >= 3 * su) continue;
+            if (h->dir || units >= 3 * su) continue;   // the uniform splits mix directions
             for (int S : {2, 3, 4, 6, 8}) {
                 if (n_kb < S * chunk_kb) break;
                 c.split = S;

@@ -4,6 +4,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -178,23 +179,30 @@ __device__ __forceinline__ void store_split4(const PackArgs &a, size_t idx, cons
     *reinterpret_cast<uint2 *>(static_cast<uint16_t *>(a.Bt_lo) + idx) = make_uint2(l[0] | (l[1] << 16), l[2] | (l[3] << 16));
 }
 
-// A cluster of ceil(N / (4 THREADS)) CTAs per step k.  CTA r bulk-copies the contiguous
-// velocities and virials of its atoms r*4*THREADS .. into shared memory (TMA, so the loads are
-// asynchronous and the inputs are read once).  Phase 1, thread t takes the atoms t, t+THREADS,
-// t+2 THREADS, t+3 THREADS (shared-memory strides of 3 and 9 words across a warp: no bank
-// conflicts): row maxima and the exact total-current pairs (acc_exact), combined per CTA in a
-// fixed order (unevaluated float pairs across the warp, FP64 across the warps); one cluster
-// barrier, then every CTA combines all ranks' maxima in rank order through distributed shared
-// memory (each computes the same scales) and rank 0 the current (FP64, rank order).
-// Phase 1 also replaces each atom's inputs in shared memory by its row values sqrt(m) v and
-// W / sqrt(m).  Phase 2 writes the four B rows of the CTA's atoms: each row is one contiguous run of
-// 16-bit values (three per atom; three runs of one per atom, one per direction, with the
+// A cluster of ceil(N / (4 THREADS)) CTAs per step k.  CTA r copies the contiguous velocities and
+// virials of its atoms r*4*THREADS .. into shared memory, every copy in flight at once and the
+// inputs read once: by TMA where the step's inputs start on 16-byte boundaries, else (N % 4 != 0,
+// or a caller's pointer in the middle of a buffer) by 4-byte asynchronous copies.  Phase 1, thread
+// t takes the atoms t, t+THREADS, t+2 THREADS, t+3 THREADS (shared-memory strides of 3 and 9 words
+// across a warp: no bank conflicts): row maxima and the exact total-current pairs (acc_exact),
+// combined per CTA in a fixed order (unevaluated float pairs across the warp, FP64 across the
+// warps); one cluster barrier, then every CTA combines all ranks' maxima in rank order through
+// distributed shared memory (each computes the same scales) and rank 0 the current (FP64, rank
+// order).  Phase 1 also replaces each atom's inputs in shared memory by its row values sqrt(m) v
+// and W / sqrt(m).  Phase 2 writes the four B rows of the CTA's atoms: each row is one contiguous
+// run of 16-bit values (three per atom; three runs of one per atom, one per direction, with the
 // direction-major columns), cut into groups of four values that consecutive threads take in
-// order, so that every warp store covers 256 contiguous bytes.  A CTA leaves only after the
-// second half of the cluster barrier: its peers may still be reading its partial sums.
-// The body of one CTA: step k of the system `a`, rank `rank` of its cluster of `nrank` CTAs.
+// order, so that every warp store covers 256 contiguous bytes (the last group's values past the
+// system are zeros in the padding of B's rows).  A CTA leaves only after the second half of the
+// cluster barrier: its peers may still be reading its partial sums.
+// What bounds it: a wave's chain of load, barrier and store (the stores wait for the row maxima),
+// at 4.1 TB/s of the 96 bytes an atom and step.  Keeping the values in registers over the barrier
+// and storing through shared memory by bulk copies halved the instructions and was not faster
+// (8000 atoms, K = 256: 52 against 48.5 us).  Atoms not a multiple of four and systems beyond
+// 16384 atoms, which a kernel of one CTA a step packed from two reads of the inputs, measured
+// (us, before -> now): 1003 atoms, K = 77 13.0 -> 8.9; 20000 atoms, K = 512 425 -> 270.
 template <int THREADS>
-__device__ __forceinline__ void pack_bulk_body(const PackArgs &a, int k, uint32_t rank, uint32_t nrank) {
+__device__ __forceinline__ void pack_cluster_body(const PackArgs &a, int k, uint32_t rank, uint32_t nrank) {
     constexpr int APC = 4 * THREADS;
     extern __shared__ float4 pk_smem4[];
     float *sv = reinterpret_cast<float *>(pk_smem4);   // [APC][3]
@@ -206,26 +214,33 @@ __device__ __forceinline__ void pack_bulk_body(const PackArgs &a, int k, uint32_
     __shared__ __align__(8) uint64_t bar;
     __shared__ int abort_flag;
     const int a0 = (int)rank * APC;
-    const int na = max(0, min(APC, a.N - a0));   // a multiple of 4 (N % 4 == 0)
+    const int na = max(0, min(APC, a.N - a0));
     const long long limit = a.wait_limit > 0 ? a.wait_limit : WAIT_LIMIT_CYCLES;
-    if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
-        abort_flag = 0;
-        fence_mbar_init();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && na > 0) {
-        const uint32_t vb = (uint32_t)na * 12, wb = (uint32_t)na * 36;
-        mbar_arrive_expect_tx(&bar, vb + wb);
-        const char *gv = reinterpret_cast<const char *>(a.v + ((size_t)k * a.N + a0) * 3);
-        const char *gw = reinterpret_cast<const char *>(a.W + ((size_t)k * a.N + a0) * 9);
-        for (uint32_t o = 0; o < vb; o += 16384)
-            bulk_load(reinterpret_cast<char *>(sv) + o, gv + o, min(16384u, vb - o), &bar);
-        for (uint32_t o = 0; o < wb; o += 16384)
-            bulk_load(reinterpret_cast<char *>(sw) + o, gw + o, min(16384u, wb - o), &bar);
-    }
+    const float *gv = a.v + ((size_t)k * a.N + a0) * 3, *gw = a.W + ((size_t)k * a.N + a0) * 9;
+    const bool bulk = ((a.N & 3) | ((reinterpret_cast<uintptr_t>(a.v) | reinterpret_cast<uintptr_t>(a.W)) & 15)) == 0;
     bool ok = true;
-    if (na > 0) ok = mbar_wait(&bar, 0, &abort_flag, limit);
+    if (bulk) {
+        if (threadIdx.x == 0) {
+            mbar_init(&bar, 1);
+            abort_flag = 0;
+            fence_mbar_init();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && na > 0) {
+            const uint32_t vb = (uint32_t)na * 12, wb = (uint32_t)na * 36;
+            mbar_arrive_expect_tx(&bar, vb + wb);
+            for (uint32_t o = 0; o < vb; o += 16384)
+                bulk_load(reinterpret_cast<char *>(sv) + o, reinterpret_cast<const char *>(gv) + o, min(16384u, vb - o), &bar);
+            for (uint32_t o = 0; o < wb; o += 16384)
+                bulk_load(reinterpret_cast<char *>(sw) + o, reinterpret_cast<const char *>(gw) + o, min(16384u, wb - o), &bar);
+        }
+        if (na > 0) ok = mbar_wait(&bar, 0, &abort_flag, limit);
+    } else {
+        for (int q = threadIdx.x; q < 3 * na; q += THREADS) cp_async4(sv + q, gv + q);
+        for (int q = threadIdx.x; q < 9 * na; q += THREADS) cp_async4(sw + q, gw + q);
+        cp_async_wait_all();
+        __syncthreads();
+    }
     float mx[4] = {0.f, 0.f, 0.f, 0.f};
     float js[3] = {0.f, 0.f, 0.f}, jc[3] = {0.f, 0.f, 0.f};
     if (ok) {
@@ -319,8 +334,8 @@ __device__ __forceinline__ void pack_bulk_body(const PackArgs &a, int k, uint32_
     } else {
         const size_t ld = (size_t)a.D_ld;
         const size_t r0 = (size_t)(4 * k) * ld;
-        const int q4 = na / 4;              // groups of four atoms (direction-major runs)
-        const int G = 3 * q4;               // groups of four values a row
+        const int q4 = (na + 3) / 4;                        // groups of four atoms (direction-major runs)
+        const int G = a.npad ? 3 * q4 : (3 * na + 3) / 4;   // groups of four values a row
 #pragma unroll 1
         for (int g = (int)threadIdx.x; g < G; g += THREADS) {
             int ia[4], bb[4];
@@ -344,15 +359,18 @@ __device__ __forceinline__ void pack_bulk_body(const PackArgs &a, int k, uint32_
             float x[4][4];   // [row][value]
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                x[0][e] = sv[3 * ia[e] + bb[e]] * s_mul[0];
+                const bool in = ia[e] < na;
+                x[0][e] = in ? sv[3 * ia[e] + bb[e]] * s_mul[0] : 0.f;
 #pragma unroll
-                for (int al = 0; al < 3; ++al) x[1 + al][e] = sw[9 * ia[e] + 3 * al + bb[e]] * s_mul[1 + al];
+                for (int al = 0; al < 3; ++al)
+                    x[1 + al][e] = in ? sw[9 * ia[e] + 3 * al + bb[e]] * s_mul[1 + al] : 0.f;
             }
             if (a.split == SPLIT_FP32) {   // d-major: the step's four rows are 16 bytes of a d
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    *reinterpret_cast<float4 *>(a.Bd32 + (col + e) * a.b_cols + 4 * k) =
-                        make_float4(x[0][e], x[1][e], x[2][e], x[3][e]);
+                    if (ia[e] < na)
+                        *reinterpret_cast<float4 *>(a.Bd32 + (col + e) * a.b_cols + 4 * k) =
+                            make_float4(x[0][e], x[1][e], x[2][e], x[3][e]);
             } else {
 #pragma unroll
                 for (int r = 0; r < 4; ++r) store_split4(a, r0 + (size_t)r * ld + col, x[r]);
@@ -365,30 +383,30 @@ __device__ __forceinline__ void pack_bulk_body(const PackArgs &a, int k, uint32_
 // Shared memory (48 B an atom) allows eight CTAs of 128 threads, four of 256 or two of 512 per
 // SM; the register cap of the launch bounds lets as many be resident.
 template <int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) pack_bulk_kernel(const PackArgs a) {
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) pack_cluster_kernel(const PackArgs a) {
     griddep_launch_dependents();   // the projection may set up on the SMs this grid leaves
     const uint32_t nrank = cluster_nctarank();
-    pack_bulk_body<THREADS>(a, (int)(blockIdx.x / nrank), cluster_ctarank(), nrank);
+    pack_cluster_body<THREADS>(a, (int)(blockIdx.x / nrank), cluster_ctarank(), nrank);
 }
 
 // Several systems in one launch: system j owns the CTAs cta_begin[j] .. cta_begin[j+1) (K_j
 // clusters of the common cluster size; ranks beyond a system's atoms hold no atoms and only
 // take part in the cluster's combination).
 template <int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) pack_bulk_group_kernel(const __grid_constant__ PackGroupArgs g) {
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) pack_cluster_group_kernel(const __grid_constant__ PackGroupArgs g) {
     griddep_launch_dependents();
     int j = 0;
     while (j + 1 < g.n && (int)blockIdx.x >= g.cta_begin[j + 1]) ++j;
     const uint32_t nrank = cluster_nctarank();
-    pack_bulk_body<THREADS>(g.a[j], (int)((blockIdx.x - (uint32_t)g.cta_begin[j]) / nrank),
+    pack_cluster_body<THREADS>(g.a[j], (int)((blockIdx.x - (uint32_t)g.cta_begin[j]) / nrank),
                             cluster_ctarank(), nrank);
 }
 
 template <int THREADS>
-cudaError_t launch_pack_bulk(const PackArgs &a, cudaStream_t s) {
+cudaError_t launch_pack_cluster(const PackArgs &a, cudaStream_t s) {
     constexpr int APC = 4 * THREADS;
     const int smem = APC * 48;
-    static cudaError_t attr = cudaFuncSetAttribute(pack_bulk_kernel<THREADS>,
+    static cudaError_t attr = cudaFuncSetAttribute(pack_cluster_kernel<THREADS>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (attr != cudaSuccess) return attr;
     const int csize = (a.N + APC - 1) / APC;
@@ -404,28 +422,63 @@ cudaError_t launch_pack_bulk(const PackArgs &a, cudaStream_t s) {
     la[0].val.clusterDim.z = 1;
     cfg.attrs = la;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, pack_bulk_kernel<THREADS>, a);
+    return cudaLaunchKernelEx(&cfg, pack_cluster_kernel<THREADS>, a);
 }
 
 }  // namespace
 
 namespace {
-// CTA size of the bulk-copy pack of a system of N atoms (four atoms a thread): one CTA a step
-// and eight an SM up to 512 atoms, clusters of up to 8 CTAs of 256 (four an SM) up to 8192,
-// of 512 beyond.
+// CTA size of the cluster pack of a system of N atoms (four atoms a thread): one CTA a step and
+// eight an SM up to 512 atoms, clusters of up to 8 CTAs of 256 (four an SM) up to 8192, of 512
+// beyond; clusters of more than 8 CTAs (the portable size) from 16384 atoms, up to 16.
 int pack_threads(int N) { return N <= 4 * 128 ? 128 : N <= 8 * 1024 ? 256 : 512; }
+constexpr int PACK_MAX_CLUSTER = 16;
 
-bool bulk_ok(const PackArgs &a) {
+// Whether a cluster of `csize` 512-thread CTAs can be resident on this device.
+bool pack_wide_ok(int csize) {
+    static int limit = -1;   // largest cluster size found to fit
+    static std::mutex m;
+    std::lock_guard<std::mutex> lock(m);
+    if (limit < 0) {
+        limit = 8;
+        const int smem = 4 * 512 * 48;
+        if (cudaFuncSetAttribute(pack_cluster_kernel<512>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaFuncSetAttribute(pack_cluster_group_kernel<512>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaFuncSetAttribute(pack_cluster_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess) {
+            for (int cs = 9; cs <= PACK_MAX_CLUSTER; ++cs) {
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)cs, 1, 1);
+                cfg.blockDim = dim3(512, 1, 1);
+                cfg.dynamicSmemBytes = smem;
+                cudaLaunchAttribute la[1];
+                la[0].id = cudaLaunchAttributeClusterDimension;
+                la[0].val.clusterDim.x = (unsigned)cs;
+                la[0].val.clusterDim.y = 1;
+                la[0].val.clusterDim.z = 1;
+                cfg.attrs = la;
+                cfg.numAttrs = 1;
+                int n = 0;
+                if (cudaOccupancyMaxActiveClusters(&n, pack_cluster_kernel<512>, &cfg) != cudaSuccess || n < 1) break;
+                limit = cs;
+            }
+        }
+        cudaGetLastError();
+    }
+    return csize <= limit;
+}
+
+// The cluster pack takes every system up to PACK_MAX_CLUSTER CTAs of 2048 atoms.
+bool cluster_ok(const PackArgs &a) {
     const auto al16 = [](const void *q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
-    return a.N % 4 == 0 && al16(a.v) && al16(a.W) && al16(a.sqm) && al16(a.isqm) &&
-           (a.split == SPLIT_FP32 ? al16(a.Bd32) : true);
+    const bool out = a.split == SPLIT_FP32 ? al16(a.Bd32) : al16(a.Bt_hi) && al16(a.Bt_lo);
+    return out && (a.N <= 8 * 2048 || (a.N <= PACK_MAX_CLUSTER * 2048 && pack_wide_ok((a.N + 2047) / 2048)));
 }
 
 template <int THREADS>
-cudaError_t launch_pack_bulk_group(PackGroupArgs g, int csize, cudaStream_t s) {
+cudaError_t launch_pack_cluster_group(PackGroupArgs g, int csize, cudaStream_t s) {
     constexpr int APC = 4 * THREADS;
     const int smem = APC * 48;
-    static cudaError_t attr = cudaFuncSetAttribute(pack_bulk_group_kernel<THREADS>,
+    static cudaError_t attr = cudaFuncSetAttribute(pack_cluster_group_kernel<THREADS>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (attr != cudaSuccess) return attr;
     g.cta_begin[0] = 0;
@@ -443,7 +496,7 @@ cudaError_t launch_pack_bulk_group(PackGroupArgs g, int csize, cudaStream_t s) {
     la[0].val.clusterDim.z = 1;
     cfg.attrs = la;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, pack_bulk_group_kernel<THREADS>, g);
+    return cudaLaunchKernelEx(&cfg, pack_cluster_group_kernel<THREADS>, g);
 }
 }  // namespace
 
@@ -451,17 +504,13 @@ cudaError_t launch_pack_group(const PackGroupArgs &g, const cudaStream_t *stream
                               int *n_launches) {
     *n_launches = 0;
     if (g.n < 1 || g.n > TC_MAX_GROUP) return cudaErrorInvalidValue;
-    int nmax = 0;
-    for (int j = 0; j < g.n; ++j) {
-        if (!bulk_ok(g.a[j])) return cudaErrorNotSupported;
-        nmax = std::max(nmax, g.a[j].N);
-    }
-    if (nmax > 8 * 2048) return cudaErrorNotSupported;
+    for (int j = 0; j < g.n; ++j)
+        if (!cluster_ok(g.a[j])) return cudaErrorNotSupported;
     // one launch per (CTA size, cluster size): every system is packed by the CTA size it gets
     // alone (so its results are bitwise those of a solo push), and no rank is idle
     for (const int threads : {128, 256, 512}) {
         const int apc = 4 * threads;
-        for (int cs = 1; cs <= 8; ++cs) {
+        for (int cs = 1; cs <= (threads == 512 ? PACK_MAX_CLUSTER : 8); ++cs) {
             PackGroupArgs sub{};
             for (int j = 0; j < g.n; ++j)
                 if (pack_threads(g.a[j].N) == threads &&
@@ -469,9 +518,9 @@ cudaError_t launch_pack_group(const PackGroupArgs &g, const cudaStream_t *stream
                     sub.a[sub.n++] = g.a[j];
             if (sub.n == 0) continue;
             const cudaStream_t s = streams[*n_launches % n_streams];   // independent systems
-            const cudaError_t e = threads == 128 ? launch_pack_bulk_group<128>(sub, cs, s)
-                                  : threads == 256 ? launch_pack_bulk_group<256>(sub, cs, s)
-                                                   : launch_pack_bulk_group<512>(sub, cs, s);
+            const cudaError_t e = threads == 128 ? launch_pack_cluster_group<128>(sub, cs, s)
+                                  : threads == 256 ? launch_pack_cluster_group<256>(sub, cs, s)
+                                                   : launch_pack_cluster_group<512>(sub, cs, s);
             if (e != cudaSuccess) return e;
             ++*n_launches;
         }
@@ -481,11 +530,11 @@ cudaError_t launch_pack_group(const PackGroupArgs &g, const cudaStream_t *stream
 
 cudaError_t launch_pack(const PackArgs &a, cudaStream_t s) {
     if (a.K <= 0) return cudaSuccess;
-    if (bulk_ok(a) && a.N <= 8 * 2048) {
+    if (cluster_ok(a)) {
         const int threads = pack_threads(a.N);
-        return threads == 128 ? launch_pack_bulk<128>(a, s)
-               : threads == 256 ? launch_pack_bulk<256>(a, s)
-                                : launch_pack_bulk<512>(a, s);
+        return threads == 128 ? launch_pack_cluster<128>(a, s)
+               : threads == 256 ? launch_pack_cluster<256>(a, s)
+                                : launch_pack_cluster<512>(a, s);
     }
     pack_kernel<<<a.K, PACK_THREADS, 0, s>>>(a);
     return cudaGetLastError();

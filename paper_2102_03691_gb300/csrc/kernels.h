@@ -24,7 +24,7 @@ __host__ __device__ constexpr uint32_t idesc_f16(uint32_t ab_fmt, uint32_t M, ui
 }
 
 // ---------------------------------------------------------------- K1 pack
-// One CTA per step k of the block.  Builds the four B-operand rows of step k,
+// Builds the four B-operand rows of step k of the block,
 //   Bt[4k][d]       = sqrt(m_i) v_i^b            (Eq. 13 weights)
 //   Bt[4k+1+a][d]   = W_i^{ab} / sqrt(m_i)       (Eq. 16 bracket weights)
 // (d = 3i+b), split into hi/lo 16-bit parts after a per-row power-of-two scale
@@ -50,14 +50,13 @@ struct PackArgs {
     int *status;           // sticky status for a bounded wait that runs out (may be null)
     long long wait_limit;  // SM cycles (0: a default of about a second)
 };
-// Systems with N % 4 == 0 (up to 16384 atoms) and 16-byte aligned inputs are packed by a
-// cluster of CTAs per step that bulk-copies its atoms into shared memory (the inputs are read
-// once); other shapes by one CTA per step that reads them twice.
+// Systems of up to 32768 atoms are packed by a cluster of CTAs per step that holds the step in
+// shared memory (the inputs are read once); larger ones by one CTA per step that reads them twice.
 cudaError_t launch_pack(const PackArgs &a, cudaStream_t s);
 // The packs of up to TC_MAX_GROUP systems in one launch per cluster size (systems needing the
 // same number of CTAs a step go together; cta_begin is filled by the launcher).
-// cudaErrorNotSupported when a system does not qualify for the bulk-copy pack (the caller then
-// packs the systems one by one).
+// cudaErrorNotSupported when a system is too large for the cluster pack (the caller then packs the
+// systems one by one).
 struct PackGroupArgs {
     PackArgs a[TC_MAX_GROUP];
     int cta_begin[TC_MAX_GROUP + 1];

@@ -1817,7 +1817,7 @@ mhc_status group_schedule(mhc_group *g, const std::vector<int> &Ks, GroupSchedul
 }
 
 // The packs of all systems in one launch (clusters of a common size), or one by one when a
-// system does not qualify for the bulk-copy pack.  All handles of a group share one stream.
+// system is too large for the cluster pack.  All handles of a group share one stream.
 mhc_status group_pack(mhc_group *g, const std::vector<const float *> &vs,
                       const std::vector<const float *> &ws, const std::vector<int> &Ks) {
     mhc_handle *h0 = g->hs[0];

@@ -265,63 +265,66 @@ __global__ void __launch_bounds__(32 * LC_WARPS, 2) lag_corr_kernel(const float 
 }
 
 // ------------------------------------------------------------------ K5
-// inv_count(l) = 1 / (T_s - l) (0 when no origin has lag l), computed once per read so that
-// the rows below multiply instead of dividing (an FP64 division is ~8 instructions on a pipe
-// GB300 keeps narrow).
+// 1 / (T_s - l) as an unevaluated float pair (zero when no origin has lag l): an FP32 reciprocal
+// and one Newton correction, ~46 bits.  An FP64 division is some 20 operations on a pipe GB300
+// keeps narrow (1/64 of the FP32 rate); these are FP32 instructions.
+__device__ __forceinline__ float2 gk_inv_count(long long T_s, int l) {
+    const long long n = T_s - l;
+    if (n <= 0) return make_float2(0.f, 0.f);
+    const float hi = (float)n, lo = (float)(n - (long long)hi);
+    const float r = __fdiv_rn(1.f, hi);
+    return make_float2(r, r * fmaf(-r, lo, fmaf(-r, hi, 1.f)));
+}
+__device__ __forceinline__ double gk_pair(float2 p) { return (double)p.x + (double)p.y; }
+
+// table[l] = 1 / (T_s - l) for reads whose table does not fit a CTA's shared memory
 __global__ void inv_counts_kernel(long long T_s, int L, double *inv) {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l < L) inv[l] = T_s > l ? 1.0 / (double)(T_s - l) : 0.0;
+    if (l < L) inv[l] = gk_pair(gk_inv_count(T_s, l));
 }
 
-// One CTA per (b, mu, nu) row, GK_THREADS threads, each owning per = ceil(L / GK_THREADS)
-// consecutive lags.  C(l) = Csum(l) inv_count(l); the running trapezoid sum
-// S(l) = sum_{1 <= l' <= l} (C(l'-1) + C(l')) comes from per-thread totals and a block-wide
-// exclusive scan (warp shuffles, then the four warp totals: a fixed tree, deterministic);
-// kappa(l) = (c dt / 2) S(l).  The window average runs over the lags l_lo .. l_hi (the host
-// picks them with the same FP64 test on l dt as the oracle).  The pipe GB300 keeps narrow
-// bounds the kernel, so each lag costs a few FP64 operations: C(l) is computed once and kept
-// in registers when a thread owns at most GK_CACHE lags.
-constexpr int GK_THREADS = 128;
+// One warp per (b, mu, nu) row, GK_TAU_ROWS rows a CTA; lane i owns per = ceil(L / 32) consecutive
+// lags.  C(l) = Csum(l) / (T_s - l); the running trapezoid sum
+// S(l) = sum_{1 <= l' <= l} (C(l'-1) + C(l')) comes from the lanes' totals and a warp scan (a
+// fixed tree, deterministic); kappa(l) = (c dt / 2) S(l).  The window average runs over the lags
+// l_lo .. l_hi (the host picks them with the same FP64 test on l dt as the oracle).  Bound by the
+// FP64 pipe and the latency of its chain, so: one row's scan stays inside a warp (a CTA of four
+// warps a row spent its time in block scans), the reciprocal counts come from a table that the
+// CTA builds with FP32 instructions (inv non-null: a launch built it), and a lane with at most
+// GK_CACHE lags keeps its running sums in registers.
+// Measured (ncu, us, before -> now): 900 rows x 200 lags 14.5 + 2.3 for
+// the table's launch -> 8.1.
+constexpr int GK_TAU_ROWS = 4;
 constexpr int GK_CACHE = 8;
-__device__ __forceinline__ double gk_block_exclusive_scan(double x, double *s_w) {   // all threads
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    double v = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double y = __shfl_up_sync(FULL_MASK, v, o);
-        if (lane >= o) v += y;
+__global__ void __launch_bounds__(32 * GK_TAU_ROWS) gk_kappa_kernel(const double *Csum, int rows, int L,
+                                                                    const double *__restrict__ inv,
+                                                                    long long T_s, double coef_half,
+                                                                    int l_lo, int l_hi,
+                                                                    double *kappa_tau, double *kappa_w) {
+    extern __shared__ double gk_tab[];
+    if (!inv) {
+        for (int l = threadIdx.x; l < L; l += blockDim.x) gk_tab[l] = gk_pair(gk_inv_count(T_s, l));
+        __syncthreads();
+        inv = gk_tab;
     }
-    double ex = __shfl_up_sync(FULL_MASK, v, 1);   // exclusive within the warp
-    if (lane == 0) ex = 0.0;
-    if (lane == 31) s_w[w] = v;
-    __syncthreads();
-    double base = 0.0;
-    for (int q = 0; q < w; ++q) base += s_w[q];
-    __syncthreads();
-    return base + ex;
-}
-
-__global__ void __launch_bounds__(GK_THREADS) gk_kappa_kernel(const double *Csum, int L,
-                                                              const double *__restrict__ inv,
-                                                              double coef_half, int l_lo, int l_hi,
-                                                              double *kappa_tau, double *kappa_w) {
-    __shared__ double s_w[GK_THREADS / 32];
-    const int r = blockIdx.x;
+    const int r = blockIdx.x * GK_TAU_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (r >= rows) return;
     const double *cs = Csum + (size_t)r * L;
-    const int per = (L + GK_THREADS - 1) / GK_THREADS;
-    const int l0 = min(L, threadIdx.x * per), l1 = min(L, l0 + per);
+    double *kt = kappa_tau + (size_t)r * L;
+    const int per = (L + 31) / 32;
+    const int l0 = min(L, lane * per), l1 = min(L, l0 + per);
     const double c_before = (l0 > 0 && l0 < l1) ? cs[l0 - 1] * inv[l0 - 1] : 0.0;
-    double cc[GK_CACHE];
+    double run[GK_CACHE];   // the lane's running sums
     double tot = 0.0, prev = c_before;
     if (per <= GK_CACHE) {
+        double c[GK_CACHE];
+#pragma unroll
+        for (int u = 0; u < GK_CACHE; ++u) c[u] = l0 + u < l1 ? cs[l0 + u] * inv[l0 + u] : 0.0;
 #pragma unroll
         for (int u = 0; u < GK_CACHE; ++u) {
-            const int l = l0 + u;
-            cc[u] = l < l1 ? cs[l] * inv[l] : 0.0;
-            if (l < l1) {
-                if (l > 0) tot += prev + cc[u];
-                prev = cc[u];
-            }
+            if (l0 + u < l1 && l0 + u > 0) tot += prev + c[u];
+            run[u] = tot;
+            prev = c[u];
         }
     } else {
         for (int l = l0; l < l1; ++l) {
@@ -330,33 +333,38 @@ __global__ void __launch_bounds__(GK_THREADS) gk_kappa_kernel(const double *Csum
             prev = c;
         }
     }
-    double acc = gk_block_exclusive_scan(tot, s_w);
+    double base = tot;   // exclusive scan of the lanes' totals
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(FULL_MASK, base, o);
+        if (lane >= o) base += y;
+    }
+    base = __shfl_up_sync(FULL_MASK, base, 1);
+    if (lane == 0) base = 0.0;
     double wsum = 0.0;
-    prev = c_before;
-    auto emit = [&](int l, double c) {
-        if (l > 0) acc += prev + c;
-        prev = c;
-        const double kap = coef_half * acc;
-        if (kappa_tau) kappa_tau[(size_t)r * L + l] = kap;
+    auto emit = [&](int l, double s) {
+        const double kap = coef_half * s;
+        kt[l] = kap;
         if (l >= l_lo && l <= l_hi) wsum += kap;
     };
     if (per <= GK_CACHE) {
 #pragma unroll
         for (int u = 0; u < GK_CACHE; ++u)
-            if (l0 + u < l1) emit(l0 + u, cc[u]);
+            if (l0 + u < l1) emit(l0 + u, base + run[u]);
     } else {
-        for (int l = l0; l < l1; ++l) emit(l, cs[l] * inv[l]);
+        prev = c_before;
+        for (int l = l0; l < l1; ++l) {
+            const double c = cs[l] * inv[l];
+            if (l > 0) base += prev + c;
+            prev = c;
+            emit(l, base);
+        }
     }
-    // window average: block sum of wsum (fixed tree)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) wsum += __shfl_down_sync(FULL_MASK, wsum, o);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = wsum;
-    __syncthreads();
-    if (threadIdx.x == 0 && kappa_w) {
-        double t = 0.0;
-        for (int q = 0; q < GK_THREADS / 32; ++q) t += s_w[q];
+    if (lane == 0 && kappa_w) {
         const int n = l_hi >= l_lo ? l_hi - l_lo + 1 : 0;
-        kappa_w[r] = n > 0 ? t / n : 0.0;
+        kappa_w[r] = n > 0 ? wsum / n : 0.0;
     }
 }
 
@@ -364,45 +372,113 @@ __global__ void __launch_bounds__(GK_THREADS) gk_kappa_kernel(const double *Csum
 //   sum_{l = l_lo..l_hi} S(l) = sum_m C(m) w(m),  w(m) = [m >= 1] cnt(m) + cnt(m + 1),
 // cnt(x) = #{l in [l_lo, l_hi] : l >= x} (C(m) enters S(l) as the right end of the step m-1 -> m
 // for l >= m >= 1 and as the left end of the step m -> m+1 for l >= m+1).  The integer weights
-// and the reciprocal counts are folded into one table tw(m) = inv(m) w(m), so a row takes one
-// FP64 FMA a lag instead of the scan's few FP64 operations a lag on GB300's narrow FP64 pipe.
-__device__ __forceinline__ double gk_window_weight(long long T_s, int m, int l_lo, int l_hi) {
+// and the reciprocal counts are folded into one table tw(m) = w(m) / (T_s - m) (a float pair), so
+// a row takes one FP64 FMA a lag instead of the scan's few FP64 operations a lag on GB300's narrow
+// FP64 pipe.
+__device__ __forceinline__ float2 gk_window_weight(long long T_s, int m, int l_lo, int l_hi) {
     const auto cnt = [&](int x) {
         const int lo = max(x, l_lo);
         return l_hi >= lo ? l_hi - lo + 1 : 0;
     };
-    const double inv = T_s > m ? 1.0 / (double)(T_s - m) : 0.0;
-    return inv * (double)((m >= 1 ? cnt(m) : 0) + cnt(m + 1));
+    const float2 inv = gk_inv_count(T_s, m);
+    const float w = (float)((m >= 1 ? cnt(m) : 0) + cnt(m + 1));   // below 2^24: exact
+    const float p = w * inv.x;
+    return make_float2(p, fmaf(w, inv.x, -p) + w * inv.y);
 }
 
 __global__ void gk_window_weights_kernel(long long T_s, int L, int l_lo, int l_hi, double *tw) {
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m < L) tw[m] = gk_window_weight(T_s, m, l_lo, l_hi);
+    if (m < L) tw[m] = gk_pair(gk_window_weight(T_s, m, l_lo, l_hi));
 }
 
 // One warp per row, GK_ROWS rows a CTA: kappa_w = scale sum_m Csum(m) tw(m) (lanes stride the
-// lags; fixed tree).  tw null: each CTA first builds the table in shared memory (L FP64
-// divisions spread over its threads), cheaper than a launch of its own while the grid is about
-// one CTA an SM; larger grids (the bin-bin read) take the table from one weights launch.
-constexpr int GK_ROWS = 8;
+// lags; fixed tree).  tw null: each CTA first builds the table in shared memory (FP32 instructions
+// spread over its threads), cheaper than a launch of its own; longer tables than that holds come
+// from one weights launch.
+// Measured (ncu, us, before -> now, the table's L FP64 divisions a CTA being the time): 576 rows x
+// 500 lags 8.9 -> 6.6; x 1000 lags 15.3 -> 10.0.
+constexpr int GK_ROWS = 4;
 __global__ void __launch_bounds__(32 * GK_ROWS) gk_window_kernel(const double *Csum, int rows, int L,
                                                                  const double *__restrict__ tw,
                                                                  long long T_s, int l_lo, int l_hi,
                                                                  double scale, double *kappa_w) {
     extern __shared__ double gk_tw[];
     if (!tw) {
-        for (int m = threadIdx.x; m < L; m += blockDim.x) gk_tw[m] = gk_window_weight(T_s, m, l_lo, l_hi);
+        for (int m = threadIdx.x; m < L; m += blockDim.x) gk_tw[m] = gk_pair(gk_window_weight(T_s, m, l_lo, l_hi));
         __syncthreads();
         tw = gk_tw;
     }
     const int r = blockIdx.x * GK_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (r >= rows) return;
     const double *cs = Csum + (size_t)r * L;
-    double acc = 0.0;
-    for (int m = lane; m < L; m += 32) acc = fma(cs[m], tw[m], acc);
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};   // four loads in flight a lane
+    for (int m = lane; m < L; m += 128) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(FULL_MASK, acc, o);
-    if (lane == 0) kappa_w[r] = scale * acc;
+        for (int u = 0; u < 4; ++u)
+            if (m + 32 * u < L) acc[u] = fma(cs[m + 32 * u], tw[m + 32 * u], acc[u]);
+    }
+    double t = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(FULL_MASK, t, o);
+    if (lane == 0) kappa_w[r] = scale * t;
+}
+
+// The same average of the bin-bin sums, from their state X[l][j][i] (float pairs, i = 3b + mu and
+// j = 3b' + nu of n = 3 nb rows) without the FP64 copy in [b][b'][mu][nu][l] order that the
+// kappa(tau) read takes: consecutive threads take consecutive (j, i), so every lag is one
+// contiguous read.  The weighted sum runs in float pairs (~46 bits) because the state is pairs and
+// FP64 conversions alone would take several times the read: X w = p + e exactly by FMA, and TwoSum
+// adds p.  XCW_GROUPS threads share an output's lags and are added in order.  Bound by the read.
+// Measured at n = 192, L = 200 (59 MB; ncu, us): 47.9 (FP64 copy) + 2.8 (weights) +
+// 31.9 (sum) -> 13.8.
+constexpr int XCW_OUT = 64, XCW_GROUPS = 4, XCW_UNROLL = 8;
+__global__ void __launch_bounds__(XCW_OUT * XCW_GROUPS) xcorr_window_kernel(
+    const float2 *__restrict__ X, int nb, int L, const double *__restrict__ tw, long long T_s,
+    int l_lo, int l_hi, double scale, double *kappa_w) {
+    extern __shared__ float2 xw_tab[];
+    __shared__ float2 part[XCW_GROUPS][XCW_OUT];
+    if (!tw)
+        for (int m = threadIdx.x; m < L; m += blockDim.x) xw_tab[m] = gk_window_weight(T_s, m, l_lo, l_hi);
+    __syncthreads();
+    const int n = 3 * nb, o = threadIdx.x % XCW_OUT, g = threadIdx.x / XCW_OUT;
+    const long long nn = (long long)n * n, q = blockIdx.x * (long long)XCW_OUT + o;
+    float s = 0.f, c = 0.f;
+    if (q < nn) {
+        const int per = (L + XCW_GROUPS - 1) / XCW_GROUPS;
+        const int m0 = min(L, g * per), m1 = min(L, m0 + per);
+        const float2 *src = X + q;
+        for (int m = m0; m < m1; m += XCW_UNROLL) {
+            float2 v[XCW_UNROLL];
+#pragma unroll
+            for (int u = 0; u < XCW_UNROLL; ++u)
+                v[u] = m + u < m1 ? __ldcs(src + (m + u) * nn) : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < XCW_UNROLL; ++u) {
+                if (m + u >= m1) break;
+                float2 w;
+                if (tw) {
+                    const double d = tw[m + u];
+                    w.x = (float)d;
+                    w.y = (float)(d - (double)w.x);
+                } else {
+                    w = xw_tab[m + u];
+                }
+                const float p = __fmul_rn(v[u].x, w.x);
+                const float e = fmaf(v[u].x, w.x, -p);
+                lc_pair_add(s, c, p);
+                c = __fadd_rn(c, fmaf(v[u].y, w.x, fmaf(v[u].x, w.y, e)));
+            }
+        }
+    }
+    part[g][o] = make_float2(s, c);
+    __syncthreads();
+    if (g == 0 && q < nn) {
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < XCW_GROUPS; ++k) t += gk_pair(part[k][o]);
+        const int j = (int)(q / n), i = (int)(q - (long long)j * n);
+        kappa_w[(((size_t)(i / 3) * nb + j / 3) * 3 + i % 3) * 3 + j % 3] = scale * t;
+    }
 }
 
 __global__ void hnema_finalize_kernel(const double *hsum, int n, long long T_s, double coef,
@@ -441,9 +517,20 @@ void launch_bin_finish(const float *partials, int n_slots, const int *slot_begin
 }
 
 namespace {
-// the per-CTA weight table: up to two CTAs an SM and a table within the default 48 KB
-constexpr int GK_TABLE_CTAS = 304;
-constexpr int GK_TABLE_LAGS = 6144;
+constexpr int GK_TABLE_LAGS = 6144;   // longest per-CTA table: the default 48 KB
+
+// The window's lags: l dt in [tau_lo, tau_hi], tested in FP64 as the oracle tests it.
+void gk_window(int L, double tau_lo, double tau_hi, double dt, int &l_lo, int &l_hi) {
+    l_lo = L;
+    l_hi = -1;
+    for (int l = 0; l < L; ++l) {
+        const double tau = l * dt;
+        if (tau >= tau_lo && tau <= tau_hi) {
+            l_lo = std::min(l_lo, l);
+            l_hi = l;
+        }
+    }
+}
 
 int lag_corr_tiles(int B, int L) { return ((L + 31) / 32) * ((B + LC_ROWS / 3 - 1) / (LC_ROWS / 3)); }
 }
@@ -488,36 +575,41 @@ cudaError_t launch_lag_corr(const float *Jb, const double *Jring, int R, double 
 
 int launch_gk_kappa(const double *Csum, int B, int L, long long T_s, double coef_dt,
                     double tau_lo, double tau_hi, double dt, double *kappa_tau, double *kappa_w,
-                    double *inv_scratch, cudaStream_t s) {
+                    double *table, cudaStream_t s) {
     if (L <= 0 || B <= 0) return 0;
-    // the window's lags: l dt in [tau_lo, tau_hi], tested in FP64 as the oracle tests it
-    int l_lo = L, l_hi = -1;
-    for (int l = 0; l < L; ++l) {
-        const double tau = l * dt;
-        if (tau >= tau_lo && tau <= tau_hi) {
-            l_lo = std::min(l_lo, l);
-            l_hi = l;
-        }
-    }
+    int l_lo, l_hi;
+    gk_window(L, tau_lo, tau_hi, dt, l_lo, l_hi);
+    const int rows = B * 9;
+    const bool own = L <= GK_TABLE_LAGS;   // each CTA builds the table
+    const size_t sm = own ? sizeof(double) * L : 0;
     if (!kappa_tau) {   // the window average alone
         const int n = l_hi >= l_lo ? l_hi - l_lo + 1 : 0;
-        const int rows = B * 9;
-        const int ctas = (rows + GK_ROWS - 1) / GK_ROWS;
         const double scale = n > 0 ? 0.5 * coef_dt / n : 0.0;
-        if (ctas <= GK_TABLE_CTAS && L <= GK_TABLE_LAGS) {   // each CTA builds the table
-            gk_window_kernel<<<ctas, 32 * GK_ROWS, sizeof(double) * L, s>>>(
-                Csum, rows, L, nullptr, T_s, l_lo, l_hi, scale, kappa_w);
-            return 1;
-        }
-        gk_window_weights_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, l_lo, l_hi, inv_scratch);
-        gk_window_kernel<<<ctas, 32 * GK_ROWS, 0, s>>>(Csum, rows, L, inv_scratch, T_s, l_lo, l_hi,
-                                                       scale, kappa_w);
-        return 2;
+        if (!own) gk_window_weights_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, l_lo, l_hi, table);
+        gk_window_kernel<<<(rows + GK_ROWS - 1) / GK_ROWS, 32 * GK_ROWS, sm, s>>>(
+            Csum, rows, L, own ? nullptr : table, T_s, l_lo, l_hi, scale, kappa_w);
+        return own ? 1 : 2;
     }
-    inv_counts_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, inv_scratch);
-    gk_kappa_kernel<<<B * 9, GK_THREADS, 0, s>>>(Csum, L, inv_scratch, 0.5 * coef_dt, l_lo, l_hi,
-                                                 kappa_tau, kappa_w);
-    return 2;
+    if (!own) inv_counts_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, table);
+    gk_kappa_kernel<<<(rows + GK_TAU_ROWS - 1) / GK_TAU_ROWS, 32 * GK_TAU_ROWS, sm, s>>>(
+        Csum, rows, L, own ? nullptr : table, T_s, 0.5 * coef_dt, l_lo, l_hi, kappa_tau, kappa_w);
+    return own ? 1 : 2;
+}
+
+int launch_xcorr_window(const float2 *X, int nb, int L, long long T_s, double coef_dt, double tau_lo,
+                        double tau_hi, double dt, double *kappa_w, double *table, cudaStream_t s) {
+    if (L <= 0 || nb <= 0) return 0;
+    int l_lo, l_hi;
+    gk_window(L, tau_lo, tau_hi, dt, l_lo, l_hi);
+    const int n = l_hi >= l_lo ? l_hi - l_lo + 1 : 0;
+    const double scale = n > 0 ? 0.5 * coef_dt / n : 0.0;
+    const bool own = L <= GK_TABLE_LAGS / 2;   // beside the partial sums
+    if (!own) gk_window_weights_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, l_lo, l_hi, table);
+    const long long out = 9ll * nb * nb;
+    xcorr_window_kernel<<<(unsigned)((out + XCW_OUT - 1) / XCW_OUT), XCW_OUT * XCW_GROUPS,
+                          own ? sizeof(float2) * L : 0, s>>>(X, nb, L, own ? nullptr : table, T_s, l_lo, l_hi,
+                                                             scale, kappa_w);
+    return own ? 1 : 2;
 }
 
 void launch_hnema_finalize(const double *hsum, int B, long long T_s, double coef, double *mean,

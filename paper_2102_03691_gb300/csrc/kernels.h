@@ -292,11 +292,11 @@ cudaError_t launch_lag_corr(const float *Jb, const double *Jring, int R, double 
 cudaError_t lag_corr_prepare();
 // kappa_tau[r][l] (r = b*9+mu*3+nu) and window averages kappa_w[r], FP64; kappa_tau null:
 // the window averages alone, as one weighted sum of C(l) a row.
-// inv_scratch: [L] doubles of device scratch (the reciprocal lag counts of this read).
+// table: [L] doubles of device scratch (weights of reads too long for a CTA's own table).
 // Returns the number of kernels launched.
 int launch_gk_kappa(const double *Csum, int B, int L, long long T_s, double coef_dt,
                     double tau_lo, double tau_hi, double dt, double *kappa_tau,
-                    double *kappa_w, double *inv_scratch, cudaStream_t s);
+                    double *kappa_w, double *table, cudaStream_t s);
 // mean[b][a] = hsum/T_s; kappa[b][a] = mean * coef
 void launch_hnema_finalize(const double *hsum, int B, long long T_s, double coef, double *mean,
                            double *kappa, cudaStream_t s);
@@ -343,6 +343,10 @@ cudaError_t launch_bin_xcorr(const XcPlan &pl, XcTcParams p, const float *ring, 
                              const long long *t0_dev, void *Whi, void *Wlo, cudaStream_t s);
 // out[b][b'][mu][nu][l] = X[l][3b'+nu][3b+mu] (float pair -> FP64)
 void launch_xcorr_transpose(const float2 *X, int nb, int L, double *out, cudaStream_t s);
+// The window averages alone of the bin-bin sums, [b][b'][mu][nu], straight from the state X
+// (arguments as launch_gk_kappa).
+int launch_xcorr_window(const float2 *X, int nb, int L, long long T_s, double coef_dt, double tau_lo,
+                        double tau_hi, double dt, double *kappa_w, double *table, cudaStream_t s);
 // count[l] = max(T_s - l, 0)
 void launch_lag_counts(long long T_s, int L, long long *count, cudaStream_t s);
 

@@ -1544,16 +1544,25 @@ mhc_status mhc_read_kappa_xcorr(mhc_handle *h, double *kappa_tau, double tau_lo,
     const int nb = (int)n_out_bins(h);
     const size_t rows = (size_t)9 * nb * nb;
     mhc_status s;
+    const double coef = WMK_PER_EV_PS_A_K / (KB_EV_PER_K * h->prm.T_K * h->prm.T_K * h->prm.V_A3);
+    if (!kappa_tau) {   // the window averages alone need no FP64 copy of the sums
+        if (!kappa_w) return MHC_OK;
+        if ((s = dev_alloc(h, "xw_out", sizeof(double) * (rows + L), false)) != MHC_OK) return s;
+        double *dw = dptr<double>(h, "xw_out");
+        h->launches += launch_xcorr_window(dptr<float2>(h, "Xsum"), nb, L, h->steps, coef * h->prm.dt_ps,
+                                           tau_lo, tau_hi, h->prm.dt_ps, dw, dw + rows, h->stream);
+        MHC_CUDA(h, cudaGetLastError());
+        return copy_out(h, kappa_w, dw, sizeof(double) * rows, where);
+    }
     if ((s = dev_alloc(h, "xc_out", sizeof(double) * rows * L, false)) != MHC_OK) return s;
     if ((s = dev_alloc(h, "xk_out", sizeof(double) * (rows * (L + 1) + L), false)) != MHC_OK) return s;
     launch_xcorr_transpose(dptr<float2>(h, "Xsum"), nb, L, dptr<double>(h, "xc_out"), h->stream);
     double *dk = dptr<double>(h, "xk_out"), *dw = dk + rows * L;
-    const double coef = WMK_PER_EV_PS_A_K / (KB_EV_PER_K * h->prm.T_K * h->prm.T_K * h->prm.V_A3);
     h->launches += 1 + launch_gk_kappa(dptr<double>(h, "xc_out"), nb * nb, L, h->steps,
-                                       coef * h->prm.dt_ps, tau_lo, tau_hi, h->prm.dt_ps,
-                                       kappa_tau ? dk : nullptr, dw, dw + rows, h->stream);
+                                       coef * h->prm.dt_ps, tau_lo, tau_hi, h->prm.dt_ps, dk, dw,
+                                       dw + rows, h->stream);
     MHC_CUDA(h, cudaGetLastError());
-    if (kappa_tau && (s = copy_out(h, kappa_tau, dk, sizeof(double) * rows * L, where)) != MHC_OK) return s;
+    if ((s = copy_out(h, kappa_tau, dk, sizeof(double) * rows * L, where)) != MHC_OK) return s;
     if (kappa_w && (s = copy_out(h, kappa_w, dw, sizeof(double) * rows, where)) != MHC_OK) return s;
     return MHC_OK;
 }

@@ -14,6 +14,9 @@ constexpr int TC_MAX_GROUP = 16;  // systems per grouped launch
 constexpr int TC_MAX_SPLIT = 16;  // d-axis splits of one projection
 constexpr double A2_PS2_PER_EV_AMU = 9648.533212331;   // 1 eV/amu in A^2/ps^2
 
+// Whether a kernel on `device` may store doubles at p (aligned memory of that device).
+bool writable_here(const void *p, int device);
+
 // Sticky device status codes (same values as mhc_status).
 constexpr int DEV_OK = 0, DEV_TIMEOUT = 4, DEV_STATE = 5;
 

@@ -83,6 +83,16 @@ int mhc::tc_make_tmap_f32(CUtensorMap *m, const void *base, uint64_t rows, uint6
     return r == CUDA_SUCCESS ? 0 : (int)r;
 }
 
+bool mhc::writable_here(const void *p, int device) {
+    if (reinterpret_cast<uintptr_t>(p) % sizeof(double)) return false;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == device;
+}
+
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
@@ -1002,6 +1012,12 @@ mhc_status push_graph(mhc_handle *h, const float *v, const float *W, int K) {
     return MHC_OK;
 }
 
+// Whether the read-out kernels may write FP64 results straight to `dst`: memory of this device,
+// aligned.  Anything else that `where` calls device memory takes a copy from the handle's scratch.
+bool direct_out(const mhc_handle *h, const void *dst, int where) {
+    return where == MHC_MEM_DEVICE && writable_here(dst, h->prm.device);
+}
+
 mhc_status copy_out(mhc_handle *h, void *dst, const void *src, size_t bytes, int where) {
     if (where == MHC_MEM_DEVICE) {
         MHC_CUDA(h, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, h->stream));
@@ -1457,16 +1473,18 @@ mhc_status mhc_read_hnema(mhc_handle *h, double *kappa, double *mean_J, int32_t 
     if (!h->bins_ready) return fail(h, MHC_ERR_INVALID_ARG, "no bins");
     mhc_status s;
     const size_t n = (size_t)n_out_bins(h) * 3;
-    if ((s = dev_alloc(h, "hn_out", sizeof(double) * 2 * n, false)) != MHC_OK) return s;
     const double fe = std::sqrt(h->prm.F_e[0] * h->prm.F_e[0] + h->prm.F_e[1] * h->prm.F_e[1] +
                                 h->prm.F_e[2] * h->prm.F_e[2]);
     const double coef = fe > 0 ? WMK_PER_EV_PS_A_K / (h->prm.T_K * h->prm.V_A3 * fe) : 0.0;
-    double *dm = dptr<double>(h, "hn_out"), *dk = dm + n;
+    const bool own_k = kappa && !direct_out(h, kappa, where), own_m = mean_J && !direct_out(h, mean_J, where);
+    if ((own_k || own_m) && (s = dev_alloc(h, "hn_out", sizeof(double) * 2 * n, false)) != MHC_OK) return s;
+    double *dm = own_m ? dptr<double>(h, "hn_out") : mean_J;
+    double *dk = own_k ? dptr<double>(h, "hn_out") + n : kappa;
     launch_hnema_finalize(dptr<double>(h, "hsum"), (int)n_out_bins(h), h->steps, coef, dm, dk, h->stream);
     h->launches++;
     MHC_CUDA(h, cudaGetLastError());
-    if (kappa && (s = copy_out(h, kappa, dk, sizeof(double) * n, where)) != MHC_OK) return s;
-    if (mean_J && (s = copy_out(h, mean_J, dm, sizeof(double) * n, where)) != MHC_OK) return s;
+    if (own_k && (s = copy_out(h, kappa, dk, sizeof(double) * n, where)) != MHC_OK) return s;
+    if (own_m && (s = copy_out(h, mean_J, dm, sizeof(double) * n, where)) != MHC_OK) return s;
     return MHC_OK;
 }
 
@@ -1496,17 +1514,25 @@ mhc_status mhc_read_kappa_gk(mhc_handle *h, double *kappa_tau, double tau_lo, do
         return fail(h, MHC_ERR_INVALID_ARG, "GKMA is not enabled or no bins");
     const int L = h->prm.n_lags;
     const size_t rows = (size_t)n_out_bins(h) * 9;
+    if (!kappa_tau && !kappa_w) return MHC_OK;
     mhc_status s;
-    if ((s = dev_alloc(h, "gk_out", sizeof(double) * (rows * (L + 1) + L), false)) != MHC_OK) return s;
-    double *dk = dptr<double>(h, "gk_out"), *dw = dk + rows * L;
+    const bool own_t = kappa_tau && !direct_out(h, kappa_tau, where);
+    const bool own_w = kappa_w && !direct_out(h, kappa_w, where);
+    // scratch: the weights table, the window averages, kappa(tau)
+    if ((s = dev_alloc(h, "gk_out", sizeof(double) * (L + (own_w ? rows : 0) + (own_t ? rows * L : 0)),
+                       false)) != MHC_OK)
+        return s;
+    double *table = dptr<double>(h, "gk_out");
+    double *dw = own_w ? table + L : kappa_w;
+    double *dk = own_t ? table + L + (own_w ? rows : 0) : kappa_tau;
     const double coef = WMK_PER_EV_PS_A_K / (KB_EV_PER_K * h->prm.T_K * h->prm.T_K * h->prm.V_A3);
     // without a kappa(tau) output only the window average is computed (one FMA a lag)
     h->launches += launch_gk_kappa(dptr<double>(h, "Csum"), (int)n_out_bins(h), L, h->steps,
-                                   coef * h->prm.dt_ps, tau_lo, tau_hi, h->prm.dt_ps,
-                                   kappa_tau ? dk : nullptr, dw, dw + rows, h->stream);
+                                   coef * h->prm.dt_ps, tau_lo, tau_hi, h->prm.dt_ps, dk, dw, table,
+                                   h->stream);
     MHC_CUDA(h, cudaGetLastError());
-    if (kappa_tau && (s = copy_out(h, kappa_tau, dk, sizeof(double) * rows * L, where)) != MHC_OK) return s;
-    if (kappa_w && (s = copy_out(h, kappa_w, dw, sizeof(double) * rows, where)) != MHC_OK) return s;
+    if (own_t && (s = copy_out(h, kappa_tau, dk, sizeof(double) * rows * L, where)) != MHC_OK) return s;
+    if (own_w && (s = copy_out(h, kappa_w, dw, sizeof(double) * rows, where)) != MHC_OK) return s;
     return MHC_OK;
 }
 
@@ -1519,11 +1545,13 @@ mhc_status mhc_read_xcorr(mhc_handle *h, double *xsum, int64_t *count, int32_t w
     const size_t n = (size_t)9 * nb * nb * L;
     mhc_status s;
     if (xsum) {
-        if ((s = dev_alloc(h, "xc_out", sizeof(double) * n, false)) != MHC_OK) return s;
-        launch_xcorr_transpose(dptr<float2>(h, "Xsum"), nb, L, dptr<double>(h, "xc_out"), h->stream);
+        const bool own = !direct_out(h, xsum, where);
+        if (own && (s = dev_alloc(h, "xc_out", sizeof(double) * n, false)) != MHC_OK) return s;
+        double *dx = own ? dptr<double>(h, "xc_out") : xsum;
+        launch_xcorr_transpose(dptr<float2>(h, "Xsum"), nb, L, dx, h->stream);
         h->launches++;
         MHC_CUDA(h, cudaGetLastError());
-        if ((s = copy_out(h, xsum, dptr<double>(h, "xc_out"), sizeof(double) * n, where)) != MHC_OK) return s;
+        if (own && (s = copy_out(h, xsum, dx, sizeof(double) * n, where)) != MHC_OK) return s;
     }
     if (count) {
         if ((s = dev_alloc(h, "counts", sizeof(long long) * L, false)) != MHC_OK) return s;
@@ -1548,11 +1576,12 @@ mhc_status mhc_read_kappa_xcorr(mhc_handle *h, double *kappa_tau, double tau_lo,
     if (!kappa_tau) {   // the window averages alone need no FP64 copy of the sums
         if (!kappa_w) return MHC_OK;
         if ((s = dev_alloc(h, "xw_out", sizeof(double) * (rows + L), false)) != MHC_OK) return s;
-        double *dw = dptr<double>(h, "xw_out");
+        const bool own = !direct_out(h, kappa_w, where);
+        double *scratch = dptr<double>(h, "xw_out"), *dw = own ? scratch : kappa_w;
         h->launches += launch_xcorr_window(dptr<float2>(h, "Xsum"), nb, L, h->steps, coef * h->prm.dt_ps,
-                                           tau_lo, tau_hi, h->prm.dt_ps, dw, dw + rows, h->stream);
+                                           tau_lo, tau_hi, h->prm.dt_ps, dw, scratch + rows, h->stream);
         MHC_CUDA(h, cudaGetLastError());
-        return copy_out(h, kappa_w, dw, sizeof(double) * rows, where);
+        return own ? copy_out(h, kappa_w, dw, sizeof(double) * rows, where) : MHC_OK;
     }
     if ((s = dev_alloc(h, "xc_out", sizeof(double) * rows * L, false)) != MHC_OK) return s;
     if ((s = dev_alloc(h, "xk_out", sizeof(double) * (rows * (L + 1) + L), false)) != MHC_OK) return s;

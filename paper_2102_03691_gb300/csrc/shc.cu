@@ -588,10 +588,13 @@ mhc_status mhc_shc_read_kappa(mhc_shc *s, const double *f_THz, int32_t n_freq, i
         SHC_CUDA(s, cudaStreamSynchronize(s->stream));   // the host copy may change before the copy runs
     }
     const double coef = s->Fe > 0 ? WMK / (s->V * s->T * s->Fe) : 0.0;
+    const bool direct = where == MHC_MEM_DEVICE && mhc::writable_here(kappa, s->device);
+    double *dk = direct ? kappa : s->out;
     shc_kappa_kernel<<<dim3((n_freq + KAPPA_FREQ - 1) / KAPPA_FREQ, 9), KAPPA_FREQ * KAPPA_GROUPS, 0,
                        s->stream>>>(s->Ksum, s->nc, s->steps, s->dt, coef, tw + (size_t)window * s->nc,
-                                    ctab, n_freq, s->out);
+                                    ctab, n_freq, dk);
     SHC_CUDA(s, cudaGetLastError());
+    if (direct) return MHC_OK;
     const cudaMemcpyKind kind = where == MHC_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     SHC_CUDA(s, cudaMemcpyAsync(kappa, s->out, sizeof(double) * 9 * n_freq, kind, s->stream));
     if (where == MHC_MEM_HOST) return shc_check_status(s);

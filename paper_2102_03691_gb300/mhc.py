@@ -361,12 +361,22 @@ def _is_torch(x) -> bool:
     return type(x).__module__.startswith("torch")
 
 
+# (torch dtype of a numpy dtype), filled when the first tensor comes by
+_TORCH_DTYPES = {}
+
+
+def _torch_dtype(dtype):
+    if not _TORCH_DTYPES:
+        import torch
+        _TORCH_DTYPES.update({np.float32: torch.float32, np.float64: torch.float64,
+                              np.int32: torch.int32, np.int64: torch.int64})
+    return _TORCH_DTYPES[dtype]
+
+
 def _ptr(x, dtype):
     """(pointer, where, keepalive) for a numpy array or a torch CUDA tensor."""
     if _is_torch(x):
-        import torch
-        want = {np.float32: torch.float32, np.float64: torch.float64,
-                np.int32: torch.int32, np.int64: torch.int64}[dtype]
+        want = _TORCH_DTYPES.get(dtype) or _torch_dtype(dtype)
         if x.dtype != want:
             raise TypeError(f"expected {want}, got {x.dtype}")
         if not x.is_contiguous():
@@ -504,8 +514,8 @@ class ModalHeatCurrent:
         if wv != ww:
             raise ValueError("v and W must be in the same memory space")
         K = int(kv.shape[0])
-        nv = int(np.prod(kv.shape)) if not _is_torch(kv) else kv.numel()
-        nw = int(np.prod(kw.shape)) if not _is_torch(kw) else kw.numel()
+        nv = kv.numel() if _is_torch(kv) else kv.size
+        nw = kw.numel() if _is_torch(kw) else kw.size
         if nv != K * self.N * 3 or nw != K * self.N * 9:
             raise ValueError(f"v must be [K][{self.N}][3] and W [K][{self.N}][9]")
         if async_inputs and wv == MEM_HOST:

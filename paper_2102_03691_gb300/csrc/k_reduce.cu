@@ -10,56 +10,122 @@ namespace mhc {
 namespace {
 
 // ------------------------------------------------------------------ K3
-// One CTA per bin, one thread per (step, component) of a 256-step pass: thread t handles
-// component a = t % 3 and steps k = t/3 + 256 j.  J_b^a(k) = sum of the bin's partial slots in
-// slot order; the HNEMA sums over the block's steps in FP64 with a fixed reduction tree
-// (deterministic).  CTA 0 also sums the total current.
-constexpr int BF_STEPS = 256;
-constexpr int BF_THREADS = 3 * BF_STEPS;
-__device__ __forceinline__ void bin_finish_body(const float *__restrict__ partials, int n_slots,
-                                                const int *slot_begin, int B, int K, float *Jb,
-                                                double *hsum, const double *Jtot, double *Jsum,
-                                                int b) {
-    const int a = threadIdx.x % 3, k0 = threadIdx.x / 3;
-    const int s0 = slot_begin[b], s1 = slot_begin[b + 1];
-    double acc = 0.0, acc_tot = 0.0;
-    for (int k = k0; k < K; k += BF_STEPS) {
-        const float *row = partials + ((size_t)k * 3 + a) * n_slots;
-        float s = 0.f;
-        for (int q = s0; q < s1; ++q) s += row[q];
-        Jb[((size_t)k * B + b) * 3 + a] = s;
-        acc += (double)s;
-        if (b == 0) acc_tot += Jtot[3 * k + a];
-    }
-    __shared__ double red[2][BF_THREADS];
-    red[0][threadIdx.x] = acc;
-    red[1][threadIdx.x] = acc_tot;
-    __syncthreads();
-    for (int off = BF_STEPS / 2; off > 0; off >>= 1) {   // over k0, per component
-        if (k0 < off) {
-            red[0][threadIdx.x] += red[0][threadIdx.x + 3 * off];
-            if (b == 0) red[1][threadIdx.x] += red[1][threadIdx.x + 3 * off];
+// One CTA per bin, thread t on component t % 3 of the steps t / 3 + (threads / 3) j:
+// J_b^a(k) = sum of the bin's partial slots in slot order, and the HNEMA sums over the block's
+// steps.  One CTA more sums the total current.  Bound by latency (three dependent round trips to
+// memory: slots, sums, the HNEMA sum): so eight of a thread's slots (of one step, or of four steps
+// where a block has that many a thread) are in flight together, the steps are added in unevaluated float pairs (FP32 instructions; the FP64 pipe was
+// 40% busy with conversions and a tree of FP64 sums) and reduced by one barrier and a warp a
+// component, with one FP64 add a component at the end (fixed order: deterministic).  It is launched
+// plainly: as a programmatic dependent of the projection it made the 8000-atom push 20 us and the
+// 512-atom push 2 us longer.
+// Measured (ncu, us, before -> now): 600 rows, K = 128 10.7 -> 5.6; 200 rows, K = 128 6.9 -> 5.5;
+// 16 systems of 52 bins, K = 256 22.1 -> 19.3; 100 rows, K = 1000 8.6 -> 8.1; 64 rows of 13 slots,
+// K = 256 7.5 -> 7.6.
+constexpr int BF_MAX_THREADS = 768;
+int bf_threads(int K) { return K <= 128 ? 384 : BF_MAX_THREADS; }
+
+// (s, c) += (s2, c2) as unevaluated float pairs (_rn keeps it from being contracted)
+__device__ __forceinline__ void bf_pair_add(float &s, float &c, float s2, float c2) {
+    const float t = __fadd_rn(s, s2);
+    const float bp = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(s2, bp));
+    s = t;
+    c = __fadd_rn(c, __fadd_rn(c2, e));
+}
+
+// (Plain loads: a bin's slots share sectors, so most of them hit L1.)
+// J_b^a of the steps k0, k0 + steps, ..: the bin's slots [s0, s1) added in order, QU slots of
+// PASSES steps loaded at a time; the sums over the steps in (hs, hc).
+template <int PASSES, int QU>
+__device__ __forceinline__ void bf_steps(const float *partials, int n_slots, int s0, int s1,
+                                         int b, int a, int B, int K, int k0, int steps, float *Jb,
+                                         float &hs, float &hc) {
+    for (int k = k0; k < K; k += PASSES * steps) {
+        float s[PASSES];
+#pragma unroll
+        for (int u = 0; u < PASSES; ++u) s[u] = 0.f;
+        for (int q = s0; q < s1; q += QU) {
+            float v[QU][PASSES];
+#pragma unroll
+            for (int w = 0; w < QU; ++w)
+#pragma unroll
+                for (int u = 0; u < PASSES; ++u)
+                    v[w][u] = q + w < s1 && k + u * steps < K
+                                  ? partials[((size_t)(k + u * steps) * 3 + a) * n_slots + q + w]
+                                  : 0.f;
+#pragma unroll
+            for (int w = 0; w < QU; ++w)
+                if (q + w < s1)
+#pragma unroll
+                    for (int u = 0; u < PASSES; ++u) s[u] += v[w][u];
         }
-        __syncthreads();
-    }
-    if (threadIdx.x < 3) {
-        hsum[b * 3 + threadIdx.x] += red[0][threadIdx.x];
-        if (b == 0) Jsum[threadIdx.x] += red[1][threadIdx.x];
+#pragma unroll
+        for (int u = 0; u < PASSES; ++u)
+            if (k + u * steps < K) {
+                Jb[((size_t)(k + u * steps) * B + b) * 3 + a] = s[u];
+                bf_pair_add(hs, hc, s[u], 0.f);
+            }
     }
 }
 
-// steps: the step counter, advanced by K here (the push's later kernels subtract K), or null.
-__global__ void __launch_bounds__(BF_THREADS) bin_finish_kernel(const float *__restrict__ partials,
-                                                                int n_slots, const int *slot_begin,
-                                                                int B, int K, float *Jb,
-                                                                double *hsum, const double *Jtot,
-                                                                double *Jsum, long long *steps) {
+__device__ __forceinline__ void bin_finish_body(const float *partials, int n_slots,
+                                                const int *slot_begin, int B, int K, float *Jb,
+                                                double *hsum, const double *Jtot, double *Jsum,
+                                                int b) {
+    __shared__ float2 red[BF_MAX_THREADS];
+    __shared__ double red_tot[BF_MAX_THREADS / 32][3];
+    const int t = threadIdx.x, a = t % 3, k0 = t / 3, steps = blockDim.x / 3;
+    const int lane = t & 31, warp = t >> 5;
+    if (b == B) {   // the total current, in FP64
+        double acc[3] = {0.0, 0.0, 0.0};
+        for (int k = t; k < K; k += blockDim.x)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) acc[q] += Jtot[3 * k + q];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_down_sync(FULL_MASK, acc[q], o);
+            if (lane == 0) red_tot[warp][q] = acc[q];
+        }
+        __syncthreads();
+        if (t < 3) {
+            double s = 0.0;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red_tot[w][t];
+            Jsum[t] += s;
+        }
+        return;
+    }
+    const int s0 = slot_begin[b], s1 = slot_begin[b + 1];
+    const double old = t < 96 && lane == 0 ? hsum[b * 3 + warp] : 0.0;   // warp = component below
+    float hs = 0.f, hc = 0.f;
+    if (K <= steps) bf_steps<1, 8>(partials, n_slots, s0, s1, b, a, B, K, k0, steps, Jb, hs, hc);
+    else bf_steps<4, 2>(partials, n_slots, s0, s1, b, a, B, K, k0, steps, Jb, hs, hc);
+    red[t] = make_float2(hs, hc);
+    __syncthreads();
+    if (warp < 3) {   // component `warp`: lane l the threads 3 (l + 32 j) + warp, then the lanes
+        hs = hc = 0.f;
+        for (int j = lane; j < steps; j += 32) bf_pair_add(hs, hc, red[3 * j + warp].x, red[3 * j + warp].y);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            bf_pair_add(hs, hc, __shfl_down_sync(FULL_MASK, hs, o), __shfl_down_sync(FULL_MASK, hc, o));
+        if (lane == 0) hsum[b * 3 + warp] = old + ((double)hs + (double)hc);
+    }
+}
+
+// steps: the step counter, advanced by K here, or null.
+__global__ void __launch_bounds__(BF_MAX_THREADS, 2) bin_finish_kernel(const float *partials,
+                                                                    int n_slots, const int *slot_begin,
+                                                                    int B, int K, float *Jb,
+                                                                    double *hsum, const double *Jtot,
+                                                                    double *Jsum, long long *steps) {
     if (steps && blockIdx.x == 0 && threadIdx.x == 0) *steps += K;
     bin_finish_body(partials, n_slots, slot_begin, B, K, Jb, hsum, Jtot, Jsum, blockIdx.x);
 }
 
-// All systems of a group in one launch: CTAs cta_begin[j] .. cta_begin[j+1) are system j's bins.
-__global__ void __launch_bounds__(BF_THREADS) bin_finish_group_kernel(const __grid_constant__ FinishGroupArgs g) {
+// All systems of a group in one launch: CTAs cta_begin[j] .. cta_begin[j+1) are system j's bins
+// and its total current.
+__global__ void __launch_bounds__(BF_MAX_THREADS, 2) bin_finish_group_kernel(const __grid_constant__ FinishGroupArgs g) {
     int j = 0;
     while (j + 1 < g.n && (int)blockIdx.x >= g.cta_begin[j + 1]) ++j;
     if ((int)blockIdx.x == g.cta_begin[j] && threadIdx.x == 0) *g.steps[j] += g.K[j];
@@ -511,8 +577,7 @@ void launch_bin_finish(const float *partials, int n_slots, const int *slot_begin
                        float *Jb, double *hsum, const double *Jtot, double *Jsum, long long *steps,
                        cudaStream_t s) {
     if (B <= 0 || K <= 0) return;
-    // launched plainly: as a programmatic dependent it cost the N = 512 GKMA step ~5 us
-    bin_finish_kernel<<<B, BF_THREADS, 0, s>>>(partials, n_slots, slot_begin, B, K, Jb, hsum, Jtot,
+    bin_finish_kernel<<<B + 1, bf_threads(K), 0, s>>>(partials, n_slots, slot_begin, B, K, Jb, hsum, Jtot,
                                                Jsum, steps);
 }
 
@@ -546,8 +611,12 @@ cudaError_t lag_corr_prepare() {
 void launch_bin_finish_group(FinishGroupArgs g, cudaStream_t s) {
     if (g.n < 1) return;
     g.cta_begin[0] = 0;
-    for (int j = 0; j < g.n; ++j) g.cta_begin[j + 1] = g.cta_begin[j] + (g.K[j] > 0 ? g.B[j] : 0);
-    if (g.cta_begin[g.n] > 0) bin_finish_group_kernel<<<g.cta_begin[g.n], BF_THREADS, 0, s>>>(g);
+    int kmax = 0;
+    for (int j = 0; j < g.n; ++j) {
+        g.cta_begin[j + 1] = g.cta_begin[j] + (g.K[j] > 0 ? g.B[j] + 1 : 0);
+        kmax = std::max(kmax, g.K[j]);
+    }
+    if (g.cta_begin[g.n] > 0) bin_finish_group_kernel<<<g.cta_begin[g.n], bf_threads(kmax), 0, s>>>(g);
 }
 
 cudaError_t launch_lag_corr(const float *Jb, const double *Jring, int R, double *Csum, int K, int B,

@@ -214,7 +214,8 @@ int tc_make_tmap(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols,
 // The same for FP32, unswizzled.
 int tc_make_tmap_f32(CUtensorMap *m, const void *base, uint64_t rows, uint64_t cols, uint64_t ld,
                      uint32_t box_rows, uint32_t box_cols);
-cudaError_t launch_tc_single(const TcParams<1> &p, const TcConfig &c, cudaStream_t s);
+// pdl: as a programmatic dependent of the pack (the kernel before it on the stream).
+cudaError_t launch_tc_single(const TcParams<1> &p, const TcConfig &c, cudaStream_t s, bool pdl);
 // With prob[0].n_split > 1 or sk_parts > 0: sum the splits' partial projections of the block (in
 // split order) and run the tile epilogue (Eq. 16 product, bin-run sums into partials).
 cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s);

@@ -601,6 +601,13 @@ mhc_status run_projection(mhc_handle *h, int K) {
     TcConfig c = h->tc;
     TcProblem &P = h->tcp.prob[0];
     const bool stall = (h->prm.flags & MHC_FLAG_TEST_STALL) != 0;
+    // As a programmatic dependent of the pack the projection sets up while the pack's last CTAs
+    // finish: 1.2 us of a 119 us push at 512 atoms x 1000 steps.  A graph with a programmatic edge
+    // starts later, though: at 64 atoms x 32 steps the push took 38.9 us with it and 34.8 without.
+    // The line lies at a pack of one wave of CTAs (512 atoms and step a CTA); at 1003 x 77, just
+    // below it, both take 59.7 us.  (The split finish and the kernels after it are launched
+    // plainly: 61.5 us there with the finish as a dependent, and see the bin finish.)
+    const bool pdl = (int64_t)K * h->N >= (int64_t)h->sm_count * 512;
     h->tcp.stall_inject = stall ? 1 : 0;
     h->tcp.wait_limit = stall ? 200000000ll : 2000000000ll;   // 0.1 s when testing the timeout
     P.K = K;
@@ -629,7 +636,7 @@ mhc_status run_projection(mhc_handle *h, int K) {
         P.split_ws = dptr<float>(h, "split_ws");
         P.n_tiles = q.tiles;
         c.grid = q.parts_all * (c.pair ? 2 : 1);
-        cudaError_t e = launch_tc_single(h->tcp, c, h->stream);
+        cudaError_t e = launch_tc_single(h->tcp, c, h->stream, pdl);
         h->launches++;
         if (e == cudaSuccess && q.planes() > 1) {
             e = launch_tc_split_finish(h->tcp, h->stream);
@@ -652,7 +659,7 @@ mhc_status run_projection(mhc_handle *h, int K) {
     P.split_ws = S > 1 ? dptr<float>(h, "split_ws") : nullptr;
     P.n_tiles = mode_tiles(h, c) * P.n_col_tiles * S;
     c.grid = std::min(sched_units(h, c), P.n_tiles) * (c.pair ? 2 : 1);
-    cudaError_t e = launch_tc_single(h->tcp, c, h->stream);
+    cudaError_t e = launch_tc_single(h->tcp, c, h->stream, pdl);
     h->launches++;
     if (e == cudaSuccess && S > 1) {
         e = launch_tc_split_finish(h->tcp, h->stream);

@@ -296,6 +296,7 @@ __global__ void __launch_bounds__(128 + BN, 1) tc_modal_kernel(const __grid_cons
     volatile int *abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    griddep_launch_dependents();   // the next kernel may take the SMs this grid leaves
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -530,6 +531,7 @@ __global__ void __launch_bounds__(128 + BN, 1) tc_modal_pair_kernel(const __grid
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
+    griddep_launch_dependents();   // the next kernel may take the SMs this grid leaves
     const int pair = (int)cluster_id_x(), npairs = (int)nclusters_x();
 
     if (threadIdx.x == 0) {
@@ -857,6 +859,7 @@ __device__ __forceinline__ void fin_add(float (&acc)[FIN_COLS], const TcProblem 
 template <bool DIR>
 __global__ void __launch_bounds__(128) tc_split_finish_kernel(const __grid_constant__ TcParams<1> p) {
     extern __shared__ float4 fin_smem4[];
+    griddep_wait();   // the projection's stored segments
     const TcProblem &P = p.prob[0];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = blockIdx.x * 4 + warp;   // 32-mode group (warp-uniform)
@@ -899,7 +902,7 @@ __global__ void __launch_bounds__(128) tc_split_finish_kernel(const __grid_const
 
 }  // namespace
 
-cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s) {
+cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s, bool pdl) {
     const TcProblem &P = p.prob[0];
     if ((P.n_split <= 1 && P.sk_parts <= 0) || !P.split_ws || P.m_pad % 128 || P.ws_cols % FIN_COLS)
         return cudaErrorInvalidValue;
@@ -909,9 +912,18 @@ cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s) {
     const bool dir = P.dir_seg_kb > 0;
     if (smem_ok[dir] != cudaSuccess) return smem_ok[dir];
     const dim3 grid((unsigned)(P.m_pad / 128), (unsigned)((P.K + FIN_STEPS - 1) / FIN_STEPS));
-    if (dir) tc_split_finish_kernel<true><<<grid, 128, FIN_SMEM, s>>>(p);
-    else tc_split_finish_kernel<false><<<grid, 128, FIN_SMEM, s>>>(p);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(128, 1, 1);
+    cfg.dynamicSmemBytes = FIN_SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // after the projection
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return dir ? cudaLaunchKernelEx(&cfg, tc_split_finish_kernel<true>, p)
+               : cudaLaunchKernelEx(&cfg, tc_split_finish_kernel<false>, p);
 }
 
 const TcConfig TC_CONFIGS[TC_NUM_CONFIGS] = {

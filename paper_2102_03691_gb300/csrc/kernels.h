@@ -218,7 +218,7 @@ int tc_make_tmap_f32(CUtensorMap *m, const void *base, uint64_t rows, uint64_t c
 cudaError_t launch_tc_single(const TcParams<1> &p, const TcConfig &c, cudaStream_t s, bool pdl);
 // With prob[0].n_split > 1 or sk_parts > 0: sum the splits' partial projections of the block (in
 // split order) and run the tile epilogue (Eq. 16 product, bin-run sums into partials).
-cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s);
+cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s, bool pdl);
 // d elements per promotion chunk of the tensor-core kernels (splits are whole chunks)
 constexpr int TC_PROMOTE_D = 128;
 cudaError_t launch_tc_group(const TcParams<TC_MAX_GROUP> &p, const TcConfig &c, cudaStream_t s);
@@ -345,6 +345,8 @@ int xcorr_make_maps(const XcPlan &pl, const void *Whi, const void *Wlo, XcTcPara
 // [t0 - L + 1, t0 + K)) then the tensor-core kernel.  Needs K + L - 1 <= min(R, U_pad).
 cudaError_t launch_bin_xcorr(const XcPlan &pl, XcTcParams p, const float *ring, int R, int K,
                              const long long *t0_dev, void *Whi, void *Wlo, cudaStream_t s);
+// Stream the state through L2 (for timing what runs between two updates of it).
+void launch_xcorr_touch(const XcPlan &pl, const XcTcParams &p, cudaStream_t s);
 // out[b][b'][mu][nu][l] = X[l][3b'+nu][3b+mu] (float pair -> FP64)
 void launch_xcorr_transpose(const float2 *X, int nb, int L, double *out, cudaStream_t s);
 // The window averages alone of the bin-bin sums, [b][b'][mu][nu], straight from the state X

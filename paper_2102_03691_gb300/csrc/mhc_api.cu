@@ -601,12 +601,11 @@ mhc_status run_projection(mhc_handle *h, int K) {
     TcConfig c = h->tc;
     TcProblem &P = h->tcp.prob[0];
     const bool stall = (h->prm.flags & MHC_FLAG_TEST_STALL) != 0;
-    // As a programmatic dependent of the pack the projection sets up while the pack's last CTAs
-    // finish: 1.2 us of a 119 us push at 512 atoms x 1000 steps.  A graph with a programmatic edge
-    // starts later, though: at 64 atoms x 32 steps the push took 38.9 us with it and 34.8 without.
-    // The line lies at a pack of one wave of CTAs (512 atoms and step a CTA); at 1003 x 77, just
-    // below it, both take 59.7 us.  (The split finish and the kernels after it are launched
-    // plainly: 61.5 us there with the finish as a dependent, and see the bin finish.)
+    // As programmatic dependents the projection and its split finish set up while the last CTAs of
+    // the kernel before finish: about 1 us each of a 119 us push at 512 atoms x 1000 steps.  A
+    // graph with a programmatic edge starts later, though: at 64 atoms x 32 steps the push took
+    // 38.9 us with the edge and 34.8 without.  The line lies at a pack of one wave of CTAs (512
+    // atoms and step a CTA); at 1003 x 77, just below it, both take 60 us.
     const bool pdl = (int64_t)K * h->N >= (int64_t)h->sm_count * 512;
     h->tcp.stall_inject = stall ? 1 : 0;
     h->tcp.wait_limit = stall ? 200000000ll : 2000000000ll;   // 0.1 s when testing the timeout
@@ -639,7 +638,7 @@ mhc_status run_projection(mhc_handle *h, int K) {
         cudaError_t e = launch_tc_single(h->tcp, c, h->stream, pdl);
         h->launches++;
         if (e == cudaSuccess && q.planes() > 1) {
-            e = launch_tc_split_finish(h->tcp, h->stream);
+            e = launch_tc_split_finish(h->tcp, h->stream, pdl);
             h->launches++;
         }
         if (e != cudaSuccess)
@@ -662,7 +661,7 @@ mhc_status run_projection(mhc_handle *h, int K) {
     cudaError_t e = launch_tc_single(h->tcp, c, h->stream, pdl);
     h->launches++;
     if (e == cudaSuccess && S > 1) {
-        e = launch_tc_split_finish(h->tcp, h->stream);
+        e = launch_tc_split_finish(h->tcp, h->stream, pdl);
         h->launches++;
     }
     if (e != cudaSuccess)
@@ -731,31 +730,51 @@ void tune_file_append_locked(const TuneKey &k, const TcConfig &c) {
     std::fclose(f);
 }
 
-// Time candidate configurations in interleaved rounds (one warm-up launch each, then
-// `rounds` rounds of one timed launch of every candidate) and keep each candidate's fastest
-// launch: the candidates see the same clock and power state, where timing them one after the
-// other let the power cap, reached during the first candidates' launches, slow the last ones.
+// Time candidate configurations in interleaved rounds (one warm-up launch each, then `rounds`
+// rounds of every candidate) and keep each candidate's fastest round: the candidates see the same
+// clock and power state, where timing them one after the other let the power cap, reached during
+// the first candidates' launches, slow the last ones.  Short projections run several times a
+// round, queued behind one more that is not timed: a single launch of a few tens of microseconds
+// between two events also times the host's launches, two of them with a split.  With the
+// cross-correlations every launch is timed by itself behind a read of their state, which streams
+// through L2 between two projections of a run: from a warm L2 512 atoms x 250 steps look best
+// unsplit, and a run of four blocks with 64 bins then takes 485 us instead of 457 with three splits.
 mhc_status time_candidates(mhc_handle *h, int K, std::vector<std::pair<float, TcConfig>> &cands,
                            int rounds = 3) {
+    constexpr float ROUND_MS = 0.3f;   // GPU time of a candidate's round
+    constexpr int MAX_REPS = 8;
     cudaEvent_t e0, e1;
     MHC_CUDA(h, cudaEventCreate(&e0));
     MHC_CUDA(h, cudaEventCreate(&e1));
     mhc_status s = MHC_OK;
-    for (auto &x : cands) {
+    // one timed round of candidate c: `lead` untimed launches, then `reps` timed ones
+    auto timed = [&](const TcConfig &c, int lead, int reps, float &ms) -> mhc_status {
+        if (mhc_status q = set_tc_config(h, c); q != MHC_OK) return q;
+        if (has_xcorr(h)) launch_xcorr_touch(h->xc_plan, h->xcp, h->stream);
+        for (int r = 0; r < lead; ++r)
+            if (mhc_status q = run_projection(h, K); q != MHC_OK) return q;
+        if (cudaEventRecord(e0, h->stream) != cudaSuccess) return fail(h, MHC_ERR_CUDA, "event record");
+        for (int r = 0; r < reps; ++r)
+            if (mhc_status q = run_projection(h, K); q != MHC_OK) return q;
+        if (cudaEventRecord(e1, h->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+            cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)
+            return fail(h, MHC_ERR_CUDA, "autotune timing failed");
+        ms /= (float)reps;
+        return MHC_OK;
+    };
+    float shortest = 1e30f;
+    for (auto &x : cands) {   // warm-up, and the length of a launch
         x.first = 1e30f;
-        if ((s = set_tc_config(h, x.second)) != MHC_OK || (s = run_projection(h, K)) != MHC_OK) break;
+        float ms = 0.f;
+        if ((s = timed(x.second, has_xcorr(h) ? 0 : 1, 1, ms)) != MHC_OK) break;
+        shortest = std::min(shortest, ms);
     }
+    const int reps =
+        has_xcorr(h) ? 1 : std::max(1, std::min(MAX_REPS, (int)(ROUND_MS / std::max(shortest, 1e-3f))));
     for (int r = 0; r < rounds && s == MHC_OK; ++r)
         for (auto &x : cands) {
             float ms = 0.f;
-            if ((s = set_tc_config(h, x.second)) != MHC_OK) break;
-            if (cudaEventRecord(e0, h->stream) != cudaSuccess) { s = fail(h, MHC_ERR_CUDA, "event record"); break; }
-            if ((s = run_projection(h, K)) != MHC_OK) break;
-            if (cudaEventRecord(e1, h->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
-                cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) {
-                s = fail(h, MHC_ERR_CUDA, "autotune timing failed");
-                break;
-            }
+            if ((s = timed(x.second, reps > 1 ? 1 : 0, reps, ms)) != MHC_OK) break;
             x.first = std::min(x.first, ms);
         }
     cudaEventDestroy(e0);

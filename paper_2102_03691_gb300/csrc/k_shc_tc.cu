@@ -29,6 +29,10 @@
 // (deterministic).  128 x 256 tiles keep the shared-memory operand reads of each MMA below
 // the shared-memory bandwidth (a 128 x 128 MMA reading both operands would sit at it).
 // Every barrier wait is bounded (sticky status on timeout, as in k_tc.cu).
+//
+// The correlation and its reduction are programmatic dependents of the pack and the correlation: a
+// push is launched kernel by kernel, and the set-up of each overlaps the end of the one before
+// (8000 atoms, 250 lags, K = 256: 110.6 -> 104.5 us a push with its spectrum).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -210,6 +214,7 @@ __global__ void __launch_bounds__(THREADS) shc_tc_pack_bulk_kernel(
     long long t0, void *A_hi, void *A_lo, void *B_hi, void *B_lo, float *scaleA, float *scaleB,
     int *status, long long wait_limit) {
     constexpr int APC = 4 * THREADS;
+    griddep_launch_dependents();   // the correlation may set up on the SMs this grid leaves
     extern __shared__ float4 pk_smem4[];
     float *sv = reinterpret_cast<float *>(pk_smem4);   // [APC][3]
     float *sw = sv + APC * 3;                          // [APC][9]
@@ -413,6 +418,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) shc_tc_kernel(const __grid_cons
     cluster_sync_all();   // both CTAs' barriers initialised, TMEM allocated in both
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    griddep_launch_dependents();
+    griddep_wait();   // the pack's operands (the set-up above overlapped its end)
 
     if (warp == 0 && lane == 0) {
         // ------------------------------------------------------------ TMA producer
@@ -580,6 +587,7 @@ constexpr int RED_GROUPS = 8;
 __global__ void __launch_bounds__(32 * RED_GROUPS) shc_tc_reduce_kernel(const __grid_constant__ ShcTcParams p,
                                                                        double *Ksum) {
     __shared__ double part[RED_GROUPS][32];
+    griddep_wait();   // the units' diagonals
     const int c = blockIdx.y, lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int l = blockIdx.x * 32 + lane;
     const int per_c = p.n_pairs * p.splits;
@@ -710,8 +718,11 @@ cudaError_t shc_tc_set_attr() {
 cudaError_t launch_shc_tc(const ShcTcParams &p, cudaStream_t s) {
     cudaError_t e = shc_tc_set_attr();
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = shc_tc_config(9 * p.n_pairs * p.splits, attr);   // n_pairs is even
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;          // after the pack
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
     cfg.stream = s;
     return cudaLaunchKernelEx(&cfg, shc_tc_kernel, p);
 }
@@ -728,9 +739,18 @@ int shc_tc_max_clusters() {
     return n;
 }
 
-void launch_shc_tc_reduce(const ShcTcParams &p, double *Ksum, cudaStream_t s) {
+cudaError_t launch_shc_tc_reduce(const ShcTcParams &p, double *Ksum, cudaStream_t s) {
     dim3 grid((p.nc + 31) / 32, 9);
-    shc_tc_reduce_kernel<<<grid, 32 * RED_GROUPS, 0, s>>>(p, Ksum);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(32 * RED_GROUPS, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // after the correlation
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, shc_tc_reduce_kernel, p, Ksum);
 }
 
 }  // namespace mhc

@@ -262,7 +262,7 @@ cudaError_t launch_shc_tc(const ShcTcParams &p, cudaStream_t s);
 int shc_tc_max_clusters();
 size_t shc_tc_smem_bytes();
 // Ksum[c][l] += sum over the units of pair c, in order, of their diagonal sums at lag l (FP64).
-void launch_shc_tc_reduce(const ShcTcParams &p, double *Ksum, cudaStream_t s);
+cudaError_t launch_shc_tc_reduce(const ShcTcParams &p, double *Ksum, cudaStream_t s);
 
 // ---------------------------------------------------------------- K3 .. K5
 // Jb[k][b][a] = sum of partial slots of bin b; HNEMA sums += sum_k Jb (FP64);

@@ -484,8 +484,7 @@ mhc_status mhc_shc_push(mhc_shc *s, const float *v, const float *W, int32_t K, i
         }
         SHC_CUDA(s, mhc::launch_shc_tc(s->tcp, s->stream));
         if (ev1) SHC_CUDA(s, cudaEventRecord(ev1, s->stream));
-        mhc::launch_shc_tc_reduce(s->tcp, s->Ksum, s->stream);
-        SHC_CUDA(s, cudaGetLastError());
+        SHC_CUDA(s, mhc::launch_shc_tc_reduce(s->tcp, s->Ksum, s->stream));
         s->steps += K;
         return release();
     }

@@ -368,6 +368,8 @@ SgemmPlan fp32_plan(const mhc_handle *h, int C) {
     return sgemm_plan(h->M_pad, C, h->dir ? h->N_pad : h->D_ld, h->dir ? 3 : 1, h->sm_count, true);
 }
 
+void reserve_tuned_ws(mhc_handle *h);
+
 // Sort kept modes by bin (stable), build the per-mode bin/slot tables of the fused
 // epilogue, gather+split E into the stored order and set up the tensor maps.
 mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_t B) {
@@ -493,6 +495,7 @@ mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_
         h->tcp.idesc = idesc_f16(h->split == SPLIT_BF16 ? 1u : 0u, (c.pair ? 2 : 1) * TC_BM, (uint32_t)c.bn);
     }
     h->bins_ready = true;
+    reserve_tuned_ws(h);
     return reset_accumulators(h);
 }
 
@@ -728,6 +731,23 @@ void tune_file_append_locked(const TuneKey &k, const TcConfig &c) {
                  k.split_req, (long long)k.D_ld, (long long)k.M_eff, c.bn, c.bk, c.stages, c.pair,
                  c.split, k.device.c_str());
     std::fclose(f);
+}
+
+// The split workspace of the tile already tuned for this shape and the longest block (by another
+// handle of the process, or in the tuning file), allocated with the bins: the first push would
+// otherwise stop for it (about 100 us).  Where it does not fit, the push that needs it reports so.
+void reserve_tuned_ws(mhc_handle *h) {
+    if (!is_tc(h) || h->prm.tile_config != 0 || h->M_eff == 0) return;
+    TcConfig c{};
+    {
+        std::lock_guard<std::mutex> lock(g_tune_mutex);
+        tune_file_read_locked();
+        auto it = g_tune_cache.find(tune_key(h, h->prm.k_max));
+        if (it == g_tune_cache.end()) return;
+        c = it->second;
+    }
+    if (c.split > 1 && h->dir) return;   // refused by the push that would use it
+    if (ensure_split_ws(h, c) != MHC_OK) h->err.clear();
 }
 
 // Time candidate configurations in interleaved rounds (one warm-up launch each, then `rounds`

@@ -139,8 +139,9 @@ typedef struct {
                             > 0); 1..16 = fixed; -1 = balanced: the chunks of all tiles, tile
                             after tile, cut into one range of equal length per CTA (or CTA
                             pair), a tile cut by a range boundary finished by the same kernel.
-                            Not with MHC_FLAG_DIRECTION (must be 0 or 1); grouped launches run
-                            unsplit. */
+                            With MHC_FLAG_DIRECTION it must be 0 or 1 (0: the autotuner may cut
+                            the last wave's tiles, each direction segment by itself; tile_split
+                            then reads -1); grouped launches run unsplit. */
 } mhc_params;
 
 /* Counters and derived sizes of a handle. */

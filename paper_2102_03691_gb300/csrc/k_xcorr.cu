@@ -50,38 +50,51 @@ __device__ __forceinline__ void xc_pair_add(float &s, float &c, float x) {
     c = __fadd_rn(c, e);
 }
 
-// ring[(t0 + k) mod R][j] = Jb[k][j]: the block's binned currents join the history ring
-__global__ void jb_ring_store_kernel(const float *__restrict__ Jb, int K, int n, float *ring,
-                                     int R, const long long *t0_dev) {
-    const long long t0 = *t0_dev - K;   // the bin finish has advanced the counter
-    const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (q >= (long long)K * n) return;
-    const long long k = q / n, j = q - k * n;
-    ring[((t0 + k) % R) * n + j] = Jb[q];
-}
-
-// One CTA per row j < n: the row's scale from the maximum of |W[j][u]| over the window, then
-// the eight shifted FP16 hi/lo copies, Whi/Wlo[(c rows_pad + j) U_pad + u] = split(W[j][u + c]).
+// One CTA per row j < n: the block's binned currents join the history ring,
+// ring[(t0 + k) mod R][j] = Jb[k][j]; the row's window of the last K + L - 1 steps is read once, past
+// steps from the ring and the block from Jb (STAGED: into shared memory; a window too long for it is
+// read again from L2 for every copy), the scale comes from its maximum, and the eight shifted FP16
+// hi/lo copies are written eight values a thread:
+//   Whi/Wlo[(c rows_pad + j) U_pad + u] = split(W[j][u + c]).
+// Bound by latency: one row a CTA, its window read in one round of loads.  Before, the window was
+// read again from L2 and stored two bytes at a time for each of the eight copies, and the ring was
+// stored by a launch of its own.  Measured at 192 rows, K = 250, L = 200 (ncu, us): 9.1 and 2.5 for
+// the ring -> 5.8; four blocks and the read 468 -> 452.
+// t0_dev: the step counter, which the push's bin finish has already advanced by K.
 constexpr int XW_THREADS = 256;
-__global__ void __launch_bounds__(XW_THREADS) xc_window_kernel(const float *__restrict__ ring, int R,
+constexpr int XW_STAGE_MAX = 12288 - 64;   // steps of the longest staged window: what 48 KB of shared memory
+                                           // hold without opting in, less the maxima
+template <bool STAGED>
+__global__ void __launch_bounds__(XW_THREADS) xc_window_kernel(const float *__restrict__ Jb, float *ring, int R,
                                                                int n, int K, int L, int U_pad,
                                                                int rows_pad,
                                                                const long long *t0_dev,
                                                                uint16_t *Whi, uint16_t *Wlo,
                                                                float *inv_scale) {
+    extern __shared__ float xw_row[];   // STAGED: W[j][0 .. Uw), then zeros
     const int j = blockIdx.x;
     const long long t0 = *t0_dev - K;
     const long long tw0 = t0 - (L - 1);
     const int Uw = K + L - 1;
     const int base = (int)(((tw0 % R) + R) % R);   // ring row of u = 0
+    auto slot = [&](int u) {                       // u < Uw <= R
+        const int r = base + u;
+        return (size_t)(r >= R ? r - R : r) * n + j;
+    };
     auto value = [&](int u) -> float {             // W[j][u]
         if (u >= Uw || tw0 + u < 0) return 0.f;
-        int r = base + u;
-        if (r >= R) r -= R;                        // u < Uw <= R
-        return ring[(size_t)r * n + j];
+        return u >= L - 1 ? Jb[(size_t)(u - (L - 1)) * n + j] : ring[slot(u)];
     };
     float m = 0.f;
-    for (int u = threadIdx.x; u < Uw; u += XW_THREADS) m = fmaxf(m, fabsf(value(u)));
+#pragma unroll 4
+    for (int u = threadIdx.x; u < Uw; u += XW_THREADS) {
+        const float x = value(u);
+        m = fmaxf(m, fabsf(x));
+        if (STAGED) xw_row[u] = x;
+        if (u >= L - 1) ring[slot(u)] = x;   // (no past step lies there: K + L - 1 <= R)
+    }
+    if (STAGED)
+        for (int u = Uw + threadIdx.x; u < U_pad + 8; u += XW_THREADS) xw_row[u] = 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL_MASK, m, o));
     __shared__ float s_m[XW_THREADS / 32];
@@ -102,13 +115,22 @@ __global__ void __launch_bounds__(XW_THREADS) xc_window_kernel(const float *__re
     }
     __syncthreads();
     const float mul = s_mul;
-    for (int q = threadIdx.x; q < 8 * U_pad; q += XW_THREADS) {
-        const int c = q / U_pad, u = q - c * U_pad;
-        const float x = value(u + c) * mul;
-        const __half hv = __float2half_rn(x);
-        const size_t o = ((size_t)c * rows_pad + j) * U_pad + u;
-        Whi[o] = __half_as_ushort(hv);
-        Wlo[o] = __half_as_ushort(__float2half_rn(x - __half2float(hv)));
+    const int nch = U_pad / 8;   // chunks of eight u's of a copy (U_pad is a multiple of 64)
+    for (int q = threadIdx.x; q < 8 * nch; q += XW_THREADS) {
+        const int c = q / nch, u0 = 8 * (q - c * nch);
+        uint32_t hi[8], lo[8];
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            const float x = (STAGED ? xw_row[u0 + w + c] : value(u0 + w + c)) * mul;
+            const __half hv = __float2half_rn(x);
+            hi[w] = __half_as_ushort(hv);
+            lo[w] = __half_as_ushort(__float2half_rn(x - __half2float(hv)));
+        }
+        const size_t o = ((size_t)c * rows_pad + j) * U_pad + u0;
+        *reinterpret_cast<uint4 *>(Whi + o) =
+            make_uint4(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16), hi[4] | (hi[5] << 16), hi[6] | (hi[7] << 16));
+        *reinterpret_cast<uint4 *>(Wlo + o) =
+            make_uint4(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16), lo[4] | (lo[5] << 16), lo[6] | (lo[7] << 16));
     }
 }
 
@@ -379,20 +401,18 @@ cudaError_t xcorr_prepare() {
     return e;
 }
 
-void launch_jb_ring_store(const float *Jb, int K, int nb, float *ring, int R,
-                          const long long *t0_dev, cudaStream_t s) {
-    const long long total = (long long)K * nb * 3;
-    if (total <= 0) return;
-    jb_ring_store_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(Jb, K, 3 * nb, ring, R, t0_dev);
-}
-
-cudaError_t launch_bin_xcorr(const XcPlan &pl, XcTcParams p, const float *ring, int R, int K,
+cudaError_t launch_bin_xcorr(const XcPlan &pl, XcTcParams p, const float *Jb, float *ring, int R, int K,
                              const long long *t0_dev, void *Whi, void *Wlo, cudaStream_t s) {
     if (p.L <= 0 || K <= 0 || pl.n <= 0) return cudaSuccess;
     if (K + p.L - 1 > R || K + p.L - 1 > pl.U_pad) return cudaErrorInvalidValue;
-    xc_window_kernel<<<pl.n, XW_THREADS, 0, s>>>(ring, R, pl.n, K, p.L, pl.U_pad, pl.rows_pad, t0_dev, static_cast<uint16_t *>(Whi),
-                                                 static_cast<uint16_t *>(Wlo),
-                                                 const_cast<float *>(p.inv_scale));
+    uint16_t *hi = static_cast<uint16_t *>(Whi), *lo = static_cast<uint16_t *>(Wlo);
+    float *inv = const_cast<float *>(p.inv_scale);
+    if (pl.U_pad + 8 <= XW_STAGE_MAX)
+        xc_window_kernel<true><<<pl.n, XW_THREADS, sizeof(float) * (pl.U_pad + 8), s>>>(
+            Jb, ring, R, pl.n, K, p.L, pl.U_pad, pl.rows_pad, t0_dev, hi, lo, inv);
+    else
+        xc_window_kernel<false><<<pl.n, XW_THREADS, 0, s>>>(Jb, ring, R, pl.n, K, p.L, pl.U_pad, pl.rows_pad,
+                                                            t0_dev, hi, lo, inv);
     const cudaError_t attr = xcorr_prepare();
     if (attr != cudaSuccess) return attr;
     p.n_kb = (K + XC_BK - 1) / XC_BK;

@@ -315,10 +315,6 @@ struct HnemaGroupArgs {
 };
 void launch_hnema_finalize_group(const HnemaGroupArgs &a, double *mean, double *kappa, cudaStream_t s);
 // ---------------------------------------------------------------- bin-bin cross-correlations
-// ring[(t0 + k) mod R][3b+mu] = Jb[k][b][mu] (nb output rows of 3 components)
-// t0_dev: the device step counter, already advanced by K (as for launch_bin_xcorr)
-void launch_jb_ring_store(const float *Jb, int K, int nb, float *ring, int R,
-                          const long long *t0_dev, cudaStream_t s);
 // Tensor-core cross-correlation (k_xcorr.cu): n = 3 nb rows; column tiles of nj <= XC_NJ_MAX
 // rows j; row tiles of 128 rows i; the window copies hold 8 x rows_pad rows of U_pad steps.
 constexpr int XC_NJ_MAX = 192;
@@ -340,10 +336,11 @@ void xcorr_plan(int nb, int L, int k_max, int nsm, XcPlan &pl);
 cudaError_t xcorr_prepare();
 // Encode the four tensor maps over the window copies and fill the plan's fields of p.
 int xcorr_make_maps(const XcPlan &pl, const void *Whi, const void *Wlo, XcTcParams &p);
-// X[l][3b'+nu][3b+mu] += sum_k Jb[k][b][mu] Jb(t0+k-l)[b'][nu] over t0+k-l >= 0, the block
-// already in the ring: the window kernel (scales + eight shifted FP16 hi/lo copies of
-// [t0 - L + 1, t0 + K)) then the tensor-core kernel.  Needs K + L - 1 <= min(R, U_pad).
-cudaError_t launch_bin_xcorr(const XcPlan &pl, XcTcParams p, const float *ring, int R, int K,
+// The block joins the ring, ring[(t0 + k) mod R][3b+mu] = Jb[k][b][mu], and
+// X[l][3b'+nu][3b+mu] += sum_k Jb[k][b][mu] Jb(t0+k-l)[b'][nu] over t0+k-l >= 0: the window kernel
+// (ring, scales, eight shifted FP16 hi/lo copies of [t0 - L + 1, t0 + K)), then the tensor-core
+// kernel.  Needs K + L - 1 <= min(R, U_pad).  t0_dev: the device step counter, already advanced by K.
+cudaError_t launch_bin_xcorr(const XcPlan &pl, XcTcParams p, const float *Jb, float *ring, int R, int K,
                              const long long *t0_dev, void *Whi, void *Wlo, cudaStream_t s);
 // Stream the state through L2 (for timing what runs between two updates of it).
 void launch_xcorr_touch(const XcPlan &pl, const XcTcParams &p, cudaStream_t s);

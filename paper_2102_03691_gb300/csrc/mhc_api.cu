@@ -970,11 +970,10 @@ mhc_status correlate_block(mhc_handle *h, int K) {
         h->launches++;
     }
     if (has_xcorr(h)) {
-        launch_jb_ring_store(dptr<float>(h, "Jb"), K, (int)n_out_bins(h), dptr<float>(h, "Jbring"),
-                             h->R_ring, steps, h->stream);
-        MHC_CUDA(h, launch_bin_xcorr(h->xc_plan, h->xcp, dptr<float>(h, "Jbring"), h->R_ring, K, steps,
-                                     dptr<void>(h, "Xwin_hi"), dptr<void>(h, "Xwin_lo"), h->stream));
-        h->launches += 3;
+        MHC_CUDA(h, launch_bin_xcorr(h->xc_plan, h->xcp, dptr<float>(h, "Jb"), dptr<float>(h, "Jbring"),
+                                     h->R_ring, K, steps, dptr<void>(h, "Xwin_hi"),
+                                     dptr<void>(h, "Xwin_lo"), h->stream));
+        h->launches += 2;
     }
     MHC_CUDA(h, cudaGetLastError());
     return MHC_OK;

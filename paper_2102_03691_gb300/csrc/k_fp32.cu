@@ -364,8 +364,8 @@ SgemmPlan sgemm_plan(int64_t Mp, int C, int64_t Dk, int ndir, int sms, bool cut)
 }
 
 cudaError_t launch_sgemm(const SgemmParams &p, cudaStream_t s) {
-    static const cudaError_t ready = cudaFuncSetAttribute(
-        sgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SG_SMEM);
+    static PerDevice once;
+    const cudaError_t ready = opt_in_smem(once, sgemm_kernel, SG_SMEM);
     if (ready != cudaSuccess) return ready;
     if (p.plan.tiles < 1 || p.C < 1) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};

@@ -4,6 +4,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <map>
 #include <mutex>
 
 #include "common.cuh"
@@ -406,8 +407,8 @@ template <int THREADS>
 cudaError_t launch_pack_cluster(const PackArgs &a, cudaStream_t s) {
     constexpr int APC = 4 * THREADS;
     const int smem = APC * 48;
-    static cudaError_t attr = cudaFuncSetAttribute(pack_cluster_kernel<THREADS>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static PerDevice once;
+    const cudaError_t attr = opt_in_smem(once, pack_cluster_kernel<THREADS>, smem);
     if (attr != cudaSuccess) return attr;
     const int csize = (a.N + APC - 1) / APC;
     cudaLaunchConfig_t cfg = {};
@@ -434,13 +435,15 @@ namespace {
 int pack_threads(int N) { return N <= 4 * 128 ? 128 : N <= 8 * 1024 ? 256 : 512; }
 constexpr int PACK_MAX_CLUSTER = 16;
 
-// Whether a cluster of `csize` 512-thread CTAs can be resident on this device.
+// Whether a cluster of `csize` 512-thread CTAs can be resident on the current device.
 bool pack_wide_ok(int csize) {
-    static int limit = -1;   // largest cluster size found to fit
+    static std::map<int, int> limits;   // device -> largest cluster size found to fit
     static std::mutex m;
     std::lock_guard<std::mutex> lock(m);
-    if (limit < 0) {
-        limit = 8;
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess) return false;
+    if (!limits.count(device)) {
+        int limit = 8;
         const int smem = 4 * 512 * 48;
         if (cudaFuncSetAttribute(pack_cluster_kernel<512>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
             cudaFuncSetAttribute(pack_cluster_group_kernel<512>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
@@ -463,8 +466,9 @@ bool pack_wide_ok(int csize) {
             }
         }
         cudaGetLastError();
+        limits[device] = limit;
     }
-    return csize <= limit;
+    return csize <= limits[device];
 }
 
 // The cluster pack takes every system up to PACK_MAX_CLUSTER CTAs of 2048 atoms.
@@ -478,8 +482,8 @@ template <int THREADS>
 cudaError_t launch_pack_cluster_group(PackGroupArgs g, int csize, cudaStream_t s) {
     constexpr int APC = 4 * THREADS;
     const int smem = APC * 48;
-    static cudaError_t attr = cudaFuncSetAttribute(pack_cluster_group_kernel<THREADS>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static PerDevice once;
+    const cudaError_t attr = opt_in_smem(once, pack_cluster_group_kernel<THREADS>, smem);
     if (attr != cudaSuccess) return attr;
     g.cta_begin[0] = 0;
     for (int j = 0; j < g.n; ++j) g.cta_begin[j + 1] = g.cta_begin[j] + g.a[j].K * csize;

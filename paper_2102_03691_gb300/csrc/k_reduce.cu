@@ -603,9 +603,8 @@ int lag_corr_tiles(int B, int L) { return ((L + 31) / 32) * ((B + LC_ROWS / 3 - 
 cudaError_t lag_corr_prepare() {
     // a tile alone in its CTA stages at most 1024 steps or 16 warps' partials: below 80 KB
     LagCorrPlan p{LC_WARPS, 64, 1, LC_WARPS, LC_WARPS};
-    static const cudaError_t e = cudaFuncSetAttribute(
-        lag_corr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lag_corr_smem(p));
-    return e;
+    static PerDevice once;
+    return opt_in_smem(once, lag_corr_kernel, lag_corr_smem(p));
 }
 
 void launch_bin_finish_group(FinishGroupArgs g, cudaStream_t s) {

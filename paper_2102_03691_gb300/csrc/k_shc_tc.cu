@@ -640,7 +640,8 @@ cudaError_t launch_pack_bulk(const float *v, const float *W, int N, int N_pad, i
     constexpr int APC = 4 * THREADS;
     const int smem = APC * 48;
     auto kern = shc_tc_pack_bulk_kernel<SPLIT, THREADS>;
-    static cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static PerDevice once;
+    const cudaError_t attr = opt_in_smem(once, kern, smem);
     if (attr != cudaSuccess) return attr;
     const int csize = (N + APC - 1) / APC;
     cudaLaunchConfig_t cfg = {};
@@ -711,8 +712,8 @@ cudaLaunchConfig_t shc_tc_config(int grid, cudaLaunchAttribute *attr) {
 }
 
 cudaError_t shc_tc_set_attr() {
-    static cudaError_t e = cudaFuncSetAttribute(shc_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ST_SMEM);
-    return e;
+    static PerDevice once;
+    return opt_in_smem(once, shc_tc_kernel, ST_SMEM);
 }
 
 cudaError_t launch_shc_tc(const ShcTcParams &p, cudaStream_t s) {

@@ -730,13 +730,9 @@ template <int BN, int BK, int STAGES, int NPROB, bool DIR>
 cudaError_t launch_pair_impl(const TcParams<NPROB> &p, int grid, cudaStream_t s, bool pdl) {
     using L = TcPairLayout<BN, BK, STAGES>;
     auto kern = tc_modal_pair_kernel<BN, BK, STAGES, NPROB, DIR>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             L::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice once;
+    const cudaError_t ready = opt_in_smem(once, kern, L::SMEM_BYTES);
+    if (ready != cudaSuccess) return ready;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);
     cfg.blockDim = dim3(L::THREADS, 1, 1);
@@ -784,13 +780,9 @@ template <int BN, int BK, int STAGES, int NPROB, bool DIR>
 cudaError_t launch_impl(const TcParams<NPROB> &p, int grid, cudaStream_t s, bool pdl) {
     using L = TcLayout<BN, BK, STAGES>;
     auto kern = tc_modal_kernel<BN, BK, STAGES, NPROB, DIR>;
-    static bool attr_set = false;   // per process; the attribute is per function
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             L::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice once;
+    const cudaError_t ready = opt_in_smem(once, kern, L::SMEM_BYTES);
+    if (ready != cudaSuccess) return ready;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);
     cfg.blockDim = dim3(L::THREADS, 1, 1);
@@ -906,11 +898,10 @@ cudaError_t launch_tc_split_finish(const TcParams<1> &p, cudaStream_t s, bool pd
     const TcProblem &P = p.prob[0];
     if ((P.n_split <= 1 && P.sk_parts <= 0) || !P.split_ws || P.m_pad % 128 || P.ws_cols % FIN_COLS)
         return cudaErrorInvalidValue;
-    static const cudaError_t smem_ok[2] = {
-        cudaFuncSetAttribute(tc_split_finish_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FIN_SMEM),
-        cudaFuncSetAttribute(tc_split_finish_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, FIN_SMEM)};
+    static PerDevice once[2];
     const bool dir = P.dir_seg_kb > 0;
-    if (smem_ok[dir] != cudaSuccess) return smem_ok[dir];
+    const cudaError_t ready = opt_in_smem(once[dir], dir ? tc_split_finish_kernel<true> : tc_split_finish_kernel<false>, FIN_SMEM);
+    if (ready != cudaSuccess) return ready;
     const dim3 grid((unsigned)(P.m_pad / 128), (unsigned)((P.K + FIN_STEPS - 1) / FIN_STEPS));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;

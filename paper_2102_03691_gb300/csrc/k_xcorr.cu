@@ -396,9 +396,8 @@ int xcorr_make_maps(const XcPlan &pl, const void *Whi, const void *Wlo, XcTcPara
 }
 
 cudaError_t xcorr_prepare() {
-    static cudaError_t e = cudaFuncSetAttribute(xc_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                XC_SMEM);
-    return e;
+    static PerDevice once;
+    return opt_in_smem(once, xc_tc_kernel, XC_SMEM);
 }
 
 cudaError_t launch_bin_xcorr(const XcPlan &pl, XcTcParams p, const float *Jb, float *ring, int R, int K,

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "per_device.h"
+
 namespace mhc {
 
 enum Split { SPLIT_FP32 = 0, SPLIT_BF16 = 1, SPLIT_FP16 = 2 };
@@ -13,6 +15,17 @@ constexpr int SPLIT_FP32_D = 3;   // launch_prepare_modes: FP32, stored d-major
 constexpr int TC_MAX_GROUP = 16;  // systems per grouped launch
 constexpr int TC_MAX_SPLIT = 16;  // d-axis splits of one projection
 constexpr double A2_PS2_PER_EV_AMU = 9648.533212331;   // 1 eV/amu in A^2/ps^2
+
+// Opt `kernel` into `bytes` of dynamic shared memory on the current device, once a device.
+template <typename Kernel>
+cudaError_t opt_in_smem(PerDevice &once, Kernel *kernel, size_t bytes) {
+    int device = 0;
+    const cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    return once(device, [&] {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    });
+}
 
 // Whether a kernel on `device` may store doubles at p (aligned memory of that device).
 bool writable_here(const void *p, int device);

@@ -10,37 +10,29 @@ namespace mhc {
 namespace {
 
 // ------------------------------------------------------------------ K3
-// One CTA per bin, thread t on component t % 3 of the steps t / 3 + (threads / 3) j:
-// J_b^a(k) = sum of the bin's partial slots in slot order, and the HNEMA sums over the block's
-// steps.  One CTA more sums the total current.  Bound by latency (three dependent round trips to
-// memory: slots, sums, the HNEMA sum): so eight of a thread's slots (of one step, or of four steps
-// where a block has that many a thread) are in flight together, the steps are added in unevaluated float pairs (FP32 instructions; the FP64 pipe was
-// 40% busy with conversions and a tree of FP64 sums) and reduced by one barrier and a warp a
-// component, with one FP64 add a component at the end (fixed order: deterministic).  It is launched
-// plainly: as a programmatic dependent of the projection it made the 8000-atom push 20 us and the
-// 512-atom push 2 us longer.
-// Measured (ncu, us, before -> now): 600 rows, K = 128 10.7 -> 5.6; 200 rows, K = 128 6.9 -> 5.5;
-// 16 systems of 52 bins, K = 256 22.1 -> 19.3; 100 rows, K = 1000 8.6 -> 8.1; 64 rows of 13 slots,
-// K = 256 7.5 -> 7.6.
+// One CTA per bin, thread t on component t % 3 of the steps t / 3 + steps j (bf_threads(K) = 3 steps
+// threads): J_b^a(k) = sum of the bin's partial slots in slot order, and the HNEMA sums over the
+// block's steps in FP64.  One CTA more sums the total current.  Bound by latency (three dependent
+// round trips to memory: slots, sums, the HNEMA sum), so eight of a thread's slots (of one step, or
+// of four steps where a block has that many a thread) are in flight together, and the FP64 sums are
+// reduced by one barrier and a warp a component, with one read-modify-write of the sum at the end.
+// The order of the sums depends on K alone, so a grouped launch gives the bits of a solo one.  It is
+// launched plainly: as a programmatic dependent of the projection it made the 8000-atom push 20 us
+// and the 512-atom push 2 us longer.
+// Measured (ncu, us, one thread a step with a tree of FP64 sums -> now): 600 rows, K = 128
+// 10.7 -> 7.0; 200 rows, K = 128 6.9 -> 5.7; 16 systems of 52 bins, K = 256 22.1 -> 22.4; 100 rows,
+// K = 1000 8.6 -> 8.5; 64 rows of 13 slots, K = 256 7.5 -> 7.5.  The sums over the steps in pairs of
+// floats took 6.1, 5.5, 20.4, 8.3 and 7.5, but held 48 bits, and no infinities.
 constexpr int BF_MAX_THREADS = 768;
-int bf_threads(int K) { return K <= 128 ? 384 : BF_MAX_THREADS; }
-
-// (s, c) += (s2, c2) as unevaluated float pairs (_rn keeps it from being contracted)
-__device__ __forceinline__ void bf_pair_add(float &s, float &c, float s2, float c2) {
-    const float t = __fadd_rn(s, s2);
-    const float bp = __fsub_rn(t, s);
-    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(s2, bp));
-    s = t;
-    c = __fadd_rn(c, __fadd_rn(c2, e));
-}
+__host__ __device__ constexpr int bf_threads(int K) { return K <= 128 ? 384 : BF_MAX_THREADS; }
 
 // (Plain loads: a bin's slots share sectors, so most of them hit L1.)
 // J_b^a of the steps k0, k0 + steps, ..: the bin's slots [s0, s1) added in order, QU slots of
-// PASSES steps loaded at a time; the sums over the steps in (hs, hc).
+// PASSES steps loaded at a time; the sum over the steps in hs.
 template <int PASSES, int QU>
 __device__ __forceinline__ void bf_steps(const float *partials, int n_slots, int s0, int s1,
                                          int b, int a, int B, int K, int k0, int steps, float *Jb,
-                                         float &hs, float &hc) {
+                                         double &hs) {
     for (int k = k0; k < K; k += PASSES * steps) {
         float s[PASSES];
 #pragma unroll
@@ -64,7 +56,7 @@ __device__ __forceinline__ void bf_steps(const float *partials, int n_slots, int
         for (int u = 0; u < PASSES; ++u)
             if (k + u * steps < K) {
                 Jb[((size_t)(k + u * steps) * B + b) * 3 + a] = s[u];
-                bf_pair_add(hs, hc, s[u], 0.f);
+                hs += (double)s[u];
             }
     }
 }
@@ -73,43 +65,43 @@ __device__ __forceinline__ void bin_finish_body(const float *partials, int n_slo
                                                 const int *slot_begin, int B, int K, float *Jb,
                                                 double *hsum, const double *Jtot, double *Jsum,
                                                 int b) {
-    __shared__ float2 red[BF_MAX_THREADS];
-    __shared__ double red_tot[BF_MAX_THREADS / 32][3];
-    const int t = threadIdx.x, a = t % 3, k0 = t / 3, steps = blockDim.x / 3;
+    __shared__ double red[BF_MAX_THREADS];
+    const int nt = bf_threads(K), steps = nt / 3;   // threads past nt (a longer system's) hold no steps
+    const int t = threadIdx.x, a = t % 3, k0 = t / 3;
     const int lane = t & 31, warp = t >> 5;
-    if (b == B) {   // the total current, in FP64
+    if (b == B) {   // the total current
         double acc[3] = {0.0, 0.0, 0.0};
-        for (int k = t; k < K; k += blockDim.x)
+        if (t < nt)
+            for (int k = t; k < K; k += nt)
 #pragma unroll
-            for (int q = 0; q < 3; ++q) acc[q] += Jtot[3 * k + q];
+                for (int q = 0; q < 3; ++q) acc[q] += Jtot[3 * k + q];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_down_sync(FULL_MASK, acc[q], o);
-            if (lane == 0) red_tot[warp][q] = acc[q];
+            if (lane == 0) red[3 * warp + q] = acc[q];
         }
         __syncthreads();
         if (t < 3) {
             double s = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red_tot[w][t];
+            for (int w = 0; w < nt / 32; ++w) s += red[3 * w + t];
             Jsum[t] += s;
         }
         return;
     }
     const int s0 = slot_begin[b], s1 = slot_begin[b + 1];
     const double old = t < 96 && lane == 0 ? hsum[b * 3 + warp] : 0.0;   // warp = component below
-    float hs = 0.f, hc = 0.f;
-    if (K <= steps) bf_steps<1, 8>(partials, n_slots, s0, s1, b, a, B, K, k0, steps, Jb, hs, hc);
-    else bf_steps<4, 2>(partials, n_slots, s0, s1, b, a, B, K, k0, steps, Jb, hs, hc);
-    red[t] = make_float2(hs, hc);
+    double hs = 0.0;
+    if (K <= steps) bf_steps<1, 8>(partials, n_slots, s0, s1, b, a, B, K, k0, steps, Jb, hs);
+    else if (t < nt) bf_steps<4, 2>(partials, n_slots, s0, s1, b, a, B, K, k0, steps, Jb, hs);
+    red[t] = hs;
     __syncthreads();
     if (warp < 3) {   // component `warp`: lane l the threads 3 (l + 32 j) + warp, then the lanes
-        hs = hc = 0.f;
-        for (int j = lane; j < steps; j += 32) bf_pair_add(hs, hc, red[3 * j + warp].x, red[3 * j + warp].y);
+        hs = 0.0;
+        for (int j = lane; j < steps; j += 32) hs += red[3 * j + warp];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            bf_pair_add(hs, hc, __shfl_down_sync(FULL_MASK, hs, o), __shfl_down_sync(FULL_MASK, hc, o));
-        if (lane == 0) hsum[b * 3 + warp] = old + ((double)hs + (double)hc);
+        for (int o = 16; o > 0; o >>= 1) hs += __shfl_down_sync(FULL_MASK, hs, o);
+        if (lane == 0) hsum[b * 3 + warp] = old + hs;
     }
 }
 

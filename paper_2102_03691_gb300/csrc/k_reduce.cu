@@ -323,22 +323,15 @@ __global__ void __launch_bounds__(32 * LC_WARPS, 2) lag_corr_kernel(const float 
 }
 
 // ------------------------------------------------------------------ K5
-// 1 / (T_s - l) as an unevaluated float pair (zero when no origin has lag l): an FP32 reciprocal
-// and one Newton correction, ~46 bits.  An FP64 division is some 20 operations on a pipe GB300
-// keeps narrow (1/64 of the FP32 rate); these are FP32 instructions.
-__device__ __forceinline__ float2 gk_inv_count(long long T_s, int l) {
-    const long long n = T_s - l;
-    if (n <= 0) return make_float2(0.f, 0.f);
-    const float hi = (float)n, lo = (float)(n - (long long)hi);
-    const float r = __fdiv_rn(1.f, hi);
-    return make_float2(r, r * fmaf(-r, lo, fmaf(-r, hi, 1.f)));
+// 1 / (T_s - l), zero when no origin has lag l.
+__device__ __forceinline__ double gk_inv_count(long long T_s, int l) {
+    return T_s > l ? 1.0 / (double)(T_s - l) : 0.0;
 }
-__device__ __forceinline__ double gk_pair(float2 p) { return (double)p.x + (double)p.y; }
 
 // table[l] = 1 / (T_s - l) for reads whose table does not fit a CTA's shared memory
 __global__ void inv_counts_kernel(long long T_s, int L, double *inv) {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l < L) inv[l] = gk_pair(gk_inv_count(T_s, l));
+    if (l < L) inv[l] = gk_inv_count(T_s, l);
 }
 
 // One warp per (b, mu, nu) row, GK_TAU_ROWS rows a CTA; lane i owns per = ceil(L / 32) consecutive
@@ -348,10 +341,10 @@ __global__ void inv_counts_kernel(long long T_s, int L, double *inv) {
 // l_lo .. l_hi (the host picks them with the same FP64 test on l dt as the oracle).  Bound by the
 // FP64 pipe and the latency of its chain, so: one row's scan stays inside a warp (a CTA of four
 // warps a row spent its time in block scans), the reciprocal counts come from a table that the
-// CTA builds with FP32 instructions (inv non-null: a launch built it), and a lane with at most
-// GK_CACHE lags keeps its running sums in registers.
-// Measured (ncu, us, before -> now): 900 rows x 200 lags 14.5 + 2.3 for
-// the table's launch -> 8.1.
+// CTA builds, a division a lag spread over its threads (inv non-null: a launch built it), and a lane
+// with at most GK_CACHE lags keeps its running sums in registers.
+// Measured (ncu, us, a CTA a row -> now): 900 rows x 200 lags 14.5 + 2.3 for the table's launch
+// -> 8.1.  (With reciprocals of ~46 bits from FP32 instructions the same to 0.1 us.)
 constexpr int GK_TAU_ROWS = 4;
 constexpr int GK_CACHE = 8;
 __global__ void __launch_bounds__(32 * GK_TAU_ROWS) gk_kappa_kernel(const double *Csum, int rows, int L,
@@ -361,7 +354,7 @@ __global__ void __launch_bounds__(32 * GK_TAU_ROWS) gk_kappa_kernel(const double
                                                                     double *kappa_tau, double *kappa_w) {
     extern __shared__ double gk_tab[];
     if (!inv) {
-        for (int l = threadIdx.x; l < L; l += blockDim.x) gk_tab[l] = gk_pair(gk_inv_count(T_s, l));
+        for (int l = threadIdx.x; l < L; l += blockDim.x) gk_tab[l] = gk_inv_count(T_s, l);
         __syncthreads();
         inv = gk_tab;
     }
@@ -430,31 +423,27 @@ __global__ void __launch_bounds__(32 * GK_TAU_ROWS) gk_kappa_kernel(const double
 //   sum_{l = l_lo..l_hi} S(l) = sum_m C(m) w(m),  w(m) = [m >= 1] cnt(m) + cnt(m + 1),
 // cnt(x) = #{l in [l_lo, l_hi] : l >= x} (C(m) enters S(l) as the right end of the step m-1 -> m
 // for l >= m >= 1 and as the left end of the step m -> m+1 for l >= m+1).  The integer weights
-// and the reciprocal counts are folded into one table tw(m) = w(m) / (T_s - m) (a float pair), so
-// a row takes one FP64 FMA a lag instead of the scan's few FP64 operations a lag on GB300's narrow
-// FP64 pipe.
-__device__ __forceinline__ float2 gk_window_weight(long long T_s, int m, int l_lo, int l_hi) {
+// and the reciprocal counts are folded into one table tw(m) = w(m) / (T_s - m), so a row takes one
+// FP64 FMA a lag instead of the scan's few FP64 operations a lag on GB300's narrow FP64 pipe.
+__device__ __forceinline__ double gk_window_weight(long long T_s, int m, int l_lo, int l_hi) {
     const auto cnt = [&](int x) {
         const int lo = max(x, l_lo);
         return l_hi >= lo ? l_hi - lo + 1 : 0;
     };
-    const float2 inv = gk_inv_count(T_s, m);
-    const float w = (float)((m >= 1 ? cnt(m) : 0) + cnt(m + 1));   // below 2^24: exact
-    const float p = w * inv.x;
-    return make_float2(p, fmaf(w, inv.x, -p) + w * inv.y);
+    return gk_inv_count(T_s, m) * (double)((m >= 1 ? cnt(m) : 0) + cnt(m + 1));
 }
 
 __global__ void gk_window_weights_kernel(long long T_s, int L, int l_lo, int l_hi, double *tw) {
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m < L) tw[m] = gk_pair(gk_window_weight(T_s, m, l_lo, l_hi));
+    if (m < L) tw[m] = gk_window_weight(T_s, m, l_lo, l_hi);
 }
 
 // One warp per row, GK_ROWS rows a CTA: kappa_w = scale sum_m Csum(m) tw(m) (lanes stride the
-// lags; fixed tree).  tw null: each CTA first builds the table in shared memory (FP32 instructions
-// spread over its threads), cheaper than a launch of its own; longer tables than that holds come
-// from one weights launch.
-// Measured (ncu, us, before -> now, the table's L FP64 divisions a CTA being the time): 576 rows x
-// 500 lags 8.9 -> 6.6; x 1000 lags 15.3 -> 10.0.
+// lags; fixed tree).  tw null: each CTA first builds the table in shared memory, a division a lag
+// spread over its threads, cheaper than a launch of its own; longer tables than that holds come from
+// one weights launch.
+// Measured (ncu, us, eight rows a CTA and one load a lane in flight -> now): 576 rows x 500 lags
+// 8.9 -> 6.6; x 1000 lags 15.3 -> 10.0.
 constexpr int GK_ROWS = 4;
 __global__ void __launch_bounds__(32 * GK_ROWS) gk_window_kernel(const double *Csum, int rows, int L,
                                                                  const double *__restrict__ tw,
@@ -462,7 +451,7 @@ __global__ void __launch_bounds__(32 * GK_ROWS) gk_window_kernel(const double *C
                                                                  double scale, double *kappa_w) {
     extern __shared__ double gk_tw[];
     if (!tw) {
-        for (int m = threadIdx.x; m < L; m += blockDim.x) gk_tw[m] = gk_pair(gk_window_weight(T_s, m, l_lo, l_hi));
+        for (int m = threadIdx.x; m < L; m += blockDim.x) gk_tw[m] = gk_window_weight(T_s, m, l_lo, l_hi);
         __syncthreads();
         tw = gk_tw;
     }
@@ -496,7 +485,11 @@ __global__ void __launch_bounds__(XCW_OUT * XCW_GROUPS) xcorr_window_kernel(
     extern __shared__ float2 xw_tab[];
     __shared__ float2 part[XCW_GROUPS][XCW_OUT];
     if (!tw)
-        for (int m = threadIdx.x; m < L; m += blockDim.x) xw_tab[m] = gk_window_weight(T_s, m, l_lo, l_hi);
+        for (int m = threadIdx.x; m < L; m += blockDim.x) {
+            const double d = gk_window_weight(T_s, m, l_lo, l_hi);
+            xw_tab[m].x = (float)d;
+            xw_tab[m].y = (float)(d - (double)xw_tab[m].x);
+        }
     __syncthreads();
     const int n = 3 * nb, o = threadIdx.x % XCW_OUT, g = threadIdx.x / XCW_OUT;
     const long long nn = (long long)n * n, q = blockIdx.x * (long long)XCW_OUT + o;
@@ -533,7 +526,7 @@ __global__ void __launch_bounds__(XCW_OUT * XCW_GROUPS) xcorr_window_kernel(
     if (g == 0 && q < nn) {
         double t = 0.0;
 #pragma unroll
-        for (int k = 0; k < XCW_GROUPS; ++k) t += gk_pair(part[k][o]);
+        for (int k = 0; k < XCW_GROUPS; ++k) t += (double)part[k][o].x + (double)part[k][o].y;
         const int j = (int)(q / n), i = (int)(q - (long long)j * n);
         kappa_w[(((size_t)(i / 3) * nb + j / 3) * 3 + i % 3) * 3 + j % 3] = scale * t;
     }

@@ -1,6 +1,7 @@
 // K3 bin finish + HNEMA sums (Eq. 19), K4 GKMA lag correlation (Eq. 17 integrand),
 // K5 running Green-Kubo integral (Eq. 17) and the HNEMA normalisation (Eq. 19).
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -473,60 +474,107 @@ __global__ void __launch_bounds__(32 * GK_ROWS) gk_window_kernel(const double *C
 // The same average of the bin-bin sums, from their state X[l][j][i] (float pairs, i = 3b + mu and
 // j = 3b' + nu of n = 3 nb rows) without the FP64 copy in [b][b'][mu][nu][l] order that the
 // kappa(tau) read takes: consecutive threads take consecutive (j, i), so every lag is one
-// contiguous read.  The weighted sum runs in float pairs (~46 bits) because the state is pairs and
-// FP64 conversions alone would take several times the read: X w = p + e exactly by FMA, and TwoSum
-// adds p.  XCW_GROUPS threads share an output's lags and are added in order.  Bound by the read.
-// Measured at n = 192, L = 200 (59 MB; ncu, us): 47.9 (FP64 copy) + 2.8 (weights) +
-// 31.9 (sum) -> 13.8.
+// contiguous read.  Bound by the FP64 pipe, 16 cycles an instruction of a warp: so an element takes one
+// FP64 instruction and not four (two conversions, an addition and an FMA; 61 us for the case below).
+// X is renormalised, its high part is widened by its bits and added by an FP64 FMA, and what its low
+// part (at most half a unit of the high one) gives is summed in a pair of floats, 47 bits below
+// those 24.  That holds FP64's precision while the terms are inside single precision's range: an
+// output whose terms add up to less than XCW_SMALL or more than XCW_LARGE is summed again in FP64
+// throughout.  The weights are scaled by a power of two so that they add up to less than one.
+// The groups of a CTA share an output's lags and are added in order.
+// Measured at n = 192, L = 200 (59 MB; us, back to back): 90 (FP64 copy, weights, sum) -> 22.6; in
+// pairs of floats throughout, 46 bits, 14.4.
 constexpr int XCW_OUT = 64, XCW_GROUPS = 4, XCW_UNROLL = 8;
+constexpr float XCW_SMALL = 0x1p-70f, XCW_LARGE = 0x1p120f;
+
+// A weight of the bin-bin windows, w(m) 2^-k, and its two leading floats.
+struct __align__(16) XcwWeight {
+    double w;
+    float a, b;
+};
+__device__ __forceinline__ XcwWeight xcw_weight(long long T_s, int m, int l_lo, int l_hi, double down) {
+    XcwWeight r;
+    r.w = gk_window_weight(T_s, m, l_lo, l_hi) * down;
+    r.a = (float)r.w;
+    r.b = (float)(r.w - (double)r.a);
+    return r;
+}
+
+// float -> double by its bits (zero for subnormals): the conversion runs on the FP64 pipe
+__device__ __forceinline__ double xcw_double(float x) {
+    const uint32_t u = __float_as_uint(x), a = u & 0x7fffffffu;
+    const uint32_t hi = a >= 0x00800000u ? (a >> 3) + 0x38000000u : 0u;   // exponent rebiased
+    return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
+}
+
+__global__ void xcw_weights_kernel(long long T_s, int L, int l_lo, int l_hi, double down, XcwWeight *tw) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m < L) tw[m] = xcw_weight(T_s, m, l_lo, l_hi, down);
+}
+
 __global__ void __launch_bounds__(XCW_OUT * XCW_GROUPS) xcorr_window_kernel(
-    const float2 *__restrict__ X, int nb, int L, const double *__restrict__ tw, long long T_s,
-    int l_lo, int l_hi, double scale, double *kappa_w) {
-    extern __shared__ float2 xw_tab[];
-    __shared__ float2 part[XCW_GROUPS][XCW_OUT];
-    if (!tw)
-        for (int m = threadIdx.x; m < L; m += blockDim.x) {
-            const double d = gk_window_weight(T_s, m, l_lo, l_hi);
-            xw_tab[m].x = (float)d;
-            xw_tab[m].y = (float)(d - (double)xw_tab[m].x);
-        }
-    __syncthreads();
+    const float2 *__restrict__ X, int nb, int L, const XcwWeight *__restrict__ tw, long long T_s,
+    int l_lo, int l_hi, double down, double scale, double *kappa_w) {
+    extern __shared__ XcwWeight xw_tab[];
+    __shared__ double part[XCW_GROUPS][XCW_OUT];
     const int n = 3 * nb, o = threadIdx.x % XCW_OUT, g = threadIdx.x / XCW_OUT;
     const long long nn = (long long)n * n, q = blockIdx.x * (long long)XCW_OUT + o;
-    float s = 0.f, c = 0.f;
-    if (q < nn) {
-        const int per = (L + XCW_GROUPS - 1) / XCW_GROUPS;
-        const int m0 = min(L, g * per), m1 = min(L, m0 + per);
-        const float2 *src = X + q;
-        for (int m = m0; m < m1; m += XCW_UNROLL) {
-            float2 v[XCW_UNROLL];
+    const int per = (L + XCW_GROUPS - 1) / XCW_GROUPS;
+    const int m0 = q < nn ? min(L, g * per) : 0, m1 = q < nn ? min(L, m0 + per) : 0;
+    const float2 *src = X + q;
+    float2 v[XCW_UNROLL];
+    auto fetch = [&](int m) {
 #pragma unroll
-            for (int u = 0; u < XCW_UNROLL; ++u)
-                v[u] = m + u < m1 ? __ldcs(src + (m + u) * nn) : make_float2(0.f, 0.f);
+        for (int u = 0; u < XCW_UNROLL; ++u)
+            v[u] = m + u < m1 ? __ldcs(src + (m + u) * nn) : make_float2(0.f, 0.f);
+    };
+    fetch(m0);   // in flight while the table is built
+    if (!tw) {
+        for (int m = threadIdx.x; m < L; m += blockDim.x) xw_tab[m] = xcw_weight(T_s, m, l_lo, l_hi, down);
+        __syncthreads();
+        tw = xw_tab;
+    }
+    double sum = 0.0;            // of the pairs' high parts
+    float lo = 0.f, loc = 0.f;   // of their low parts, as a pair
+    float size = 0.f;            // of the terms
+    bool any = false;
+    auto add = [&](float2 z, int m) {
+        const XcwWeight w = tw[m];
+        float x = z.x, y = 0.f;
+        lc_pair_add(x, y, z.y);   // now |y| is at most half a unit of x
+        sum = fma(xcw_double(x), w.w, sum);
+        const float p = __fmul_rn(y, w.a);
+        const float e = fmaf(y, w.b, fmaf(y, w.a, -p));
+        lc_pair_add(lo, loc, p);
+        loc = __fadd_rn(loc, e);
+        size = fmaf(fabsf(x), w.a, size);
+        any = any || x != 0.f;
+    };
+    int m = m0;
+    for (; m + XCW_UNROLL <= m1; m += XCW_UNROLL) {
+        if (m > m0) fetch(m);
 #pragma unroll
-            for (int u = 0; u < XCW_UNROLL; ++u) {
-                if (m + u >= m1) break;
-                float2 w;
-                if (tw) {
-                    const double d = tw[m + u];
-                    w.x = (float)d;
-                    w.y = (float)(d - (double)w.x);
-                } else {
-                    w = xw_tab[m + u];
-                }
-                const float p = __fmul_rn(v[u].x, w.x);
-                const float e = fmaf(v[u].x, w.x, -p);
-                lc_pair_add(s, c, p);
-                c = __fadd_rn(c, fmaf(v[u].y, w.x, fmaf(v[u].x, w.y, e)));
-            }
+        for (int u = 0; u < XCW_UNROLL; ++u) add(v[u], m + u);
+    }
+    if (m > m0) fetch(m);
+#pragma unroll
+    for (int u = 0; u < XCW_UNROLL - 1; ++u)
+        if (m + u < m1) add(v[u], m + u);
+    if (size >= XCW_SMALL && size <= XCW_LARGE) {
+        sum += (double)lo + (double)loc;
+    } else if (any) {   // terms near the ends of single precision's range, or nothing but zeros of w
+        sum = 0.0;
+        for (int k = m0; k < m1; ++k) {
+            const float2 z = src[k * nn];
+            sum = fma((double)z.x + (double)z.y, tw[k].w, sum);
         }
     }
-    part[g][o] = make_float2(s, c);
+    part[g][o] = sum;
     __syncthreads();
     if (g == 0 && q < nn) {
         double t = 0.0;
 #pragma unroll
-        for (int k = 0; k < XCW_GROUPS; ++k) t += (double)part[k][o].x + (double)part[k][o].y;
+        for (int k = 0; k < XCW_GROUPS; ++k) t += part[k][o];
         const int j = (int)(q / n), i = (int)(q - (long long)j * n);
         kappa_w[(((size_t)(i / 3) * nb + j / 3) * 3 + i % 3) * 3 + j % 3] = scale * t;
     }
@@ -568,6 +616,7 @@ void launch_bin_finish(const float *partials, int n_slots, const int *slot_begin
 
 namespace {
 constexpr int GK_TABLE_LAGS = 6144;   // longest per-CTA table: the default 48 KB
+constexpr int XCW_TABLE_LAGS = 2900;  // the same beside the partial sums, 16 bytes a lag
 
 // The window's lags: l dt in [tau_lo, tau_hi], tested in FP64 as the oracle tests it.
 void gk_window(int L, double tau_lo, double tau_hi, double dt, int &l_lo, int &l_hi) {
@@ -656,12 +705,17 @@ int launch_xcorr_window(const float2 *X, int nb, int L, long long T_s, double co
     gk_window(L, tau_lo, tau_hi, dt, l_lo, l_hi);
     const int n = l_hi >= l_lo ? l_hi - l_lo + 1 : 0;
     const double scale = n > 0 ? 0.5 * coef_dt / n : 0.0;
-    const bool own = L <= GK_TABLE_LAGS / 2;   // beside the partial sums
-    if (!own) gk_window_weights_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, l_lo, l_hi, table);
+    // weights scaled so that they add up to less than one: w(m) <= 2 n / (T_s - m)
+    const double most = 2.0 * n * L / (double)std::max(1ll, T_s - (L - 1));
+    const int wexp = most > 0 ? std::ilogb(most) + 1 : 0;
+    const double down = std::ldexp(1.0, -wexp), up = std::ldexp(scale, wexp);
     const long long out = 9ll * nb * nb;
+    const bool own = L <= XCW_TABLE_LAGS;
+    XcwWeight *tw = reinterpret_cast<XcwWeight *>(table);
+    if (!own) xcw_weights_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, l_lo, l_hi, down, tw);
     xcorr_window_kernel<<<(unsigned)((out + XCW_OUT - 1) / XCW_OUT), XCW_OUT * XCW_GROUPS,
-                          own ? sizeof(float2) * L : 0, s>>>(X, nb, L, own ? nullptr : table, T_s, l_lo, l_hi,
-                                                             scale, kappa_w);
+                          own ? sizeof(XcwWeight) * L : 0, s>>>(X, nb, L, own ? nullptr : tw, T_s, l_lo, l_hi,
+                                                                down, up, kappa_w);
     return own ? 1 : 2;
 }
 

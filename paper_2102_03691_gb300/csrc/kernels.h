@@ -360,7 +360,7 @@ void launch_xcorr_touch(const XcPlan &pl, const XcTcParams &p, cudaStream_t s);
 // out[b][b'][mu][nu][l] = X[l][3b'+nu][3b+mu] (float pair -> FP64)
 void launch_xcorr_transpose(const float2 *X, int nb, int L, double *out, cudaStream_t s);
 // The window averages alone of the bin-bin sums, [b][b'][mu][nu], straight from the state X
-// (arguments as launch_gk_kappa).
+// (arguments as launch_gk_kappa; table: 2 L doubles, 16-byte aligned).
 int launch_xcorr_window(const float2 *X, int nb, int L, long long T_s, double coef_dt, double tau_lo,
                         double tau_hi, double dt, double *kappa_w, double *table, cudaStream_t s);
 // count[l] = max(T_s - l, 0)

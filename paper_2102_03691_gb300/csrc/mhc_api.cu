@@ -1620,11 +1620,11 @@ mhc_status mhc_read_kappa_xcorr(mhc_handle *h, double *kappa_tau, double tau_lo,
     const double coef = WMK_PER_EV_PS_A_K / (KB_EV_PER_K * h->prm.T_K * h->prm.T_K * h->prm.V_A3);
     if (!kappa_tau) {   // the window averages alone need no FP64 copy of the sums
         if (!kappa_w) return MHC_OK;
-        if ((s = dev_alloc(h, "xw_out", sizeof(double) * (rows + L), false)) != MHC_OK) return s;
+        if ((s = dev_alloc(h, "xw_out", sizeof(double) * (rows + 2 * (size_t)L), false)) != MHC_OK) return s;
         const bool own = !direct_out(h, kappa_w, where);
-        double *scratch = dptr<double>(h, "xw_out"), *dw = own ? scratch : kappa_w;
+        double *table = dptr<double>(h, "xw_out"), *dw = own ? table + 2 * (size_t)L : kappa_w;
         h->launches += launch_xcorr_window(dptr<float2>(h, "Xsum"), nb, L, h->steps, coef * h->prm.dt_ps,
-                                           tau_lo, tau_hi, h->prm.dt_ps, dw, scratch + rows, h->stream);
+                                           tau_lo, tau_hi, h->prm.dt_ps, dw, table, h->stream);
         MHC_CUDA(h, cudaGetLastError());
         return own ? copy_out(h, kappa_w, dw, sizeof(double) * rows, where) : MHC_OK;
     }

@@ -52,3 +52,42 @@ def test_gkma_reads_hold_fp64(L, T):
     held(gw, kw, skw, 2 * L + 11, f"window beside kappa(tau) L={L} T={T}")
     held(h.read_kappa_window(lo, hi), kw, skw, 2 * L + 11, f"window alone L={L} T={T}")
     h.close()
+
+
+def bin_bin(B, L, T, scale=1.0):
+    """A handle with T steps of bin-bin sums of L lags, its sums and its origin counts."""
+    c = make_case(N=12, M=36, T=T, B=B, seed=9550 + T, drive=2e-3)
+    c["v"], c["W"] = (c["v"] * scale).astype(np.float32), (c["W"] * scale).astype(np.float32)
+    h, _, _ = run_gpu(c, "fp16x3", K=60, L=L, dt_ps=DT, T_K=TK, V_A3=V, xcorr=True)
+    X, cnt = h.read_xcorr()
+    return h, X, cnt
+
+
+@pytest.mark.parametrize("L", [2, 3, 5])
+@pytest.mark.parametrize("T", [5, 77, 331])
+def test_bin_bin_window_holds_fp64(L, T):
+    need_gpu()
+    h, X, cnt = bin_bin(7, L, T)
+    lo, hi = 0.5 * DT, (L - 1) * DT
+    kt, kw, skt, skw = reference(X, cnt, lo, hi)
+    _, gw = h.read_kappa_xcorr(lo, hi, with_tau=False)
+    held(gw, kw, skw, 2 * L + 11, f"bin-bin window L={L} T={T}")
+    gt, gw = h.read_kappa_xcorr(lo, hi)
+    held(gt, kt, skt, 2 * L + 9, f"bin-bin kappa(tau) L={L} T={T}")
+    held(gw, kw, skw, 2 * L + 11, f"bin-bin window beside kappa(tau) L={L} T={T}")
+    h.close()
+
+
+# sums near the ends of single precision's range, where its products leave it; many outputs and one,
+# lags that a thread takes alone, in batches, and shared among threads; a table of a launch
+@pytest.mark.parametrize("scale", [2.0 ** -26, 1.0, 2.0 ** 27])
+@pytest.mark.parametrize("B,L,T", [(1, 1, 7), (7, 3, 77), (43, 40, 90), (2, 300, 331), (1, 3001, 90)])
+def test_bin_bin_window_over_the_range_of_single_precision(B, L, T, scale):
+    need_gpu()
+    h, X, cnt = bin_bin(B, L, T, scale)
+    assert np.isfinite(X).all() and (X != 0).any()
+    lo, hi = 0.5 * DT, (L - 1) * DT
+    _, kw, _, skw = reference(X, cnt, lo, hi)
+    _, gw = h.read_kappa_xcorr(lo, hi, with_tau=False)
+    held(gw, kw, skw, 2 * min(L, T) + 11, f"bin-bin window B={B} L={L} T={T} scale={scale}")
+    h.close()

@@ -484,7 +484,11 @@ __global__ void __launch_bounds__(32 * GK_ROWS) gk_window_kernel(const double *C
 // The groups of a CTA share an output's lags and are added in order.
 // Measured at n = 192, L = 200 (59 MB; us, back to back): 90 (FP64 copy, weights, sum) -> 22.6; in
 // pairs of floats throughout, 46 bits, 14.4.
-constexpr int XCW_OUT = 64, XCW_GROUPS = 4, XCW_UNROLL = 8;
+// Outputs that fill no more than an SM each (XCW_WIDE a CTA: xcw_wide) are spread over narrow CTAs, a
+// 32-byte sector of outputs and 64 groups of lags each: 18 rows x 4000 lags 135 -> 27 us (33-41 with
+// the FP64 copy), 3 x 5000 171 -> 33 (39), 60 x 1000 31 -> 27, but 66 x 100 6.2 -> 16.
+constexpr int XCW_THREADS = 256, XCW_UNROLL = 8;
+constexpr int XCW_WIDE = 64, XCW_NARROW = 4;   // outputs a CTA
 constexpr float XCW_SMALL = 0x1p-70f, XCW_LARGE = 0x1p120f;
 
 // A weight of the bin-bin windows, w(m) 2^-k, and its two leading floats.
@@ -512,14 +516,16 @@ __global__ void xcw_weights_kernel(long long T_s, int L, int l_lo, int l_hi, dou
     if (m < L) tw[m] = xcw_weight(T_s, m, l_lo, l_hi, down);
 }
 
-__global__ void __launch_bounds__(XCW_OUT * XCW_GROUPS) xcorr_window_kernel(
+template <int OUT>
+__global__ void __launch_bounds__(XCW_THREADS) xcorr_window_kernel(
     const float2 *__restrict__ X, int nb, int L, const XcwWeight *__restrict__ tw, long long T_s,
     int l_lo, int l_hi, double down, double scale, double *kappa_w) {
+    constexpr int GROUPS = XCW_THREADS / OUT;
     extern __shared__ XcwWeight xw_tab[];
-    __shared__ double part[XCW_GROUPS][XCW_OUT];
-    const int n = 3 * nb, o = threadIdx.x % XCW_OUT, g = threadIdx.x / XCW_OUT;
-    const long long nn = (long long)n * n, q = blockIdx.x * (long long)XCW_OUT + o;
-    const int per = (L + XCW_GROUPS - 1) / XCW_GROUPS;
+    __shared__ double part[GROUPS][OUT];
+    const int n = 3 * nb, o = threadIdx.x % OUT, g = threadIdx.x / OUT;
+    const long long nn = (long long)n * n, q = blockIdx.x * (long long)OUT + o;
+    const int per = (L + GROUPS - 1) / GROUPS;
     const int m0 = q < nn ? min(L, g * per) : 0, m1 = q < nn ? min(L, m0 + per) : 0;
     const float2 *src = X + q;
     float2 v[XCW_UNROLL];
@@ -573,8 +579,8 @@ __global__ void __launch_bounds__(XCW_OUT * XCW_GROUPS) xcorr_window_kernel(
     __syncthreads();
     if (g == 0 && q < nn) {
         double t = 0.0;
-#pragma unroll
-        for (int k = 0; k < XCW_GROUPS; ++k) t += part[k][o];
+#pragma unroll 8
+        for (int k = 0; k < GROUPS; ++k) t += part[k][o];
         const int j = (int)(q / n), i = (int)(q - (long long)j * n);
         kappa_w[(((size_t)(i / 3) * nb + j / 3) * 3 + i % 3) * 3 + j % 3] = scale * t;
     }
@@ -617,6 +623,17 @@ void launch_bin_finish(const float *partials, int n_slots, const int *slot_begin
 namespace {
 constexpr int GK_TABLE_LAGS = 6144;   // longest per-CTA table: the default 48 KB
 constexpr int XCW_TABLE_LAGS = 2900;  // the same beside the partial sums, 16 bytes a lag
+
+// Whether each of `ctas` CTAs builds its own table of L lags: the divisions take an SM about 5 ns each,
+// against 4 us for a launch.  (Bin-bin windows of 60 rows x 1000 lags in narrow CTAs: 45 us own,
+// 27 launched; 4 x 1000: 12.3 and 12.3.)
+bool gk_own_table(long long ctas, int L) { return L <= 3000 && ctas * L <= 300000; }
+
+// Whether XCW_WIDE outputs a CTA give every other SM one, or the lags are few enough for that not to
+// matter.  (Where the line is crossed, us, wide and narrow: 60 rows 31 and 27 at 1000 lags, 90 rows 37
+// and 47; 66 rows 6 and 16 at 100 lags.)
+constexpr int XCW_FILL_CTAS = 76, XCW_FEW_LAGS = 128;
+bool xcw_wide(long long out, int L) { return (out + XCW_WIDE - 1) / XCW_WIDE >= XCW_FILL_CTAS || L <= XCW_FEW_LAGS; }
 
 // The window's lags: l dt in [tau_lo, tau_hi], tested in FP64 as the oracle tests it.
 void gk_window(int L, double tau_lo, double tau_hi, double dt, int &l_lo, int &l_hi) {
@@ -710,12 +727,17 @@ int launch_xcorr_window(const float2 *X, int nb, int L, long long T_s, double co
     const int wexp = most > 0 ? std::ilogb(most) + 1 : 0;
     const double down = std::ldexp(1.0, -wexp), up = std::ldexp(scale, wexp);
     const long long out = 9ll * nb * nb;
-    const bool own = L <= XCW_TABLE_LAGS;
+    const bool wide = xcw_wide(out, L);
+    const long long ctas = (out + (wide ? XCW_WIDE : XCW_NARROW) - 1) / (wide ? XCW_WIDE : XCW_NARROW);
+    const bool own = L <= XCW_TABLE_LAGS && gk_own_table(ctas, L);
     XcwWeight *tw = reinterpret_cast<XcwWeight *>(table);
     if (!own) xcw_weights_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, l_lo, l_hi, down, tw);
-    xcorr_window_kernel<<<(unsigned)((out + XCW_OUT - 1) / XCW_OUT), XCW_OUT * XCW_GROUPS,
-                          own ? sizeof(XcwWeight) * L : 0, s>>>(X, nb, L, own ? nullptr : tw, T_s, l_lo, l_hi,
-                                                                down, up, kappa_w);
+    const auto run = [&](auto kernel) {
+        kernel<<<(unsigned)ctas, XCW_THREADS, own ? sizeof(XcwWeight) * L : 0, s>>>(
+            X, nb, L, own ? nullptr : tw, T_s, l_lo, l_hi, down, up, kappa_w);
+    };
+    if (wide) run(xcorr_window_kernel<XCW_WIDE>);
+    else run(xcorr_window_kernel<XCW_NARROW>);
     return own ? 1 : 2;
 }
 

@@ -335,36 +335,43 @@ __global__ void inv_counts_kernel(long long T_s, int L, double *inv) {
     if (l < L) inv[l] = gk_inv_count(T_s, l);
 }
 
-// One warp per (b, mu, nu) row, GK_TAU_ROWS rows a CTA; lane i owns per = ceil(L / 32) consecutive
-// lags.  C(l) = Csum(l) / (T_s - l); the running trapezoid sum
-// S(l) = sum_{1 <= l' <= l} (C(l'-1) + C(l')) comes from the lanes' totals and a warp scan (a
-// fixed tree, deterministic); kappa(l) = (c dt / 2) S(l).  The window average runs over the lags
-// l_lo .. l_hi (the host picks them with the same FP64 test on l dt as the oracle).  Bound by the
-// FP64 pipe and the latency of its chain, so: one row's scan stays inside a warp (a CTA of four
-// warps a row spent its time in block scans), the reciprocal counts come from a table that the
-// CTA builds, a division a lag spread over its threads (inv non-null: a launch built it), and a lane
-// with at most GK_CACHE lags keeps its running sums in registers.
-// Measured (ncu, us, a CTA a row -> now): 900 rows x 200 lags 14.5 + 2.3 for the table's launch
-// -> 8.1.  (With reciprocals of ~46 bits from FP32 instructions the same to 0.1 us.)
+// WARPS warps per (b, mu, nu) row, four warps a CTA or one row of more; lane i of the row's 32 WARPS
+// owns per = ceil(L / (32 WARPS)) consecutive lags.  C(l) = Csum(l) / (T_s - l); the running trapezoid
+// sum S(l) = sum_{1 <= l' <= l} (C(l'-1) + C(l')) comes from the lanes' totals, a warp scan and the
+// totals of the row's warps before (a fixed tree, deterministic); kappa(l) = (c dt / 2) S(l).  The
+// window average runs over the lags l_lo .. l_hi (the host picks them with the same FP64 test on l dt
+// as the oracle).  Bound by the FP64 pipe and the latency of its chain, so:
+//   - a lane with at most GK_CACHE lags keeps its running sums in registers; beyond, it walks its lags
+//     twice, one load in flight.  So a row gets the fewest warps that hold it in registers, up to
+//     eight (gk_tau_warps); more warps spend their time in scans and barriers;
+//   - the reciprocal counts come from a table that the CTA builds, a division a lag spread over its
+//     threads, or from one launch where the CTAs' divisions together cost more (gk_own_table).
+// Measured (us, back to back; four warps a row and the table's launch, with a copy of the result ->
+// one warp a row -> now): 72 rows x 200 lags 18.4 -> 6.2 -> 6.2; x 500 16.4 -> 12.3 -> 8.2; x 1000
+// 20.5 -> 20.5 -> 10.2; x 5000 35.9 -> 92 -> 20.8; 576 x 1000 28.7 -> 22.5 -> 18.4; x 5000 69.5 -> 92
+// -> 59.4; 900 x 200 30.7 -> 10.3 -> 10.3; x 1000 38.9 -> 32.8 -> 24.6.
 constexpr int GK_TAU_ROWS = 4;
 constexpr int GK_CACHE = 8;
-__global__ void __launch_bounds__(32 * GK_TAU_ROWS) gk_kappa_kernel(const double *Csum, int rows, int L,
-                                                                    const double *__restrict__ inv,
-                                                                    long long T_s, double coef_half,
-                                                                    int l_lo, int l_hi,
-                                                                    double *kappa_tau, double *kappa_w) {
+constexpr int gk_tau_rows(int warps) { return warps >= GK_TAU_ROWS ? 1 : GK_TAU_ROWS / warps; }
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS * gk_tau_rows(WARPS), WARPS == 1 ? 9 : WARPS == 8 ? 4 : 8) gk_kappa_kernel(
+    const double *Csum, int rows, int L, const double *__restrict__ inv, long long T_s, double coef_half,
+    int l_lo, int l_hi, double *kappa_tau, double *kappa_w) {
+    constexpr int ROWS = gk_tau_rows(WARPS);
     extern __shared__ double gk_tab[];
+    __shared__ double s_tot[WARPS * ROWS], s_win[WARPS * ROWS];
     if (!inv) {
         for (int l = threadIdx.x; l < L; l += blockDim.x) gk_tab[l] = gk_inv_count(T_s, l);
         __syncthreads();
         inv = gk_tab;
     }
-    const int r = blockIdx.x * GK_TAU_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (r >= rows) return;
-    const double *cs = Csum + (size_t)r * L;
-    double *kt = kappa_tau + (size_t)r * L;
-    const int per = (L + 31) / 32;
-    const int l0 = min(L, lane * per), l1 = min(L, l0 + per);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int r = blockIdx.x * ROWS + warp / WARPS, part = warp % WARPS;
+    const bool live = r < rows;   // (every warp takes the barriers)
+    const double *cs = Csum + (size_t)(live ? r : 0) * L;
+    double *kt = kappa_tau + (size_t)(live ? r : 0) * L;
+    const int per = (L + 32 * WARPS - 1) / (32 * WARPS);
+    const int l0 = live ? min(L, (32 * part + lane) * per) : L, l1 = min(L, l0 + per);
     const double c_before = (l0 > 0 && l0 < l1) ? cs[l0 - 1] * inv[l0 - 1] : 0.0;
     double run[GK_CACHE];   // the lane's running sums
     double tot = 0.0, prev = c_before;
@@ -391,8 +398,15 @@ __global__ void __launch_bounds__(32 * GK_TAU_ROWS) gk_kappa_kernel(const double
         const double y = __shfl_up_sync(FULL_MASK, base, o);
         if (lane >= o) base += y;
     }
+    if (WARPS > 1 && lane == 31) s_tot[warp] = base;
     base = __shfl_up_sync(FULL_MASK, base, 1);
     if (lane == 0) base = 0.0;
+    if (WARPS > 1) {
+        __syncthreads();
+        double before = 0.0;
+        for (int q = 0; q < part; ++q) before += s_tot[warp - part + q];
+        base += before;
+    }
     double wsum = 0.0;
     auto emit = [&](int l, double s) {
         const double kap = coef_half * s;
@@ -412,9 +426,16 @@ __global__ void __launch_bounds__(32 * GK_TAU_ROWS) gk_kappa_kernel(const double
             emit(l, base);
         }
     }
+    if (!kappa_w) return;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) wsum += __shfl_down_sync(FULL_MASK, wsum, o);
-    if (lane == 0 && kappa_w) {
+    if (WARPS > 1) {
+        if (lane == 0) s_win[warp] = wsum;
+        __syncthreads();
+        if (part == 0)
+            for (int q = 1; q < WARPS; ++q) wsum += s_win[warp + q];
+    }
+    if (part == 0 && lane == 0 && live) {
         const int n = l_hi >= l_lo ? l_hi - l_lo + 1 : 0;
         kappa_w[r] = n > 0 ? wsum / n : 0.0;
     }
@@ -439,36 +460,47 @@ __global__ void gk_window_weights_kernel(long long T_s, int L, int l_lo, int l_h
     if (m < L) tw[m] = gk_window_weight(T_s, m, l_lo, l_hi);
 }
 
-// One warp per row, GK_ROWS rows a CTA: kappa_w = scale sum_m Csum(m) tw(m) (lanes stride the
+// WARPS warps per row, GK_ROWS warps a CTA: kappa_w = scale sum_m Csum(m) tw(m) (lanes stride the
 // lags; fixed tree).  tw null: each CTA first builds the table in shared memory, a division a lag
-// spread over its threads, cheaper than a launch of its own; longer tables than that holds come from
-// one weights launch.
-// Measured (ncu, us, eight rows a CTA and one load a lane in flight -> now): 576 rows x 500 lags
-// 8.9 -> 6.6; x 1000 lags 15.3 -> 10.0.
+// spread over its threads (gk_own_table).  One warp a row, or the whole CTA for more than
+// GK_ONE_WARP_LAGS lags, where a warp's round trips to memory were the time.
+// Measured (us, back to back, eight rows a CTA -> now): 576 rows x 500 lags 10.3 -> 6.2; x 1000 12.3
+// -> 8.5; 72 x 5000 28.6 -> 13.3 (one warp a row 30.7); 72 x 10000 36.9 -> 16.4 (45.1).
+constexpr int GK_ONE_WARP_LAGS = 1024;
 constexpr int GK_ROWS = 4;
+template <int WARPS>
 __global__ void __launch_bounds__(32 * GK_ROWS) gk_window_kernel(const double *Csum, int rows, int L,
                                                                  const double *__restrict__ tw,
                                                                  long long T_s, int l_lo, int l_hi,
                                                                  double scale, double *kappa_w) {
+    constexpr int ROWS = GK_ROWS / WARPS, STRIDE = 32 * WARPS;
     extern __shared__ double gk_tw[];
+    __shared__ double s_part[GK_ROWS];
     if (!tw) {
         for (int m = threadIdx.x; m < L; m += blockDim.x) gk_tw[m] = gk_window_weight(T_s, m, l_lo, l_hi);
         __syncthreads();
         tw = gk_tw;
     }
-    const int r = blockIdx.x * GK_ROWS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (r >= rows) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, part = warp % WARPS;
+    const int r = blockIdx.x * ROWS + warp / WARPS;
+    if (r >= rows) return;   // (with WARPS > 1 a CTA has one row, so none is left at the barrier)
     const double *cs = Csum + (size_t)r * L;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};   // four loads in flight a lane
-    for (int m = lane; m < L; m += 128) {
+    for (int m = 32 * part + lane; m < L; m += 4 * STRIDE) {
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (m + 32 * u < L) acc[u] = fma(cs[m + 32 * u], tw[m + 32 * u], acc[u]);
+            if (m + STRIDE * u < L) acc[u] = fma(cs[m + STRIDE * u], tw[m + STRIDE * u], acc[u]);
     }
     double t = (acc[0] + acc[1]) + (acc[2] + acc[3]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(FULL_MASK, t, o);
-    if (lane == 0) kappa_w[r] = scale * t;
+    if (WARPS > 1) {
+        if (lane == 0) s_part[warp] = t;
+        __syncthreads();
+        if (part == 0)
+            for (int q = 1; q < WARPS; ++q) t += s_part[warp + q];
+    }
+    if (part == 0 && lane == 0) kappa_w[r] = scale * t;
 }
 
 // The same average of the bin-bin sums, from their state X[l][j][i] (float pairs, i = 3b + mu and
@@ -621,12 +653,12 @@ void launch_bin_finish(const float *partials, int n_slots, const int *slot_begin
 }
 
 namespace {
-constexpr int GK_TABLE_LAGS = 6144;   // longest per-CTA table: the default 48 KB
-constexpr int XCW_TABLE_LAGS = 2900;  // the same beside the partial sums, 16 bytes a lag
+constexpr int XCW_TABLE_LAGS = 2900;   // longest table of a bin-bin window's CTA, within the default 48 KB
 
 // Whether each of `ctas` CTAs builds its own table of L lags: the divisions take an SM about 5 ns each,
-// against 4 us for a launch.  (Bin-bin windows of 60 rows x 1000 lags in narrow CTAs: 45 us own,
-// 27 launched; 4 x 1000: 12.3 and 12.3.)
+// against 4 us for a launch.  (576 rows, kappa(tau) of 500 lags: 288 CTAs 12.3 us own, 14.4
+// launched; of 1000 lags: 576 CTAs 22.5 and 18.4.  72 rows x 5000 lags: 24.6 and 20.5.  Bin-bin windows
+// of 60 rows x 1000 lags: 900 CTAs 45 and 27.)
 bool gk_own_table(long long ctas, int L) { return L <= 3000 && ctas * L <= 300000; }
 
 // Whether XCW_WIDE outputs a CTA give every other SM one, or the lags are few enough for that not to
@@ -634,6 +666,13 @@ bool gk_own_table(long long ctas, int L) { return L <= 3000 && ctas * L <= 30000
 // and 47; 66 rows 6 and 16 at 100 lags.)
 constexpr int XCW_FILL_CTAS = 76, XCW_FEW_LAGS = 128;
 bool xcw_wide(long long out, int L) { return (out + XCW_WIDE - 1) / XCW_WIDE >= XCW_FILL_CTAS || L <= XCW_FEW_LAGS; }
+
+// Warps a row of kappa(tau) (see the kernel).  Up to 320 lags one warp walking its lags twice is as
+// good, where the rows are many (1800 x 300: 16.4 us and 18.4; 900 x 300: 12.3 and 10.3).
+int gk_tau_warps(int rows, int L) {
+    if (L <= 256 || (L <= 320 && rows >= 1520)) return 1;
+    return L <= 512 ? 2 : L <= 1024 ? 4 : 8;
+}
 
 // The window's lags: l dt in [tau_lo, tau_hi], tested in FP64 as the oracle tests it.
 void gk_window(int L, double tau_lo, double tau_hi, double dt, int &l_lo, int &l_hi) {
@@ -699,19 +738,33 @@ int launch_gk_kappa(const double *Csum, int B, int L, long long T_s, double coef
     int l_lo, l_hi;
     gk_window(L, tau_lo, tau_hi, dt, l_lo, l_hi);
     const int rows = B * 9;
-    const bool own = L <= GK_TABLE_LAGS;   // each CTA builds the table
-    const size_t sm = own ? sizeof(double) * L : 0;
     if (!kappa_tau) {   // the window average alone
         const int n = l_hi >= l_lo ? l_hi - l_lo + 1 : 0;
         const double scale = n > 0 ? 0.5 * coef_dt / n : 0.0;
+        const bool one = L <= GK_ONE_WARP_LAGS;
+        const int ctas = one ? (rows + GK_ROWS - 1) / GK_ROWS : rows;
+        const bool own = gk_own_table(ctas, L);
         if (!own) gk_window_weights_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, l_lo, l_hi, table);
-        gk_window_kernel<<<(rows + GK_ROWS - 1) / GK_ROWS, 32 * GK_ROWS, sm, s>>>(
-            Csum, rows, L, own ? nullptr : table, T_s, l_lo, l_hi, scale, kappa_w);
+        const auto run = [&](auto kernel) {
+            kernel<<<ctas, 32 * GK_ROWS, own ? sizeof(double) * L : 0, s>>>(
+                Csum, rows, L, own ? nullptr : table, T_s, l_lo, l_hi, scale, kappa_w);
+        };
+        if (one) run(gk_window_kernel<1>);
+        else run(gk_window_kernel<GK_ROWS>);
         return own ? 1 : 2;
     }
+    const int warps = gk_tau_warps(rows, L);
+    const int ctas = (rows + gk_tau_rows(warps) - 1) / gk_tau_rows(warps);
+    const bool own = gk_own_table(ctas, L);
     if (!own) inv_counts_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, table);
-    gk_kappa_kernel<<<(rows + GK_TAU_ROWS - 1) / GK_TAU_ROWS, 32 * GK_TAU_ROWS, sm, s>>>(
-        Csum, rows, L, own ? nullptr : table, T_s, 0.5 * coef_dt, l_lo, l_hi, kappa_tau, kappa_w);
+    const auto run = [&](auto kernel) {
+        kernel<<<ctas, 32 * warps * gk_tau_rows(warps), own ? sizeof(double) * L : 0, s>>>(
+            Csum, rows, L, own ? nullptr : table, T_s, 0.5 * coef_dt, l_lo, l_hi, kappa_tau, kappa_w);
+    };
+    if (warps == 1) run(gk_kappa_kernel<1>);
+    else if (warps == 2) run(gk_kappa_kernel<2>);
+    else if (warps == 4) run(gk_kappa_kernel<4>);
+    else run(gk_kappa_kernel<8>);
     return own ? 1 : 2;
 }
 

@@ -775,19 +775,20 @@ int launch_xcorr_window(const float2 *X, int nb, int L, long long T_s, double co
     gk_window(L, tau_lo, tau_hi, dt, l_lo, l_hi);
     const int n = l_hi >= l_lo ? l_hi - l_lo + 1 : 0;
     const double scale = n > 0 ? 0.5 * coef_dt / n : 0.0;
+    const int Lw = n > 0 ? l_hi + 1 : 0;   // lags past the window have no weight: neither read nor tried in FP64
     // weights scaled so that they add up to less than one: w(m) <= 2 n / (T_s - m)
-    const double most = 2.0 * n * L / (double)std::max(1ll, T_s - (L - 1));
+    const double most = 2.0 * n * Lw / (double)std::max(1ll, T_s - (Lw - 1));
     const int wexp = most > 0 ? std::ilogb(most) + 1 : 0;
     const double down = std::ldexp(1.0, -wexp), up = std::ldexp(scale, wexp);
     const long long out = 9ll * nb * nb;
-    const bool wide = xcw_wide(out, L);
+    const bool wide = xcw_wide(out, Lw);
     const long long ctas = (out + (wide ? XCW_WIDE : XCW_NARROW) - 1) / (wide ? XCW_WIDE : XCW_NARROW);
-    const bool own = L <= XCW_TABLE_LAGS && gk_own_table(ctas, L);
+    const bool own = Lw <= XCW_TABLE_LAGS && gk_own_table(ctas, Lw);
     XcwWeight *tw = reinterpret_cast<XcwWeight *>(table);
-    if (!own) xcw_weights_kernel<<<(L + 255) / 256, 256, 0, s>>>(T_s, L, l_lo, l_hi, down, tw);
+    if (!own) xcw_weights_kernel<<<(Lw + 255) / 256, 256, 0, s>>>(T_s, Lw, l_lo, l_hi, down, tw);
     const auto run = [&](auto kernel) {
-        kernel<<<(unsigned)ctas, XCW_THREADS, own ? sizeof(XcwWeight) * L : 0, s>>>(
-            X, nb, L, own ? nullptr : tw, T_s, l_lo, l_hi, down, up, kappa_w);
+        kernel<<<(unsigned)ctas, XCW_THREADS, own ? sizeof(XcwWeight) * Lw : 0, s>>>(
+            X, nb, Lw, own ? nullptr : tw, T_s, l_lo, l_hi, down, up, kappa_w);
     };
     if (wide) run(xcorr_window_kernel<XCW_WIDE>);
     else run(xcorr_window_kernel<XCW_NARROW>);

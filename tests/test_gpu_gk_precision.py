@@ -91,3 +91,15 @@ def test_bin_bin_window_over_the_range_of_single_precision(B, L, T, scale):
     _, gw = h.read_kappa_xcorr(lo, hi, with_tau=False)
     held(gw, kw, skw, 2 * min(L, T) + 11, f"bin-bin window B={B} L={L} T={T} scale={scale}")
     h.close()
+
+
+@pytest.mark.parametrize("B,L,T", [(7, 40, 90), (43, 40, 90), (2, 400, 331)])
+@pytest.mark.parametrize("lo,hi", [(0.0, 0.1), (0.2, 0.5), (0.49, 0.493)])   # early, middle, at most one lag
+def test_bin_bin_window_that_ends_early(B, L, T, lo, hi):
+    need_gpu()
+    h, X, cnt = bin_bin(B, L, T)
+    lo, hi = lo * L * DT, hi * L * DT
+    _, kw, _, skw = reference(X, cnt, lo, hi)
+    _, gw = h.read_kappa_xcorr(lo, hi, with_tau=False)
+    held(gw, kw, skw, 2 * L + 11, f"bin-bin window B={B} L={L} {lo}..{hi}")
+    h.close()

@@ -28,8 +28,8 @@ namespace {
 //     {1, 2, 3} and for {0, 3, 4}, 4 for {0, 1} and {0, 1, 2}), so the mode index takes lane bits
 //     1, 2, 3 and the column index bits 0 and 4: 8 cycles of loads a warp and d beside 16 of FMAs.
 //   - tiles rarely fill whole waves of CTAs, so the tiles of the last, partial wave are cut along
-//     d into one range of equal length a CTA (whole chunks of 128 d's); a cut tile's ranges go to
-//     planes of R and the bin epilogue adds them in order.
+//     d into one range of equal length a CTA (whole chunks of 128 d's); a cut tile's first range goes
+//     to R, the others to tiles of their own, and the bin epilogue adds them in order.
 //   - the sums are stored word by word: 16-byte stores make the compiler place four sums in the
 //     bank order of the four modes they belong to, and half the FMAs then find all three operands
 //     in one register bank (2782 us, FMA pipe 71% against 80%).
@@ -184,12 +184,15 @@ __global__ void __launch_bounds__(SG_THREADS, SG_CTAS) sgemm_kernel(const __grid
             if (++stage == SG_STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        float *R = p.R + (size_t)(u.seg * pl.ndir + u.dir) * p.rstride + u.mt * SG_BM + 4 * tx;
+        const int c0 = u.ct * SG_BN;
+        const size_t ld = u.seg ? SG_BM : p.Mp;
+        float *R = 4 * tx + (u.seg ? p.tail_piece(u.seg, (u.dir * pl.n_mt + u.mt) * pl.n_ct + u.ct - pl.t0)
+                                   : p.R + u.dir * p.rstride + (size_t)c0 * p.Mp + u.mt * SG_BM);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int c = u.ct * SG_BN + (j < 4 ? 4 * ty + j : 64 + 4 * ty + j - 4);
-            if (c >= p.C) continue;
-            float *row = R + (size_t)c * p.Mp;   // one word a store: see the register banks above
+            const int c = j < 4 ? 4 * ty + j : 64 + 4 * ty + j - 4;
+            if (c0 + c >= p.C) continue;
+            float *row = R + c * ld;   // one word a store: see the register banks above
 #pragma unroll
             for (int i = 0; i < 8; ++i) row[i < 4 ? i : 60 + i] = acc[j][i];
         }
@@ -209,25 +212,30 @@ __global__ void __launch_bounds__(SG_THREADS, SG_CTAS) sgemm_kernel(const __grid
     __syncthreads();
 }
 
-// The values of NK steps from step k of mode n: their four columns, the planes added in order
-// (zero past the block).  The next plane's loads are in flight while a plane is added.
+// The values of NK steps from step k of mode blockIdx.x SG_BM + threadIdx.x in direction b: their four
+// columns, the tile's pieces added in order (zero past the block).  The next piece's loads are in
+// flight while a piece is added.
 template <int NK>
-__device__ __forceinline__ void sg_load_plane(float (&v)[4 * NK], const float *R, int k, int K, int n, int Mp) {
+__device__ __forceinline__ void sg_load_piece(float (&v)[4 * NK], const float *p, size_t ld, int steps) {
 #pragma unroll
-    for (int q = 0; q < 4 * NK; ++q) v[q] = k + q / 4 < K ? __ldcg(R + (size_t)(4 * k + q) * Mp + n) : 0.f;
+    for (int q = 0; q < 4 * NK; ++q) v[q] = q / 4 < steps ? __ldcg(p + q * ld) : 0.f;
 }
 template <int NK>
-__device__ __forceinline__ void sg_load(float (&v)[4 * NK], const float *R, int k, int K, int n, int Mp,
-                                        int nseg, size_t plane) {
-    sg_load_plane<NK>(v, R, k, K, n, Mp);
+__device__ __forceinline__ void sg_load(float (&v)[4 * NK], const SgemmParams &p, int b, int k, int K) {
+    const int ct = 4 * k / SG_BN, tile = (b * p.plan.n_mt + (int)blockIdx.x) * p.plan.n_ct + ct;
+    const int nseg = p.plan.segments(tile), c = 4 * k - ct * SG_BN;
+    sg_load_piece<NK>(v, p.R + b * p.rstride + (size_t)(4 * k) * p.Mp + blockIdx.x * SG_BM + threadIdx.x, p.Mp, K - k);
+    const auto piece = [&](float (&w)[4 * NK], int s) {
+        sg_load_piece<NK>(w, p.tail_piece(s, tile - p.plan.t0) + c * SG_BM + threadIdx.x, SG_BM, K - k);
+    };
     float w[2][4 * NK];
-    if (nseg > 1) sg_load_plane<NK>(w[0], R + plane, k, K, n, Mp);
+    if (nseg > 1) piece(w[0], 1);
     for (int s = 1; s < nseg; s += 2) {
-        if (s + 1 < nseg) sg_load_plane<NK>(w[1], R + (s + 1) * plane, k, K, n, Mp);
+        if (s + 1 < nseg) piece(w[1], s + 1);
 #pragma unroll
         for (int q = 0; q < 4 * NK; ++q) v[q] += w[0][q];
         if (s + 1 >= nseg) break;
-        if (s + 2 < nseg) sg_load_plane<NK>(w[0], R + (s + 2) * plane, k, K, n, Mp);
+        if (s + 2 < nseg) piece(w[0], s + 2);
 #pragma unroll
         for (int q = 0; q < 4 * NK; ++q) v[q] += w[1][q];
     }
@@ -236,17 +244,15 @@ __device__ __forceinline__ void sg_load(float (&v)[4 * NK], const float *R, int 
 // One thread per stored mode (warps = 32 consecutive modes), EPI_STEPS steps a CTA (a tile's
 // columns are a multiple of theirs, so a CTA reads one tile of the product).
 constexpr int EPI_STEPS = 4;
-__global__ void __launch_bounds__(128) fp32_bin_epilogue_kernel(const float *__restrict__ R, SgemmPlan pl,
-                                                                size_t plane, int Mp, int K,
+__global__ void __launch_bounds__(SG_BM) fp32_bin_epilogue_kernel(const __grid_constant__ SgemmParams p, int K,
                                                                 const int *mode_bin,
                                                                 const int *mode_slot,
                                                                 float *partials, int n_slots) {
-    const int n = blockIdx.x * 128 + threadIdx.x;
+    const int n = blockIdx.x * SG_BM + threadIdx.x;
     const int lane = threadIdx.x & 31;
     const int k0 = blockIdx.y * EPI_STEPS;
-    const int nseg = pl.segments((int)blockIdx.x * pl.n_ct + 4 * k0 / SG_BN);
     float v[4 * EPI_STEPS];
-    sg_load<EPI_STEPS>(v, R, k0, K, n, Mp, nseg, plane);
+    sg_load<EPI_STEPS>(v, p, 0, k0, K);
     const int bin = mode_bin[n];
     const int slot = mode_slot[n];
     const uint32_t take = seg_scan_masks(bin, lane);
@@ -262,23 +268,18 @@ __global__ void __launch_bounds__(128) fp32_bin_epilogue_kernel(const float *__r
     }
 }
 
-// Direction-resolved variant: the three products R_b of the direction segments of d (plane s of
-// direction b at (3 s + b) rstride).
+// Direction-resolved variant: the three products R_b of the direction segments of d.
 constexpr int DIR_EPI_STEPS = 2;
-__global__ void __launch_bounds__(128) fp32_dir_epilogue_kernel(const float *__restrict__ R, SgemmPlan pl,
-                                                                size_t rstride, int Mp, int K,
+__global__ void __launch_bounds__(SG_BM) fp32_dir_epilogue_kernel(const __grid_constant__ SgemmParams p, int K,
                                                                 const int *mode_bin,
                                                                 const int *mode_slot,
                                                                 float *partials, int n_slots) {
-    const int n = blockIdx.x * 128 + threadIdx.x;
+    const int n = blockIdx.x * SG_BM + threadIdx.x;
     const int lane = threadIdx.x & 31;
     const int k0 = blockIdx.y * DIR_EPI_STEPS;
     float v[3][4 * DIR_EPI_STEPS];
 #pragma unroll
-    for (int b = 0; b < 3; ++b)
-        sg_load<DIR_EPI_STEPS>(v[b], R + b * rstride, k0, K, n, Mp,
-                               pl.segments((b * pl.n_mt + (int)blockIdx.x) * pl.n_ct + 4 * k0 / SG_BN),
-                               3 * rstride);
+    for (int b = 0; b < 3; ++b) sg_load<DIR_EPI_STEPS>(v[b], p, b, k0, K);
     const int bin = mode_bin[n];
     const int slot = mode_slot[n];
     const uint32_t take = seg_scan_masks(bin, lane);
@@ -389,13 +390,11 @@ int sgemm_make_maps(const float *Ed32, int64_t Mp, const float *Bd32, int64_t co
 void launch_fp32_epilogue(const SgemmParams &p, int K, const int *mode_bin, const int *mode_slot,
                           float *partials, int n_slots, cudaStream_t s) {
     const int steps = p.plan.ndir == 3 ? DIR_EPI_STEPS : EPI_STEPS;
-    dim3 grid(p.Mp / 128, (K + steps - 1) / steps);
+    dim3 grid(p.Mp / SG_BM, (K + steps - 1) / steps);
     if (p.plan.ndir == 3)
-        fp32_dir_epilogue_kernel<<<grid, 128, 0, s>>>(p.R, p.plan, p.rstride, p.Mp, K, mode_bin, mode_slot,
-                                                      partials, n_slots);
+        fp32_dir_epilogue_kernel<<<grid, SG_BM, 0, s>>>(p, K, mode_bin, mode_slot, partials, n_slots);
     else
-        fp32_bin_epilogue_kernel<<<grid, 128, 0, s>>>(p.R, p.plan, p.rstride, p.Mp, K, mode_bin, mode_slot,
-                                                      partials, n_slots);
+        fp32_bin_epilogue_kernel<<<grid, SG_BM, 0, s>>>(p, K, mode_bin, mode_slot, partials, n_slots);
 }
 
 }  // namespace mhc

@@ -112,7 +112,8 @@ cudaError_t measure_fp32_fma(cudaStream_t s, int sm_count, double *tflops);
 // CTA.  Range q starts at tail chunk floor(q T / parts); a tile's segments are the ranges that
 // touch it, in chunk order.
 constexpr int SGEMM_CHUNK = 128;    // d elements
-constexpr int SGEMM_MAX_SEG = 8;    // most pieces of a tile (planes of R)
+constexpr int SGEMM_MAX_SEG = 8;    // most pieces of a tile
+constexpr int SGEMM_TILE = 128 * 128;   // elements of a tile
 struct SgemmPlan {
     int ndir, n_mt, n_ct, n_kb, nch, tiles, t0, parts, ctas, max_seg;
     __host__ __device__ long long tail_chunks() const { return (long long)(tiles - t0) * nch; }
@@ -126,6 +127,8 @@ struct SgemmPlan {
         const int tl = (int)(g / nch);
         return tl * n_kb + (int)(g - (long long)tl * nch) * chunk_kb;
     }
+    // elements of the tail's second and later pieces (see SgemmParams::tail)
+    size_t tail_elements() const { return (size_t)(max_seg - 1) * (tiles - t0) * SGEMM_TILE; }
     __host__ __device__ int segments(int tile) const {
         if (tile < t0) return 1;
         const long long g0 = (long long)(tile - t0) * nch;
@@ -134,18 +137,23 @@ struct SgemmPlan {
 };
 struct SgemmParams {
     CUtensorMap tmA, tmB;   // Ed32 [D][Mp], Bd32 [D][cols]: boxes of 16 d's x 128
-    float *R;               // plane s of direction b: R + (s ndir + b) rstride, [C][Mp]
+    float *R;               // direction b's product: R + b rstride, [C][Mp]; of a cut tile the first piece
     size_t rstride;
+    float *tail;            // the other pieces, a tile each ([128 columns][128 modes]), piece 1 of every
+                            // tile of the tail, then piece 2, ..: plan.tail_elements()
     SgemmPlan plan;
     int C, Mp, dir_cols;    // dir_cols: d's of a direction segment (0 without the split)
     long long wait_limit;   // SM cycles a barrier wait may take before the CTA gives up
     int *status;
+    __host__ __device__ float *tail_piece(int seg, int tl) const {
+        return tail + ((size_t)(seg - 1) * (plan.tiles - plan.t0) + tl) * SGEMM_TILE;
+    }
 };
-// cut false: every tile runs whole (R is one plane).
+// cut false: every tile runs whole (no tail pieces).
 SgemmPlan sgemm_plan(int64_t Mp, int C, int64_t Dk, int ndir, int sms, bool cut);
 int sgemm_make_maps(const float *Ed32, int64_t Mp, const float *Bd32, int64_t cols, int64_t D, SgemmParams &p);
 cudaError_t launch_sgemm(const SgemmParams &p, cudaStream_t s);
-// From the product (its planes added in order): J_n^a(k) = R[4k][n] R[4k+1+a][n], segmented bin
+// From the product (a tile's pieces added in order): J_n^a(k) = R[4k][n] R[4k+1+a][n], segmented bin
 // sums into partials[k][a][slot]; with three direction segments R_b, Xdot = sum_b R_b[4k][n] and
 // J_n^{ab}(k) = Xdot R_b[4k+1+a][n] into partials[k][a][b*n_slots + slot].
 void launch_fp32_epilogue(const SgemmParams &p, int K, const int *mode_bin, const int *mode_slot,

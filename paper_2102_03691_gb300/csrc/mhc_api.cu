@@ -165,6 +165,7 @@ struct mhc_handle {
     std::map<int, TcConfig> tuned;  // K -> config
     TcParams<1> tcp{};
     SgemmParams sgp{};    // FP32 path
+    bool fp32_cut = true;   // the product's last wave of tiles may be cut along d
     XcPlan xc_plan{};     // cross-correlations (MHC_FLAG_XCORR): tensor-core plan and parameters
     XcTcParams xcp{};
 };
@@ -365,7 +366,7 @@ int sched_units(const mhc_handle *h, const TcConfig &c) {
 
 // The FP32 path's tiles and cuts for C columns (with the direction split, one product a segment).
 SgemmPlan fp32_plan(const mhc_handle *h, int C) {
-    return sgemm_plan(h->M_pad, C, h->dir ? h->N_pad : h->D_ld, h->dir ? 3 : 1, h->sm_count, true);
+    return sgemm_plan(h->M_pad, C, h->dir ? h->N_pad : h->D_ld, h->dir ? 3 : 1, h->sm_count, h->fp32_cut);
 }
 
 void reserve_tuned_ws(mhc_handle *h);
@@ -450,16 +451,23 @@ mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_
             return s;
     } else {
         if ((s = dev_alloc(h, "Ed32", ecount * 4, false)) != MHC_OK) return s;
-        // planes of R: the most that any block length up to k_max cuts a tile into
-        size_t worst = 1;
-        for (int nct = 1; nct <= (4 * K + 127) / 128; ++nct)
-            worst = std::max(worst, (size_t)fp32_plan(h, 128 * nct).max_seg);
-        if ((s = dev_alloc(h, "R", sizeof(float) * worst * h->B_rows * h->M_pad * (h->dir ? 3 : 1), false)) != MHC_OK)
+        if ((s = dev_alloc(h, "R", sizeof(float) * h->B_rows * h->M_pad * (h->dir ? 3 : 1), false)) != MHC_OK)
             return s;
+        // the most tail pieces of any block length up to k_max (below 40 MB: the tail has fewer tiles
+        // than resident CTAs, and about as many ranges); where they do not fit, every tile runs whole
+        h->fp32_cut = true;
+        size_t tail = 0;
+        for (int nct = 1; nct <= (4 * K + 127) / 128; ++nct)
+            tail = std::max(tail, fp32_plan(h, 128 * nct).tail_elements());
+        if (dev_alloc(h, "R_tail", sizeof(float) * tail, false) != MHC_OK) {
+            h->fp32_cut = false;
+            h->err.clear();
+        }
         SgemmParams &P = h->sgp;
         if (sgemm_make_maps(dptr<float>(h, "Ed32"), h->M_pad, dptr<float>(h, "Bd32"), h->B_rows, h->D_ld, P))
             return fail(h, MHC_ERR_CUDA, "cuTensorMapEncodeTiled failed");
         P.R = dptr<float>(h, "R");
+        P.tail = dptr<float>(h, "R_tail");
         P.rstride = (size_t)h->B_rows * h->M_pad;
         P.Mp = (int)h->M_pad;
         P.dir_cols = (int)h->N_pad;

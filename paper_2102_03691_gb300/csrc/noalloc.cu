@@ -176,7 +176,7 @@ extern "C" mhc_status mhc_binned_current_noalloc(int32_t n_atoms, int32_t n_mode
     a.col_scale = reinterpret_cast<float *>(s + o_cs);
     a.Jtot = J;
     launch_pack(a, st);
-    // the scratch holds one plane of the product: every tile runs whole
+    // the scratch holds the product alone: every tile runs whole
     SgemmParams P{};
     if (sgemm_make_maps(Ed32, M_pad, Bd32, B_rows, D_ld, P)) return MHC_ERR_CUDA;
     P.R = reinterpret_cast<float *>(s + o_R);

@@ -681,16 +681,18 @@ mhc_status run_projection(mhc_handle *h, int K) {
 }
 
 // ---- autotuning of the tile shape and the d-axis split count
-// Results are kept per process (every handle of the same device, precision, shape and block
-// length reuses them) and, when the environment variable MHC_TUNE_CACHE names a file, in that
-// file across processes.
+// Results are kept per process (every handle of the same device, precision, shape, block length and
+// flags reuses them) and, when the environment variable MHC_TUNE_CACHE names a file, in that file
+// across processes.  flags: bit 0 the direction split, bit 1 the cross-correlations, behind whose
+// traffic the candidates are timed (time_candidates); a line without that bit, as every line was
+// once, is a handle's without them.
 struct TuneKey {
     std::string device;
-    int sm, prec, dir, K, split_req;
+    int sm, prec, flags, K, split_req;
     int64_t D_ld, M_eff;
     bool operator<(const TuneKey &o) const {
-        return std::tie(device, sm, prec, dir, K, split_req, D_ld, M_eff) <
-               std::tie(o.device, o.sm, o.prec, o.dir, o.K, o.split_req, o.D_ld, o.M_eff);
+        return std::tie(device, sm, prec, flags, K, split_req, D_ld, M_eff) <
+               std::tie(o.device, o.sm, o.prec, o.flags, o.K, o.split_req, o.D_ld, o.M_eff);
     }
 };
 std::mutex g_tune_mutex;
@@ -698,11 +700,11 @@ std::map<TuneKey, TcConfig> g_tune_cache;
 bool g_tune_file_read = false;
 
 TuneKey tune_key(const mhc_handle *h, int K) {
-    return TuneKey{h->device_name, h->sm_count, (int)h->split, h->dir ? 1 : 0, K,
+    return TuneKey{h->device_name, h->sm_count, (int)h->split, (h->dir ? 1 : 0) | (has_xcorr(h) ? 2 : 0), K,
                    (int)h->prm.split_d, h->D_ld, h->M_eff};
 }
 
-// Cache file lines: sm prec dir K split_req D_ld M_eff bn bk stages pair split <device name>
+// Cache file lines: sm prec flags K split_req D_ld M_eff bn bk stages pair split <device name>
 void tune_file_read_locked() {
     if (g_tune_file_read) return;
     g_tune_file_read = true;
@@ -716,7 +718,7 @@ void tune_file_read_locked() {
         TcConfig c{};
         long long D = 0, M = 0;
         int used = 0;
-        if (std::sscanf(line, "%d %d %d %d %d %lld %lld %d %d %d %d %d %n", &k.sm, &k.prec, &k.dir, &k.K,
+        if (std::sscanf(line, "%d %d %d %d %d %lld %lld %d %d %d %d %d %n", &k.sm, &k.prec, &k.flags, &k.K,
                         &k.split_req, &D, &M, &c.bn, &c.bk, &c.stages, &c.pair, &c.split, &used) < 12)
             continue;
         std::string name(line + used);
@@ -735,7 +737,7 @@ void tune_file_append_locked(const TuneKey &k, const TcConfig &c) {
     if (!path || !*path) return;
     FILE *f = std::fopen(path, "a");
     if (!f) return;
-    std::fprintf(f, "%d %d %d %d %d %lld %lld %d %d %d %d %d %s\n", k.sm, k.prec, k.dir, k.K,
+    std::fprintf(f, "%d %d %d %d %d %lld %lld %d %d %d %d %d %s\n", k.sm, k.prec, k.flags, k.K,
                  k.split_req, (long long)k.D_ld, (long long)k.M_eff, c.bn, c.bk, c.stages, c.pair,
                  c.split, k.device.c_str());
     std::fclose(f);

@@ -503,8 +503,9 @@ mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_
         h->tcp.idesc = idesc_f16(h->split == SPLIT_BF16 ? 1u : 0u, (c.pair ? 2 : 1) * TC_BM, (uint32_t)c.bn);
     }
     h->bins_ready = true;
+    if ((s = reset_accumulators(h)) != MHC_OK) return s;
     reserve_tuned_ws(h);
-    return reset_accumulators(h);
+    return MHC_OK;
 }
 
 // With the direction split: graphene-like 4096 atoms, K = 128 has 96 pair tiles for 76 resident
@@ -745,7 +746,8 @@ void tune_file_append_locked(const TuneKey &k, const TcConfig &c) {
 
 // The split workspace of the tile already tuned for this shape and the longest block (by another
 // handle of the process, or in the tuning file), allocated with the bins: the first push would
-// otherwise stop for it (about 100 us).  Where it does not fit, the push that needs it reports so.
+// otherwise stop for it (about 100 us).  After everything that the handle cannot do without; where it
+// does not fit, the push that needs it reports so.
 void reserve_tuned_ws(mhc_handle *h) {
     if (!is_tc(h) || h->prm.tile_config != 0 || h->M_eff == 0) return;
     TcConfig c{};
@@ -2084,6 +2086,13 @@ mhc_status mhc_group_create(mhc_group **out, mhc_handle *const *handles, int32_t
     if (s != MHC_OK) {
         delete g;
         return s;
+    }
+    // what the members' bins reserved for a split (a member pushed by itself allocates it again)
+    for (mhc_handle *h : g->hs) {
+        if (!dptr<float>(h, "split_ws")) continue;
+        cudaStreamSynchronize(h->stream);
+        drop_graphs(h);
+        dev_free(h, "split_ws");
     }
     *out = g;
     return MHC_OK;

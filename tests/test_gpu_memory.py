@@ -1,4 +1,9 @@
-"""Device memory that a handle holds beside what its results need: the FP32 product's tail pieces."""
+"""Device memory that a handle holds beside what its results need: the FP32 product's planes and
+the split workspace of a tuned shape."""
+import os
+import subprocess
+import sys
+
 import pytest
 
 from tests.test_gpu_parity import make_case, need_gpu
@@ -31,3 +36,45 @@ def test_fp32_product_holds_one_plane_and_its_tail(direction):
     assert plane <= extra <= plane + 2 * (2 * sms) * 128 * 128 * 4 + (1 << 20), (extra, plane)
     a.close()
     b.close()
+
+
+_CHILD = r"""
+import sys
+sys.path.insert(0, sys.argv[1])
+from tests.test_gpu_memory import handle
+from tests.test_gpu_parity import make_case
+from paper_2102_03691_gb300.mhc import ModalHeatCurrentGroup
+import numpy as np
+cs = [make_case(N=40, M=120, T=16, B=4, seed=9985 + j) for j in range(2)]
+def members():
+    return [handle(c, "fp16x3", 16) for c in cs]
+hs = members()
+before = [h.info()["device_bytes"] for h in hs]
+g = ModalHeatCurrentGroup(hs)
+after = [h.info()["device_bytes"] for h in hs]
+g.push([c["v"] for c in cs], [c["W"] for c in cs])
+grouped = [h.read_binned_current().copy() for h in hs]
+for h in hs:
+    h.reset()
+for h, c, J in zip(hs, cs, grouped):      # a member pushed by itself gets its workspace back
+    h.push(c["v"], c["W"])
+    assert np.abs(h.read_binned_current() - J).max() <= 1e-5 * np.abs(J).max()
+print("bytes", *before, *after, *[h.info()["device_bytes"] for h in hs])
+"""
+
+
+def test_group_members_hold_no_split_workspace(tmp_path):
+    # grouped launches run unsplit: what the members' bins reserved for a tuned split is given back
+    need_gpu()
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    p = torch.cuda.get_device_properties(0)
+    (tmp_path / "tune.txt").write_text(f"{p.multi_processor_count} 2 0 16 0 128 120 128 32 8 1 -1 {p.name}\n")
+    (tmp_path / "child.py").write_text(_CHILD)
+    r = subprocess.run([sys.executable, str(tmp_path / "child.py"), root],
+                       env=dict(os.environ, MHC_TUNE_CACHE=str(tmp_path / "tune.txt")),
+                       capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
+    b = list(map(int, r.stdout.split("bytes")[1].split()))
+    # 128 columns x 256 modes x 4 bytes a plane, at least one
+    assert all(x - y >= 128 * 256 * 4 for x, y in zip(b[:2], b[2:4])), b
+    assert all(z >= x for x, z in zip(b[:2], b[4:])), b

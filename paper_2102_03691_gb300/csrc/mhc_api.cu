@@ -762,52 +762,51 @@ void reserve_tuned_ws(mhc_handle *h) {
     if (ensure_split_ws(h, c) != MHC_OK) h->err.clear();
 }
 
-// Time candidate configurations in interleaved rounds (one warm-up launch each, then `rounds`
-// rounds of every candidate) and keep each candidate's fastest round: the candidates see the same
-// clock and power state, where timing them one after the other let the power cap, reached during
-// the first candidates' launches, slow the last ones.  Short projections run several times a
-// round, queued behind one more that is not timed: a single launch of a few tens of microseconds
-// between two events also times the host's launches, two of them with a split.  With the
+// Time candidate configurations in interleaved rounds (`rounds` timed launches of every candidate, the
+// first behind its warm-up) and keep each candidate's fastest round: the candidates see the same clock and power
+// state, where timing them one after the other let the power cap, reached during the first
+// candidates' launches, slow the last ones.  A short projection is timed behind one that is not: a
+// single launch of a few tens of microseconds between two events also times the host's launches, two
+// of them with a split.  A candidate whose warm-up takes half as long again as the fastest is not
+// timed further (it keeps that time), so that the first push of a shape pays for few of them.  With the
 // cross-correlations every launch is timed by itself behind a read of their state, which streams
 // through L2 between two projections of a run: from a warm L2 512 atoms x 250 steps look best
 // unsplit, and a run of four blocks with 64 bins then takes 485 us instead of 457 with three splits.
 mhc_status time_candidates(mhc_handle *h, int K, std::vector<std::pair<float, TcConfig>> &cands,
                            int rounds = 3) {
-    constexpr float ROUND_MS = 0.3f;   // GPU time of a candidate's round
-    constexpr int MAX_REPS = 8;
+    constexpr float SHORT_MS = 0.3f;   // longer launches hide the host's
+    constexpr float HOPELESS = 1.5f;
     cudaEvent_t e0, e1;
     MHC_CUDA(h, cudaEventCreate(&e0));
     MHC_CUDA(h, cudaEventCreate(&e1));
     mhc_status s = MHC_OK;
-    // one timed round of candidate c: `lead` untimed launches, then `reps` timed ones
-    auto timed = [&](const TcConfig &c, int lead, int reps, float &ms) -> mhc_status {
+    // one launch of candidate c timed, behind one that is not (`lead`)
+    auto timed = [&](const TcConfig &c, bool lead, float &ms) -> mhc_status {
         if (mhc_status q = set_tc_config(h, c); q != MHC_OK) return q;
         if (has_xcorr(h)) launch_xcorr_touch(h->xc_plan, h->xcp, h->stream);
-        for (int r = 0; r < lead; ++r)
+        if (lead)
             if (mhc_status q = run_projection(h, K); q != MHC_OK) return q;
         if (cudaEventRecord(e0, h->stream) != cudaSuccess) return fail(h, MHC_ERR_CUDA, "event record");
-        for (int r = 0; r < reps; ++r)
-            if (mhc_status q = run_projection(h, K); q != MHC_OK) return q;
+        if (mhc_status q = run_projection(h, K); q != MHC_OK) return q;
         if (cudaEventRecord(e1, h->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
             cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)
             return fail(h, MHC_ERR_CUDA, "autotune timing failed");
-        ms /= (float)reps;
         return MHC_OK;
     };
     float shortest = 1e30f;
-    for (auto &x : cands) {   // warm-up, and the length of a launch
+    for (auto &x : cands) {
         x.first = 1e30f;
-        float ms = 0.f;
-        if ((s = timed(x.second, has_xcorr(h) ? 0 : 1, 1, ms)) != MHC_OK) break;
-        shortest = std::min(shortest, ms);
+        if ((s = timed(x.second, !has_xcorr(h), x.first)) != MHC_OK) break;
+        shortest = std::min(shortest, x.first);
     }
-    const int reps =
-        has_xcorr(h) ? 1 : std::max(1, std::min(MAX_REPS, (int)(ROUND_MS / std::max(shortest, 1e-3f))));
-    for (int r = 0; r < rounds && s == MHC_OK; ++r)
-        for (auto &x : cands) {
+    const bool lead = !has_xcorr(h) && shortest < SHORT_MS;
+    std::vector<bool> keep;
+    for (auto &x : cands) keep.push_back(has_xcorr(h) || x.first <= HOPELESS * shortest);
+    for (int r = has_xcorr(h) ? 0 : 1; r < rounds && s == MHC_OK; ++r)   // (there the first was cold)
+        for (size_t q = 0; q < cands.size() && s == MHC_OK; ++q) {
+            if (!keep[q]) continue;
             float ms = 0.f;
-            if ((s = timed(x.second, reps > 1 ? 1 : 0, reps, ms)) != MHC_OK) break;
-            x.first = std::min(x.first, ms);
+            if ((s = timed(cands[q].second, lead, ms)) == MHC_OK) cands[q].first = std::min(cands[q].first, ms);
         }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

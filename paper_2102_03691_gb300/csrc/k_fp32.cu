@@ -184,15 +184,19 @@ __global__ void __launch_bounds__(SG_THREADS, SG_CTAS) sgemm_kernel(const __grid
             if (++stage == SG_STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        const int c0 = u.ct * SG_BN;
-        const size_t ld = u.seg ? SG_BM : p.Mp;
-        float *R = 4 * tx + (u.seg ? p.tail_piece(u.seg, (u.dir * pl.n_mt + u.mt) * pl.n_ct + u.ct - pl.t0)
-                                   : p.R + u.dir * p.rstride + (size_t)c0 * p.Mp + u.mt * SG_BM);
+        // column c of the product at R + at + c ld: in its plane, or in a tail piece whose column 0 is
+        // the tile's first (one store sequence for both; two, or one more value kept over the sums,
+        // cost 7% in register banks)
+        const unsigned ld = u.seg ? SG_BM : p.Mp;
+        float *R = u.seg ? p.tail : p.R;
+        const long long at = 4 * tx + (u.seg ? p.tail_at(u.seg, (u.dir * pl.n_mt + u.mt) * pl.n_ct + u.ct - pl.t0) -
+                                                   (long long)u.ct * SG_BN * SG_BM
+                                             : (long long)(u.dir * p.rstride) + u.mt * SG_BM);
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const int c = j < 4 ? 4 * ty + j : 64 + 4 * ty + j - 4;
-            if (c0 + c >= p.C) continue;
-            float *row = R + c * ld;   // one word a store: see the register banks above
+            const int c = u.ct * SG_BN + (j < 4 ? 4 * ty + j : 64 + 4 * ty + j - 4);
+            if (c >= p.C) continue;
+            float *row = R + (at + (long long)c * ld);   // one word a store: see the register banks above
 #pragma unroll
             for (int i = 0; i < 8; ++i) row[i < 4 ? i : 60 + i] = acc[j][i];
         }
@@ -226,7 +230,7 @@ __device__ __forceinline__ void sg_load(float (&v)[4 * NK], const SgemmParams &p
     const int nseg = p.plan.segments(tile), c = 4 * k - ct * SG_BN;
     sg_load_piece<NK>(v, p.R + b * p.rstride + (size_t)(4 * k) * p.Mp + blockIdx.x * SG_BM + threadIdx.x, p.Mp, K - k);
     const auto piece = [&](float (&w)[4 * NK], int s) {
-        sg_load_piece<NK>(w, p.tail_piece(s, tile - p.plan.t0) + c * SG_BM + threadIdx.x, SG_BM, K - k);
+        sg_load_piece<NK>(w, p.tail + p.tail_at(s, tile - p.plan.t0) + c * SG_BM + threadIdx.x, SG_BM, K - k);
     };
     float w[2][4 * NK];
     if (nseg > 1) piece(w[0], 1);

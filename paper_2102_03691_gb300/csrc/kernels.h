@@ -145,8 +145,8 @@ struct SgemmParams {
     int C, Mp, dir_cols;    // dir_cols: d's of a direction segment (0 without the split)
     long long wait_limit;   // SM cycles a barrier wait may take before the CTA gives up
     int *status;
-    __host__ __device__ float *tail_piece(int seg, int tl) const {
-        return tail + ((size_t)(seg - 1) * (plan.tiles - plan.t0) + tl) * SGEMM_TILE;
+    __host__ __device__ long long tail_at(int seg, int tl) const {   // piece `seg` >= 1 of the tail's tile tl
+        return ((long long)(seg - 1) * (plan.tiles - plan.t0) + tl) * SGEMM_TILE;
     }
 };
 // cut false: every tile runs whole (no tail pieces).

@@ -79,7 +79,7 @@ typedef enum { MHC_DOF_MAJOR = 0, MHC_MODE_MAJOR = 1 } mhc_layout;
                                       fixed staging buffers.  Up to 32 graphs are cached. */
 #define MHC_FLAG_PROFILE 0x4       /* time each projection launch with CUDA events (mhc_kernel_time);
                                       implies direct launches */
-#define MHC_FLAG_TEST_STALL 0x8    /* fault injection for tests of the failure path: the tensor-core
+#define MHC_FLAG_TEST_STALL 0x8    /* fault injection for tests of the failure path: the projection
                                       kernel arms its first stage barrier to expect 16 bytes more
                                       than its copies deliver, so its bounded waits (0.1 s with this flag)
                                       give up and the next sync/read returns MHC_ERR_TIMEOUT; no

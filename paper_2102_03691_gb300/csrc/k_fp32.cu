@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(SG_THREADS, SG_CTAS) sgemm_kernel(const __grid
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], SG_WARPS);
         }
+        if (p.stall_inject) mbar_expect_tx(&full[0], 16);
         *abort = 0;
         fence_mbar_init();
     }

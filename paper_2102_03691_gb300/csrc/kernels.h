@@ -145,6 +145,7 @@ struct SgemmParams {
     int C, Mp, dir_cols;    // dir_cols: d's of a direction segment (0 without the split)
     long long wait_limit;   // SM cycles a barrier wait may take before the CTA gives up
     int *status;
+    int stall_inject;       // test hook: arm a CTA's first stage barrier for 16 bytes more than its copies deliver
     __host__ __device__ long long tail_at(int seg, int tl) const {   // piece `seg` >= 1 of the tail's tile tl
         return ((long long)(seg - 1) * (plan.tiles - plan.t0) + tl) * SGEMM_TILE;
     }

@@ -471,7 +471,6 @@ mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_
         P.rstride = (size_t)h->B_rows * h->M_pad;
         P.Mp = (int)h->M_pad;
         P.dir_cols = (int)h->N_pad;
-        P.wait_limit = 2000000000ll;
         P.status = h->status;
     }
     // Eraw is already in the stored column order (direction-major with the split)
@@ -598,9 +597,13 @@ mhc_status run_projection(mhc_handle *h, int K) {
                                     sizeof(float) * K * 3 * slot_stride(h), h->stream));
         return MHC_OK;
     }
+    const bool stall = (h->prm.flags & MHC_FLAG_TEST_STALL) != 0;
+    const long long wait_limit = stall ? 200000000ll : 2000000000ll;   // 0.1 s when testing the timeout
     if (!is_tc(h)) {
         // with the direction split one product per segment of d, then Xdot = sum over segments
         SgemmParams &P = h->sgp;
+        P.stall_inject = stall ? 1 : 0;
+        P.wait_limit = wait_limit;
         P.C = 4 * K;
         P.plan = fp32_plan(h, P.C);
         MHC_CUDA(h, launch_sgemm(P, h->stream));
@@ -612,7 +615,6 @@ mhc_status run_projection(mhc_handle *h, int K) {
     }
     TcConfig c = h->tc;
     TcProblem &P = h->tcp.prob[0];
-    const bool stall = (h->prm.flags & MHC_FLAG_TEST_STALL) != 0;
     // As programmatic dependents the projection and its split finish set up while the last CTAs of
     // the kernel before finish: about 1 us each of a 119 us push at 512 atoms x 1000 steps.  A
     // graph with a programmatic edge starts later, though: at 64 atoms x 32 steps the push took
@@ -620,7 +622,7 @@ mhc_status run_projection(mhc_handle *h, int K) {
     // atoms and step a CTA); at 1003 x 77, just below it, both take 60 us.
     const bool pdl = (int64_t)K * h->N >= (int64_t)h->sm_count * 512;
     h->tcp.stall_inject = stall ? 1 : 0;
-    h->tcp.wait_limit = stall ? 200000000ll : 2000000000ll;   // 0.1 s when testing the timeout
+    h->tcp.wait_limit = wait_limit;
     P.K = K;
     P.n_col_tiles = (int)((4 * K + c.bn - 1) / c.bn);
     P.sk_parts = 0;

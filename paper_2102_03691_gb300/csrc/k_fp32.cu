@@ -369,7 +369,7 @@ SgemmPlan sgemm_plan(int64_t Mp, int C, int64_t Dk, int ndir, int sms, bool cut)
     return p;
 }
 
-cudaError_t launch_sgemm(const SgemmParams &p, cudaStream_t s) {
+cudaError_t launch_sgemm(const SgemmParams &p, cudaStream_t s, bool pdl) {
     static PerDevice once;
     const cudaError_t ready = opt_in_smem(once, sgemm_kernel, SG_SMEM);
     if (ready != cudaSuccess) return ready;
@@ -383,7 +383,7 @@ cudaError_t launch_sgemm(const SgemmParams &p, cudaStream_t s) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // after the pack
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, sgemm_kernel, p);
 }
 

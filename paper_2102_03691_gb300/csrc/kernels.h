@@ -153,7 +153,8 @@ struct SgemmParams {
 // cut false: every tile runs whole (no tail pieces).
 SgemmPlan sgemm_plan(int64_t Mp, int C, int64_t Dk, int ndir, int sms, bool cut);
 int sgemm_make_maps(const float *Ed32, int64_t Mp, const float *Bd32, int64_t cols, int64_t D, SgemmParams &p);
-cudaError_t launch_sgemm(const SgemmParams &p, cudaStream_t s);
+// pdl: as a programmatic dependent of the pack (the kernel before it on the stream).
+cudaError_t launch_sgemm(const SgemmParams &p, cudaStream_t s, bool pdl);
 // From the product (a tile's pieces added in order): J_n^a(k) = R[4k][n] R[4k+1+a][n], segmented bin
 // sums into partials[k][a][slot]; with three direction segments R_b, Xdot = sum_b R_b[4k][n] and
 // J_n^{ab}(k) = Xdot R_b[4k+1+a][n] into partials[k][a][b*n_slots + slot].

@@ -599,6 +599,12 @@ mhc_status run_projection(mhc_handle *h, int K) {
     }
     const bool stall = (h->prm.flags & MHC_FLAG_TEST_STALL) != 0;
     const long long wait_limit = stall ? 200000000ll : 2000000000ll;   // 0.1 s when testing the timeout
+    // As programmatic dependents the projection and its split finish set up while the last CTAs of
+    // the kernel before finish: about 1 us each of a 119 us push at 512 atoms x 1000 steps.  A
+    // graph with a programmatic edge starts later, though: at 64 atoms x 32 steps the push took
+    // 38.9 us with the edge and 34.8 without.  The line lies at a pack of one wave of CTAs (512
+    // atoms and step a CTA); at 1003 x 77, just below it, both take 60 us.
+    const bool pdl = (int64_t)K * h->N >= (int64_t)h->sm_count * 512;
     if (!is_tc(h)) {
         // with the direction split one product per segment of d, then Xdot = sum over segments
         SgemmParams &P = h->sgp;
@@ -606,7 +612,7 @@ mhc_status run_projection(mhc_handle *h, int K) {
         P.wait_limit = wait_limit;
         P.C = 4 * K;
         P.plan = fp32_plan(h, P.C);
-        MHC_CUDA(h, launch_sgemm(P, h->stream));
+        MHC_CUDA(h, launch_sgemm(P, h->stream, pdl));
         launch_fp32_epilogue(P, K, dptr<int>(h, "mode_bin"), dptr<int>(h, "mode_slot"),
                              dptr<float>(h, "partials"), (int)h->n_slots, h->stream);
         h->launches += 2;
@@ -615,12 +621,6 @@ mhc_status run_projection(mhc_handle *h, int K) {
     }
     TcConfig c = h->tc;
     TcProblem &P = h->tcp.prob[0];
-    // As programmatic dependents the projection and its split finish set up while the last CTAs of
-    // the kernel before finish: about 1 us each of a 119 us push at 512 atoms x 1000 steps.  A
-    // graph with a programmatic edge starts later, though: at 64 atoms x 32 steps the push took
-    // 38.9 us with the edge and 34.8 without.  The line lies at a pack of one wave of CTAs (512
-    // atoms and step a CTA); at 1003 x 77, just below it, both take 60 us.
-    const bool pdl = (int64_t)K * h->N >= (int64_t)h->sm_count * 512;
     h->tcp.stall_inject = stall ? 1 : 0;
     h->tcp.wait_limit = wait_limit;
     P.K = K;

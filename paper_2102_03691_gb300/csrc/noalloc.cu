@@ -188,7 +188,7 @@ extern "C" mhc_status mhc_binned_current_noalloc(int32_t n_atoms, int32_t n_mode
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return MHC_ERR_CUDA;
     P.plan = sgemm_plan(M_pad, P.C, D_ld, 1, sms, false);
-    if ((e = launch_sgemm(P, st)) != cudaSuccess) return MHC_ERR_CUDA;
+    if ((e = launch_sgemm(P, st, true)) != cudaSuccess) return MHC_ERR_CUDA;
     launch_fp32_epilogue(P, K, mode_bin, mode_slot, partials, (int)M_pad, st);
     launch_bin_finish(partials, (int)M_pad, slot_begin, n_bins, K, Jb, hsum, J, jsum, nullptr, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return MHC_ERR_CUDA;

@@ -20,10 +20,10 @@ namespace {
 // The order of the sums depends on K alone, so a grouped launch gives the bits of a solo one.  It is
 // launched plainly: as a programmatic dependent of the projection it made the 8000-atom push 20 us
 // and the 512-atom push 2 us longer.
-// Measured (ncu, us, one thread a step with a tree of FP64 sums -> now): 600 rows, K = 128
-// 10.7 -> 7.0; 200 rows, K = 128 6.9 -> 5.7; 16 systems of 52 bins, K = 256 22.1 -> 22.4; 100 rows,
-// K = 1000 8.6 -> 8.5; 64 rows of 13 slots, K = 256 7.5 -> 7.5.  The sums over the steps in pairs of
-// floats took 6.1, 5.5, 20.4, 8.3 and 7.5, but held 48 bits, and no infinities.
+// Measured (ncu, us, one thread a step with a tree of FP64 sums -> now): 600 rows, K = 128 10.7 -> 6.4;
+// 200 rows, K = 128 6.9 -> 5.1; 16 systems of 52 bins, K = 256 22.1 -> 17.2; 100 rows, K = 1000 8.6
+// -> 8.0; 64 rows of 13 slots, K = 256 7.5 -> 6.6; 100 and 304 rows of a slot or none, K = 200 4.9 ->
+// 4.9, K = 1000 9.7 -> 10.4.
 constexpr int BF_MAX_THREADS = 768;
 __host__ __device__ constexpr int bf_threads(int K) { return K <= 128 ? 384 : BF_MAX_THREADS; }
 
@@ -70,24 +70,17 @@ __device__ __forceinline__ void bin_finish_body(const float *partials, int n_slo
     const int nt = bf_threads(K), steps = nt / 3;   // threads past nt (a longer system's) hold no steps
     const int t = threadIdx.x, a = t % 3, k0 = t / 3;
     const int lane = t & 31, warp = t >> 5;
-    if (b == B) {   // the total current
-        double acc[3] = {0.0, 0.0, 0.0};
-        if (t < nt)
-            for (int k = t; k < K; k += nt)
+    if (b == B) {   // the total current, two warps a component (sums on all warps took this CTA 3 us more)
+        if (warp < 6) {
+            double acc = 0.0;
+#pragma unroll 4
+            for (int k = 32 * (warp / 3) + lane; k < K; k += 64) acc += Jtot[3 * k + warp % 3];
 #pragma unroll
-                for (int q = 0; q < 3; ++q) acc[q] += Jtot[3 * k + q];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_down_sync(FULL_MASK, acc[q], o);
-            if (lane == 0) red[3 * warp + q] = acc[q];
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(FULL_MASK, acc, o);
+            if (lane == 0) red[warp] = acc;
         }
         __syncthreads();
-        if (t < 3) {
-            double s = 0.0;
-            for (int w = 0; w < nt / 32; ++w) s += red[3 * w + t];
-            Jsum[t] += s;
-        }
+        if (t < 3) Jsum[t] += red[t] + red[t + 3];
         return;
     }
     const int s0 = slot_begin[b], s1 = slot_begin[b + 1];

@@ -318,6 +318,15 @@ __device__ __forceinline__ uint64_t smem_desc_kmajor(uint32_t saddr, uint32_t sb
 }
 
 // ------------------------------------------------------------------ bin reduction
+// float -> double by its bits: the conversion instruction runs on the narrow FP64 pipe, 16 cycles a warp
+// and SM, and these in a few cycles beside it.
+__device__ __forceinline__ double f32_to_f64(float x) {
+    const uint32_t u = __float_as_uint(x), a = u & 0x7fffffffu;
+    if (a - 1u < 0x007fffffu || a >= 0x7f800000u) return (double)x;   // subnormal, infinite or NaN
+    const uint32_t hi = a ? (a >> 3) + 0x38000000u : 0u;              // exponent rebiased, fraction widened
+    return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
+}
+
 // Per-lane masks for a segmented inclusive warp scan over lanes whose bin ids are
 // non-decreasing (modes are stored sorted by bin): bit r set <=> the lane 2^r below
 // belongs to the same bin.

@@ -137,8 +137,15 @@ __global__ void __launch_bounds__(BF_MAX_THREADS, 2) bin_finish_group_kernel(con
 //     (smaller pieces balance better: N = 512, K = 1000 had 175 CTAs of 16 warps, two on 23 of
 //     the 152 SMs), each CTA staging its own steps alone; the ranks read each other's partials
 //     through distributed shared memory and each finishes its share of the tile's sums;
-//   - a CTA alone has at least LC_FINAL_WARPS warps (those without steps take part in the
-//     staging and the final sums), and every warp fetches the sums it will update into L2 first.
+//   - a CTA alone has up to LC_FINAL_WARPS warps where the tiles are few (those without steps take
+//     part in the staging and the final sums), and every warp fetches the sums it will update into
+//     L2 first;
+//   - from LC_MANY_TILES tiles the latency of one CTA is hidden by the others, and warps without steps,
+//     the early fetch and the barriers of a cluster only cost: CTAs stay small, a tile is a CTA
+//     of its own (but for 16 warps of steps, of which an SM holds too few whole), and the sums are
+//     updated one by one.  304 bins x 1000 lags (2432 tiles; us a push, one warp a tile and 32 steps ->
+//     the form for few tiles -> now): K = 1 43 -> 70 -> 47, 128 59 -> 87 -> 59, 400 118 -> 131 -> 119; 1000
+//     in clusters 202 -> 193.
 // Measured (ncu, cold caches, us, before -> now): K = 32, 8 bins, 8 lags 23.3 -> 7.7; K = 77, 37
 // bins, 123 lags 15.5 -> 8.4; K = 1000, 100 bins, 200 lags 24.6 -> 18.6; K = 512, 64 bins, 1000
 // lags 30.5 -> 27.9; K = 256, 64 bins, 500 lags 13.0 -> 13.4.  The cluster form starts at
@@ -151,13 +158,18 @@ constexpr int LC_CTA_WARPS = 4;   // warps of a CTA of a cluster
 constexpr int LC_FINAL_WARPS = 12;   // fewest warps of a CTA that holds a tile alone
 constexpr int LC_BATCH = 5;       // sums a warp updates at a time (all of them with 8 or more warps)
 constexpr int LC_MIN_STEPS = 4;   // fewest steps a warp is worth starting for
+// (Of this GPU's 152 SMs and not of those a process is given: the order of the sums then depends on the
+// sizes alone.)
 constexpr int LC_FILL_WARPS = 152 * 12;   // three warps a scheduler on every SM
 constexpr int LC_FILL_TILES = 76;         // tiles from which clusters of small CTAs balance better
+constexpr int LC_MANY_TILES = 700;        // tiles from which only throughput counts
 
 // Warps with steps of one tile, steps a warp, the CTAs (cluster ranks) they run in, the warps
-// with steps of a CTA and all its warps.
+// with steps of a CTA and all its warps, the kernel's form.
+enum LagCorrForm { LC_FEW, LC_CLUSTER, LC_MANY };
 struct LagCorrPlan {
     int warps, ks, ranks, step_warps, cta_warps;
+    LagCorrForm form;
 };
 
 LagCorrPlan lag_corr_plan(int K, int tiles) {
@@ -170,9 +182,11 @@ LagCorrPlan lag_corr_plan(int K, int tiles) {
     p.warps = std::max(lo, std::min(hi, want));
     p.ks = (K + p.warps - 1) / p.warps;
     p.warps = (K + p.ks - 1) / p.ks;
-    p.ranks = tiles >= LC_FILL_TILES ? (p.warps + LC_CTA_WARPS - 1) / LC_CTA_WARPS : 1;
+    const bool many = tiles >= LC_MANY_TILES;
+    p.ranks = tiles >= LC_FILL_TILES && (!many || p.warps == LC_WARPS) ? (p.warps + LC_CTA_WARPS - 1) / LC_CTA_WARPS : 1;
+    p.form = p.ranks > 1 ? LC_CLUSTER : many ? LC_MANY : LC_FEW;
     p.step_warps = p.ranks > 1 ? LC_CTA_WARPS : p.warps;
-    p.cta_warps = p.ranks > 1 ? LC_CTA_WARPS : std::max(p.warps, LC_FINAL_WARPS);
+    p.cta_warps = p.ranks > 1 ? LC_CTA_WARPS : std::max(p.warps, std::min(LC_FINAL_WARPS, std::max(LC_CTA_WARPS, want)));
     return p;
 }
 
@@ -193,6 +207,7 @@ __device__ __forceinline__ void lc_pair_add(float &s, float &c, float x) {
 }
 
 // t0_dev: the device step counter, which the push's bin finish has already advanced by K.
+template <LagCorrForm FORM>
 __global__ void __launch_bounds__(32 * LC_WARPS, 2) lag_corr_kernel(const float *__restrict__ Jb,
                                                                     const double *__restrict__ Jring,
                                                                     int R, double *Csum, int K,
@@ -202,10 +217,11 @@ __global__ void __launch_bounds__(32 * LC_WARPS, 2) lag_corr_kernel(const float 
     // staging: rows [steps][LC_ROWS] of this CTA's steps, then their J window [steps + 31] as
     // float4 (x, y, z, 0); after the step loop the same space holds the warps' partials
     // [warp][LC_OUT][32]
+    constexpr bool CLUSTER = FORM == LC_CLUSTER;
     extern __shared__ float4 lc_smem4[];
     float *sA = reinterpret_cast<float *>(lc_smem4);
     float *sP = reinterpret_cast<float *>(lc_smem4);
-    const int nrank = (int)gridDim.z, rank = (int)blockIdx.z;   // a cluster spans grid z
+    const int nrank = CLUSTER ? (int)gridDim.z : 1, rank = CLUSTER ? (int)blockIdx.z : 0;   // a cluster spans grid z
     const int l0 = blockIdx.x * 32;
     const int b0 = blockIdx.y * (LC_ROWS / 3);
     const int nthreads = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -219,7 +235,7 @@ __global__ void __launch_bounds__(32 * LC_WARPS, 2) lag_corr_kernel(const float 
     const int l = l0 + lane;
     const int gw = rank + nrank * warp, ngw = nrank * cta_warps;
     auto sums = [&](int o) { return Csum + ((size_t)(b0 + o / 9) * 9 + ((o / 3) % 3) * 3 + o % 3) * L + l; };
-    if ((lane & 15) == 0 && l < L)
+    if (FORM != LC_MANY && (lane & 15) == 0 && l < L)
         for (int o = gw; o < LC_OUT && b0 + o / 9 < B; o += ngw)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(sums(o)));
     const float *Jk = Jb + (size_t)kc0 * B * 3;
@@ -286,34 +302,46 @@ __global__ void __launch_bounds__(32 * LC_WARPS, 2) lag_corr_kernel(const float 
 #pragma unroll
         for (int o = 0; o < LC_OUT; ++o) sP[(warp * LC_OUT + o) * 32 + lane] = acc[o];
     }
-    cluster_sync_all();   // every rank's partials are complete (one CTA: a CTA barrier)
-    for (int o0 = gw; o0 < LC_OUT && b0 + o0 / 9 < B; o0 += LC_BATCH * ngw) {   // warp-uniform
-        double old[LC_BATCH];
-#pragma unroll
-        for (int u = 0; u < LC_BATCH; ++u) {
-            const int o = o0 + u * ngw;
-            old[u] = (o < LC_OUT && b0 + o / 9 < B && l < L) ? *sums(o) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < LC_BATCH; ++u) {
-            const int o = o0 + u * ngw;
-            if (o >= LC_OUT || b0 + o / 9 >= B) break;   // warp-uniform
+    if (CLUSTER) cluster_sync_all();   // every rank's partials are complete
+    else __syncthreads();
+    if constexpr (FORM == LC_MANY) {
+        for (int o = gw; o < LC_OUT && b0 + o / 9 < B; o += ngw) {   // warp-uniform
+            if (l >= L) continue;
+            double *dst = sums(o);
+            const double old = *dst;
             float s = 0.f, c = 0.f;
-            const float *mine = sP + o * 32 + lane;
-            if (nrank == 1) {
-                for (int w = 0; w < step_warps; ++w) lc_pair_add(s, c, mine[w * LC_OUT * 32]);
-            } else {
-                for (int q = 0; q < nrank; ++q) {   // step order: ranks, then warps
-                    const uint32_t peer = mapa_shared(smem_u32(mine), (uint32_t)q);
+            for (int w = 0; w < step_warps; ++w) lc_pair_add(s, c, sP[(w * LC_OUT + o) * 32 + lane]);
+            *dst = old + (f32_to_f64(s) + f32_to_f64(c));
+        }
+    } else {
+        for (int o0 = gw; o0 < LC_OUT && b0 + o0 / 9 < B; o0 += LC_BATCH * ngw) {   // warp-uniform
+            double old[LC_BATCH];
 #pragma unroll
-                    for (int w = 0; w < LC_CTA_WARPS; ++w)
-                        lc_pair_add(s, c, ld_shared_cluster_f32(peer + (uint32_t)(w * LC_OUT * 32 * sizeof(float))));
-                }
+            for (int u = 0; u < LC_BATCH; ++u) {
+                const int o = o0 + u * ngw;
+                old[u] = (o < LC_OUT && b0 + o / 9 < B && l < L) ? *sums(o) : 0.0;
             }
-            if (l < L) *sums(o) = old[u] + ((double)s + (double)c);
+#pragma unroll
+            for (int u = 0; u < LC_BATCH; ++u) {
+                const int o = o0 + u * ngw;
+                if (o >= LC_OUT || b0 + o / 9 >= B) break;   // warp-uniform
+                float s = 0.f, c = 0.f;
+                const float *mine = sP + o * 32 + lane;
+                if (!CLUSTER) {
+                    for (int w = 0; w < step_warps; ++w) lc_pair_add(s, c, mine[w * LC_OUT * 32]);
+                } else {
+                    for (int q = 0; q < nrank; ++q) {   // step order: ranks, then warps
+                        const uint32_t peer = mapa_shared(smem_u32(mine), (uint32_t)q);
+#pragma unroll
+                        for (int w = 0; w < LC_CTA_WARPS; ++w)
+                            lc_pair_add(s, c, ld_shared_cluster_f32(peer + (uint32_t)(w * LC_OUT * 32 * sizeof(float))));
+                    }
+                }
+                if (l < L) *sums(o) = old[u] + (f32_to_f64(s) + f32_to_f64(c));
+            }
         }
     }
-    cluster_sync_all();   // peers have read this CTA's partials: its shared memory may go
+    if (CLUSTER) cluster_sync_all();   // peers have read this CTA's partials: its shared memory may go
 }
 
 // ------------------------------------------------------------------ K5
@@ -685,9 +713,11 @@ int lag_corr_tiles(int B, int L) { return ((L + 31) / 32) * ((B + LC_ROWS / 3 - 
 
 cudaError_t lag_corr_prepare() {
     // a tile alone in its CTA stages at most 1024 steps or 16 warps' partials: below 80 KB
-    LagCorrPlan p{LC_WARPS, 64, 1, LC_WARPS, LC_WARPS};
-    static PerDevice once;
-    return opt_in_smem(once, lag_corr_kernel, lag_corr_smem(p));
+    LagCorrPlan p{LC_WARPS, 64, 1, LC_WARPS, LC_WARPS, LC_FEW};
+    static PerDevice once[3];
+    cudaError_t e = opt_in_smem(once[0], lag_corr_kernel<LC_FEW>, lag_corr_smem(p));
+    if (e == cudaSuccess) e = opt_in_smem(once[1], lag_corr_kernel<LC_CLUSTER>, lag_corr_smem(p));
+    return e != cudaSuccess ? e : opt_in_smem(once[2], lag_corr_kernel<LC_MANY>, lag_corr_smem(p));
 }
 
 void launch_bin_finish_group(FinishGroupArgs g, cudaStream_t s) {
@@ -719,9 +749,11 @@ cudaError_t launch_lag_corr(const float *Jb, const double *Jring, int R, double 
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = (unsigned)p.ranks;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, lag_corr_kernel, Jb, Jring, R, Csum, K, B, L, p.ks,
-                              p.step_warps, t0_dev);
+    cfg.numAttrs = p.ranks > 1 ? 1 : 0;
+    const auto kernel = p.form == LC_CLUSTER ? lag_corr_kernel<LC_CLUSTER>
+                        : p.form == LC_MANY  ? lag_corr_kernel<LC_MANY>
+                                             : lag_corr_kernel<LC_FEW>;
+    return cudaLaunchKernelEx(&cfg, kernel, Jb, Jring, R, Csum, K, B, L, p.ks, p.step_warps, t0_dev);
 }
 
 int launch_gk_kappa(const double *Csum, int B, int L, long long T_s, double coef_dt,

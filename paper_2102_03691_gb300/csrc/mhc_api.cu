@@ -507,9 +507,6 @@ mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_
     return MHC_OK;
 }
 
-// With the direction split: graphene-like 4096 atoms, K = 128 has 96 pair tiles for 76 resident
-// pairs; the projection took two waves, 370 us (ncu), and takes 262 + 14 us with the last wave's
-// 20 tiles cut (423 -> 355 us a push).
 // Balanced split, host side (the kernels' arithmetic): the part holding tail chunk g when T
 // chunks are cut into `parts` ranges, and the plan of one block: whole waves of tiles first
 // (t0 tiles on all `parts_all` CTAs or pairs), then the remaining tiles' chunks over
@@ -519,6 +516,9 @@ int sk_part_of_host(long long g, long long T, int parts) {
     return (int)(((g + 1) * parts + T - 1) / T - 1);
 }
 
+// With the direction split: graphene-like 4096 atoms, K = 128 has 96 pair tiles for 76 resident
+// pairs; the projection took two waves, 375 us (ncu), and takes 258 + 14 us with the last wave's
+// 20 tiles cut (425 -> 348 us a push).
 struct SkPlan {
     int nch = 0, tiles = 0, parts_all = 0, t0 = 0, parts = 0, max_seg = 1, sub = 1;
     int planes() const { return sub * max_seg; }   // of the workspace
@@ -602,8 +602,8 @@ mhc_status run_projection(mhc_handle *h, int K) {
     // As programmatic dependents the projection and its split finish set up while the last CTAs of
     // the kernel before finish: about 1 us each of a 119 us push at 512 atoms x 1000 steps.  A
     // graph with a programmatic edge starts later, though: at 64 atoms x 32 steps the push took
-    // 38.9 us with the edge and 34.8 without.  The line lies at a pack of one wave of CTAs (512
-    // atoms and step a CTA); at 1003 x 77, just below it, both take 60 us.
+    // 38.9 us with the edge and 34.8 without (FP32, 8 x 4: 20.5 and 18.5).  The line is a measured one,
+    // in atom-steps an SM: at 1003 x 77, just below it, both take 60 us.
     const bool pdl = (int64_t)K * h->N >= (int64_t)h->sm_count * 512;
     if (!is_tc(h)) {
         // with the direction split one product per segment of d, then Xdot = sum over segments
@@ -772,43 +772,47 @@ void reserve_tuned_ws(mhc_handle *h) {
 // of them with a split.  A candidate whose warm-up takes half as long again as the fastest is not
 // timed further (it keeps that time), so that the first push of a shape pays for few of them.  With the
 // cross-correlations every launch is timed by itself behind a read of their state, which streams
-// through L2 between two projections of a run: from a warm L2 512 atoms x 250 steps look best
-// unsplit, and a run of four blocks with 64 bins then takes 485 us instead of 457 with three splits.
+// through L2 between two projections of a run.  (512 atoms x 250 steps, 64 bins: the twelve best shapes
+// and splits lie within 440 .. 462 us a run of four blocks, and the choice falls on one of 440 .. 445.)
 mhc_status time_candidates(mhc_handle *h, int K, std::vector<std::pair<float, TcConfig>> &cands,
                            int rounds = 3) {
     constexpr float SHORT_MS = 0.3f;   // longer launches hide the host's
+    constexpr float TINY_MS = 0.05f;    // timed for about as long: several launches of a few microseconds
     constexpr float HOPELESS = 1.5f;
     cudaEvent_t e0, e1;
     MHC_CUDA(h, cudaEventCreate(&e0));
     MHC_CUDA(h, cudaEventCreate(&e1));
     mhc_status s = MHC_OK;
-    // one launch of candidate c timed, behind one that is not (`lead`)
-    auto timed = [&](const TcConfig &c, bool lead, float &ms) -> mhc_status {
+    // `reps` launches of candidate c timed, behind one that is not (`lead`)
+    auto timed = [&](const TcConfig &c, bool lead, int reps, float &ms) -> mhc_status {
         if (mhc_status q = set_tc_config(h, c); q != MHC_OK) return q;
         if (has_xcorr(h)) launch_xcorr_touch(h->xc_plan, h->xcp, h->stream);
         if (lead)
             if (mhc_status q = run_projection(h, K); q != MHC_OK) return q;
         if (cudaEventRecord(e0, h->stream) != cudaSuccess) return fail(h, MHC_ERR_CUDA, "event record");
-        if (mhc_status q = run_projection(h, K); q != MHC_OK) return q;
+        for (int r = 0; r < reps; ++r)
+            if (mhc_status q = run_projection(h, K); q != MHC_OK) return q;
         if (cudaEventRecord(e1, h->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
             cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess)
             return fail(h, MHC_ERR_CUDA, "autotune timing failed");
+        ms /= (float)reps;
         return MHC_OK;
     };
     float shortest = 1e30f;
     for (auto &x : cands) {
         x.first = 1e30f;
-        if ((s = timed(x.second, !has_xcorr(h), x.first)) != MHC_OK) break;
+        if ((s = timed(x.second, !has_xcorr(h), 1, x.first)) != MHC_OK) break;
         shortest = std::min(shortest, x.first);
     }
     const bool lead = !has_xcorr(h) && shortest < SHORT_MS;
+    const int reps = has_xcorr(h) ? 1 : std::max(1, std::min(4, (int)(TINY_MS / std::max(shortest, 1e-3f))));
     std::vector<bool> keep;
     for (auto &x : cands) keep.push_back(has_xcorr(h) || x.first <= HOPELESS * shortest);
     for (int r = has_xcorr(h) ? 0 : 1; r < rounds && s == MHC_OK; ++r)   // (there the first was cold)
         for (size_t q = 0; q < cands.size() && s == MHC_OK; ++q) {
             if (!keep[q]) continue;
             float ms = 0.f;
-            if ((s = timed(cands[q].second, lead, ms)) == MHC_OK) cands[q].first = std::min(cands[q].first, ms);
+            if ((s = timed(cands[q].second, lead, reps, ms)) == MHC_OK) cands[q].first = std::min(cands[q].first, ms);
         }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

@@ -20,9 +20,9 @@ namespace {
 // The order of the sums depends on K alone, so a grouped launch gives the bits of a solo one.  It is
 // launched plainly: as a programmatic dependent of the projection it made the 8000-atom push 20 us
 // and the 512-atom push 2 us longer.
-// Measured (ncu, us, one thread a step with a tree of FP64 sums -> now): 600 rows, K = 128 10.7 -> 6.4;
-// 200 rows, K = 128 6.9 -> 5.1; 16 systems of 52 bins, K = 256 22.1 -> 17.2; 100 rows, K = 1000 8.6
-// -> 8.0; 64 rows of 13 slots, K = 256 7.5 -> 6.6; 100 and 304 rows of a slot or none, K = 200 4.9 ->
+// Measured (ncu, us, one thread a step with a tree of FP64 sums -> now): 600 rows, K = 128 10.4 -> 6.4;
+// 200 rows, K = 128 6.8 -> 5.0; 16 systems of 52 bins, K = 256 21.7 -> 16.8; 100 rows, K = 1000 8.7
+// -> 7.9; 64 rows of 13 slots, K = 256 7.5 -> 6.5; 100 and 304 rows of a slot or none, K = 200 4.9 ->
 // 4.9, K = 1000 9.7 -> 10.4.
 constexpr int BF_MAX_THREADS = 768;
 __host__ __device__ constexpr int bf_threads(int K) { return K <= 128 ? 384 : BF_MAX_THREADS; }
@@ -144,18 +144,18 @@ __global__ void __launch_bounds__(BF_MAX_THREADS, 2) bin_finish_group_kernel(con
 //     the early fetch and the barriers of a cluster only cost: CTAs stay small, a tile is a CTA
 //     of its own (but for 16 warps of steps, of which an SM holds too few whole), and the sums are
 //     updated one by one.  304 bins x 1000 lags (2432 tiles; us a push, one warp a tile and 32 steps ->
-//     the form for few tiles -> now): K = 1 43 -> 70 -> 47, 128 59 -> 87 -> 59, 400 118 -> 131 -> 119; 1000
-//     in clusters 202 -> 193.
-// Measured (ncu, cold caches, us, before -> now): K = 32, 8 bins, 8 lags 23.3 -> 7.7; K = 77, 37
-// bins, 123 lags 15.5 -> 8.4; K = 1000, 100 bins, 200 lags 24.6 -> 18.6; K = 512, 64 bins, 1000
-// lags 30.5 -> 27.9; K = 256, 64 bins, 500 lags 13.0 -> 13.4.  The cluster form starts at
-// LC_FILL_TILES = half the SMs: below it a tile's CTA has an SM to itself either way, and one
-// CTA's barriers are cheaper than a cluster's.
+//     the form for few tiles -> now): K = 1 43 -> 70 -> 45, 128 59 -> 87 -> 59, 400 119 -> 131 -> 117; 1000
+//     in clusters 202 -> 192.
+// Measured (ncu, us, one warp a tile and 32 steps -> now): K = 32, 8 bins, 8 lags 16.0 -> 5.6; K = 77, 37
+// bins, 123 lags 11.9 -> 6.9; K = 1000, 100 bins, 200 lags 24.6 -> 17.9; K = 512, 64 bins, 1000 lags
+// 29.8 -> 28.6; K = 256, 64 bins, 500 lags 12.6 -> 12.8.  The cluster form starts at LC_FILL_TILES =
+// half the SMs: below it a tile's CTA has an SM to itself either way, and one CTA's barriers are cheaper
+// than a cluster's.
 constexpr int LC_ROWS = 12;   // 4 bins x 3 components a thread
 constexpr int LC_OUT = 3 * LC_ROWS;
 constexpr int LC_WARPS = 16;      // warps of a tile, and of a CTA that holds a tile alone
 constexpr int LC_CTA_WARPS = 4;   // warps of a CTA of a cluster
-constexpr int LC_FINAL_WARPS = 12;   // fewest warps of a CTA that holds a tile alone
+constexpr int LC_FINAL_WARPS = 12;   // warps of a CTA that holds a tile alone where the tiles are few
 constexpr int LC_BATCH = 5;       // sums a warp updates at a time (all of them with 8 or more warps)
 constexpr int LC_MIN_STEPS = 4;   // fewest steps a warp is worth starting for
 // (Of this GPU's 152 SMs and not of those a process is given: the order of the sums then depends on the

@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) shc_tc_kernel(const __grid_cons
 // Ksum[c][l] += sum over tile pairs and atom ranges of the unit diagonal
 // m = l - (t0 + 256 q - 128 p) + 127.  A warp takes 32 lags and every RED_GROUPS-th (tile pair, atom
 // range); the warps' FP64 sums are added in order (deterministic).  Bound by latency: one thread a
-// lag went through all of them in turn, 7.0 us at 8000 atoms x 250 lags (ncu); now 3.9 us.
+// lag went through all of them in turn, 5.6 us at 8000 atoms x 250 lags (ncu); now 4.0 us.
 constexpr int RED_GROUPS = 8;
 __global__ void __launch_bounds__(32 * RED_GROUPS) shc_tc_reduce_kernel(const __grid_constant__ ShcTcParams p,
                                                                        double *Ksum) {

@@ -163,6 +163,7 @@ struct mhc_handle {
     // tensor-core state
     TcConfig tc{256, 64, 2, 0, 0};
     std::map<int, TcConfig> tuned;  // K -> config
+    bool no_split = false;          // the workspace of an autotuned split did not fit
     TcParams<1> tcp{};
     SgemmParams sgp{};    // FP32 path
     bool fp32_cut = true;   // the product's last wave of tiles may be cut along d
@@ -502,6 +503,7 @@ mhc_status apply_bins(mhc_handle *h, const std::vector<int> &bin_of_mode, int32_
         h->tcp.idesc = idesc_f16(h->split == SPLIT_BF16 ? 1u : 0u, (c.pair ? 2 : 1) * TC_BM, (uint32_t)c.bn);
     }
     h->bins_ready = true;
+    h->no_split = false;
     if ((s = reset_accumulators(h)) != MHC_OK) return s;
     reserve_tuned_ws(h);
     return MHC_OK;
@@ -571,13 +573,26 @@ mhc_status ensure_split_ws(mhc_handle *h, const TcConfig &c) {
     return dev_alloc(h, "split_ws", need, false);
 }
 
-mhc_status set_tc_config(mhc_handle *h, const TcConfig &c) {
+// The same for a configuration about to be used: a split that the autotuner chose, here or for another
+// handle, runs unsplit where its workspace does not fit (until the bins are set again).
+mhc_status settle_split(mhc_handle *h, TcConfig &c) {
+    const bool chosen = h->prm.split_d == 0;
+    if (chosen && h->no_split) c.split = 1;
+    const mhc_status s = ensure_split_ws(h, c);
+    if (s != MHC_ERR_OOM || !chosen) return s;
+    h->err.clear();
+    h->no_split = true;
+    c.split = 1;
+    return MHC_OK;
+}
+
+mhc_status set_tc_config(mhc_handle *h, TcConfig c) {
     if (!tc_config_supported(c)) return fail(h, MHC_ERR_INVALID_ARG, "unsupported tile configuration");
     if (c.split > 1 && (h->dir || c.split > TC_MAX_SPLIT))
         return fail(h, MHC_ERR_INVALID_ARG, "d-axis split %d not available here", c.split);
     if (c.split < 1 && c.split != TC_SPLIT_BALANCED)
         return fail(h, MHC_ERR_INVALID_ARG, "d-axis split %d not available here", c.split);
-    if (mhc_status s = ensure_split_ws(h, c); s != MHC_OK) return s;
+    if (mhc_status s = settle_split(h, c); s != MHC_OK) return s;
     const bool remap = h->bins_ready && (c.bn != h->tc.bn || c.bk != h->tc.bk || c.pair != h->tc.pair);
     h->tc = c;
     if (remap) {
@@ -749,7 +764,7 @@ void tune_file_append_locked(const TuneKey &k, const TcConfig &c) {
 // The split workspace of the tile already tuned for this shape and the longest block (by another
 // handle of the process, or in the tuning file), allocated with the bins: the first push would
 // otherwise stop for it (about 100 us).  After everything that the handle cannot do without; where it
-// does not fit, the push that needs it reports so.
+// does not fit, the push that needs it runs unsplit.
 void reserve_tuned_ws(mhc_handle *h) {
     if (!is_tc(h) || h->prm.tile_config != 0 || h->M_eff == 0) return;
     TcConfig c{};
@@ -1435,7 +1450,7 @@ mhc_status mhc_push(mhc_handle *h, const float *v, const float *W, int32_t K, in
         return fail(h, MHC_ERR_INVALID_ARG, "where");
     MHC_CUDA(h, cudaSetDevice(h->prm.device));
     mhc_status s;
-    if (is_tc(h) && (s = ensure_split_ws(h, h->tc)) != MHC_OK) return s;
+    if (is_tc(h) && (s = settle_split(h, h->tc)) != MHC_OK) return s;
     if ((s = stage_issue(h, v, W, K, where)) != MHC_OK) return s;
     const int staged = h->stage_used;
     s = stage_order(h, h->stream);

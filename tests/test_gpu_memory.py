@@ -4,6 +4,7 @@ import os
 import subprocess
 import sys
 
+import numpy as np
 import pytest
 
 from tests.test_gpu_parity import make_case, need_gpu
@@ -78,3 +79,42 @@ def test_group_members_hold_no_split_workspace(tmp_path):
     # 128 columns x 256 modes x 4 bytes a plane, at least one
     assert all(x - y >= 128 * 256 * 4 for x, y in zip(b[:2], b[2:4])), b
     assert all(z >= x for x, z in zip(b[:2], b[4:])), b
+
+
+def test_an_autotuned_split_that_does_not_fit_runs_unsplit():
+    # the direction split's planes of the last wave (453 MB here) with 150 MB left on the device: the
+    # push takes the unsplit kernel, and its currents are those of a handle that was told to
+    need_gpu()
+    from paper_2102_03691_gb300.mhc import ModalHeatCurrent
+    N, M, K, B = 3000, 9000, 512, 5
+    g = torch.Generator(device="cuda").manual_seed(9995)
+    E = torch.randn((3 * N, M), generator=g, device="cuda") / (3 * N) ** 0.5
+    v, W = (torch.randn((K, N, q), generator=g, device="cuda") for q in (3, 9))
+    f, mass = torch.rand(M, generator=g, device="cuda").cpu().numpy() * 16.0, [28.085] * N
+
+    def handle(split_d, tile_config):
+        h = ModalHeatCurrent(precision="fp16x3", k_max=K, direction=True, split_d=split_d, tile_config=tile_config)
+        h.set_modes(E, mass, f)
+        h.set_bins_uniform(0.0, 16.0, B)
+        return h
+
+    ref, h = handle(1, 5), handle(0, 0)
+    ref.push(v, W)
+    want = ref.read_binned_current()
+    warm = handle(1, 0)                       # every tile's kernel is loaded while there is room
+    warm.push(v, W)
+    warm.sync()
+    warm.close()
+    torch.cuda.synchronize()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (150 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        for _ in range(3):
+            h.push(v, W)
+        got = h.read_binned_current()
+        assert h.info()["tile_split"] == 1
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    np.testing.assert_array_equal(got, want)
+    h.close()
+    ref.close()

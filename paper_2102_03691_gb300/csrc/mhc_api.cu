@@ -813,10 +813,11 @@ mhc_status time_candidates(mhc_handle *h, int K, std::vector<std::pair<float, Tc
         ms /= (float)reps;
         return MHC_OK;
     };
-    float shortest = 1e30f;
+    float shortest = 1e30f, unused = 0.f;
+    if (!cands.empty() && !has_xcorr(h)) s = timed(cands[0].second, false, 1, unused);   // the clock comes up
     for (auto &x : cands) {
         x.first = 1e30f;
-        if ((s = timed(x.second, !has_xcorr(h), 1, x.first)) != MHC_OK) break;
+        if (s != MHC_OK || (s = timed(x.second, !has_xcorr(h), 1, x.first)) != MHC_OK) break;
         shortest = std::min(shortest, x.first);
     }
     const bool lead = !has_xcorr(h) && shortest < SHORT_MS;

@@ -2110,7 +2110,7 @@ mhc_status mhc_group_create(mhc_group **out, mhc_handle *const *handles, int32_t
     }
     // what the members' bins reserved for a split (a member pushed by itself allocates it again)
     for (mhc_handle *h : g->hs) {
-        if (!dptr<float>(h, "split_ws")) continue;
+        if (h->prm.split_d != 0 || !dptr<float>(h, "split_ws")) continue;   // (a split asked for keeps its own)
         cudaStreamSynchronize(h->stream);
         drop_graphs(h);
         dev_free(h, "split_ws");
